@@ -193,13 +193,17 @@ afe_status afe_stage_times(afe_mesh* m, double* ms, int64_t* nsteps, int reset);
 
 /* How the handle's step runs (a host-side report; no GPU work).  The FP32 form keeps each
  * cell's fixed-point iteration in the shared memory of one predictor block when the cell fits
- * (fp32_shared = 1): the right-hand side of Eq. ader4 is formed in chunks of sub-tets (16 per
- * chunk at N = 2, 3 when the cell leaves room for them, else 8: a "narrow" cell) and M_i^-1
- * streams through a ring of stages of 32 rows (in the tensor-memory form 16 or 8 rows when a
- * large cell leaves less room; as many stages as fit, at most 8; a cell whose N_i is not a
- * multiple of the stage height ends with a partial, "masked" stage).  Meshes whose largest cell
- * does not fit that plan run the FP32 form with global-memory scratch on the CUDA cores
- * (fp32_shared = 0), as does, always, the FP64 form. */
+ * (fp32_shared = 1).  Meshes whose largest cell leaves room for at least two such blocks per SM
+ * run the form with several cells in flight per SM (M_i^-1 as split 16-bit pairs streamed from L2).
+ * The others, and the tensor-memory variant, run one block per SM: the right-hand side of Eq.
+ * ader4 is formed in chunks of sub-tets (16 per chunk at N = 2, 3 when the cell leaves room for
+ * them, else 8: a "narrow" cell) and M_i^-1 streams through a ring of stages of 32 rows (in the
+ * tensor-memory form 16 or 8 rows when a large cell leaves less room; as many stages as fit, at
+ * most 8; a cell whose N_i is not a multiple of the stage height ends with a partial, "masked"
+ * stage).  The ring, chunk and stage fields below report that one-block plan for every mesh with
+ * fp32_shared = 1, smem_bytes the form that runs.  Meshes whose largest cell does not fit it run
+ * the FP32 form with global-memory scratch on the CUDA cores (fp32_shared = 0), as does, always,
+ * the FP64 form. */
 typedef struct {
   int32_t fp32_shared;     /* 1: FP32 shared-memory predictor (M_i^-1 apply on the tensor cores)  */
   int32_t corrector_block; /* 1: FP32 corrector with one block per cell                           */
@@ -219,8 +223,8 @@ afe_status afe_plan_info(const afe_mesh* m, afe_plan* out);
 /* Which form of the FP32 predictor's M_i^-1 apply a handle uses: 0 (the default) the
  * warp-level mma.sync form; 1 the form on the 5th-generation tensor cores with tensor memory
  * (tcgen05), for meshes whose every cell fits its shared-memory plan (up to 640 nodes per cell;
- * else AFE_EINVAL).  Both compute the same 3xTF32 product (results agree to FP32 rounding, not
- * bit for bit); on the measured workloads the mma.sync form is the faster one.  A batch takes
+ * else AFE_EINVAL).  Both form FP32-level products of split operands (16-bit pairs or 3xTF32; results
+ * agree to FP32 rounding, not bit for bit); on the measured workloads form 0 is the faster one.  A batch takes
  * the tensor-memory form only when every member asks for it.  Other values: AFE_EINVAL. */
 afe_status afe_set_predictor_variant(afe_mesh* m, int32_t variant);
 
@@ -243,8 +247,9 @@ afe_status afe_set_wait_limit(afe_mesh* m, int32_t polls);
  *               its members); 0: index order.
  *   variant     0: mma.sync form of the M_i^-1 apply; 1: tcgen05 / tensor-memory form (only if
  *               every cell fits its plan; see afe_set_predictor_variant).
- *   ring_cap    most M_i^-1 stages in flight in the ring (0: as many as fit, at most 8).
- *   narrow      1: right-hand side in chunks of 8 sub-tets even where 16 fit.
+ *   ring_cap    one-block form: most M_i^-1 stages in flight in the ring (0: as many as fit, at
+ *               most 8).
+ *   narrow      one-block form: 1: right-hand side in chunks of 8 sub-tets even where 16 fit.
  * Other values: AFE_EINVAL. */
 typedef struct {
   int32_t cost_order;
@@ -256,8 +261,8 @@ afe_status afe_set_schedule(afe_mesh* m, const afe_schedule* s);
 afe_status afe_get_schedule(const afe_mesh* m, afe_schedule* s);
 
 /* Choose the schedule by measurement: with the time step of the current state computed on the
- * device, every candidate (cost_order 0/1; variant 0, and 1 where the cells fit; ring_cap 0 or
- * 2; narrow 0, and 1 where wide chunks are used) times `trials` launches of the predictor alone
+ * device, every candidate (cost_order 0/1; for meshes on the one-block form also variant 0, and 1
+ * where the cells fit; ring_cap 0 or 2; narrow 0, and 1 where wide chunks are used) times `trials` launches of the predictor alone
  * (CUDA events on the handle's stream; the predictor writes only per-step intermediates, so
  * the state is unchanged), and the fastest is set.  *best receives it, *best_ms and
  * *default_ms (either may be NULL) the mean predictor time with it and with the default

@@ -2,7 +2,7 @@
 
 First g++ builds and runs ``gen_sref`` (csrc/gen_sref.cpp with the reference-element code),
 which writes ``lib/gen/sref_gen.cuh``: the FP32 predictor's reference-stiffness contractions
-with the matrix entries as immediates.  Then nvcc compiles the CUDA translation unit and g++
+with the matrix entries as immediates.  Then nvcc compiles the CUDA translation units and g++
 the host topology and reference-element code, in parallel, and ``nvcc -shared`` links them.
 """
 from __future__ import annotations
@@ -54,9 +54,12 @@ def build(verbose: bool = False, extra_flags=None) -> str:
         obj = os.path.join(objdir, src + ".o")
         jobs.append([os.environ.get("CXX", "g++"), *common, "-fPIC", "-Wall", "-c",
                      os.path.join(CSRC, src), "-o", obj])
-    cu_obj = os.path.join(objdir, "afe.cu.o")
-    jobs.append([nvcc, *common, *ARCH, "-lineinfo", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
-                 *extra, "-c", os.path.join(CSRC, "afe.cu"), "-o", cu_obj])
+    # the CUDA translation units: the library, and one per order of predictor_cells
+    units = [("afe.cu", "afe.cu.o", [])]
+    units += [("predictor_cells.cu", f"predictor_cells_{n}.o", [f"-DAFE_ORDER={n}"]) for n in (1, 2, 3)]
+    for src, obj, flags in units:
+        jobs.append([nvcc, *common, *ARCH, "-lineinfo", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
+                     *flags, *extra, "-c", os.path.join(CSRC, src), "-o", os.path.join(objdir, obj)])
     with ThreadPoolExecutor(len(jobs)) as ex:
         outs = list(ex.map(_run, jobs))
     if verbose:

@@ -15,6 +15,7 @@
 
 #include "afe.h"
 #include "kernels.cuh"
+#include "predictor_cells.hpp"
 #include "predictor_f32.cuh"
 #include "refelem.hpp"
 #include "topology.hpp"
@@ -66,6 +67,8 @@ struct afe_mesh {
   afe_schedule sched{};  // predictor schedule (cost order, ring cap, narrow chunks; variant above)
   int32_t* d_order = nullptr;  // the cells in decreasing cost (allocated when first asked for)
   size_t f32_smem = 0;
+  afe::PcRef pref{};     // time-basis constants of the predictor with several cells per SM
+  afe::PcPlan pc{};           // its plan for this mesh's cells (blocks = 0: not used)
   double* d_totals_partial = nullptr;
   double* d_totals = nullptr;
   int totals_blocks = 256;
@@ -121,13 +124,29 @@ struct StepPlan {
   int order = 1, fp32 = 0, limiter = 0, n_sm = 1, diag = 0;
   int f32_ok = 0, f32_tc = 0;
   size_t f32_smem = 0;
+  afe::PcPlan pc;
+  afe::PcRef pref{};
+  int inviscid = 0, viscous = 0;  // cells without / with viscous fluxes may be present
   const afe::RefData* d_ref = nullptr;
   afe_mesh* single = nullptr;  // nullptr for a batch (FP32 shared-memory kernels only)
   afe_mesh* prof = nullptr;    // stage events are recorded on this mesh when profiling
 };
 
+// Adds the kinds of cells a mesh may hold: with mu or kappa every cell is viscous (in FP32, as
+// the predictor tests it), with the limiter any cell may be.
+void add_kinds(StepPlan* P, const afe_mesh* m) {
+  const afe::DevMesh& d = m->dm;
+  const double kap = d.kappa0 >= 0.0 ? d.kappa0 : d.mu0 * d.gamma * d.cv / d.Pr;
+  const bool visc = (float)d.mu0 != 0.f || (float)kap != 0.f;
+  if (visc || m->p.limiter) P->viscous = 1;
+  if (!visc) P->inviscid = 1;
+  // a limiter may undo a viscosity below FP32's range: both kinds are possible
+  if (visc && m->p.limiter) P->inviscid = 1;
+}
+
 StepPlan plan_of(afe_mesh* m) {
   StepPlan P;
+  add_kinds(&P, m);
   P.b = &m->self;
   P.st = m->stream;
   P.order = m->p.order;
@@ -138,6 +157,8 @@ StepPlan plan_of(afe_mesh* m) {
   P.f32_ok = m->f32_ok;
   P.f32_tc = m->f32_tc;
   P.f32_smem = m->f32_smem;
+  P.pc = m->pc;
+  P.pref = m->pref;
   P.d_ref = m->d_ref;
   P.single = m;
   P.prof = m;
@@ -146,9 +167,25 @@ StepPlan plan_of(afe_mesh* m) {
 
 bool corrector_f32_fits(int Nmax) { return Nmax <= 2 * 4 * afe::kCorrThreads; }
 
+// Plan of the FP32 predictor with several cells per SM (blocks = 0: the one-block form runs).
+afe_status plan_cells(int order, int device, int n_sm, int64_t cells, int Nmax, int Smax, int Fmax, afe::PcPlan* out) {
+  *out = afe::PcPlan{};
+  switch (order) {
+    case 1: AFE_CUDA(afe::pc_plan<1>(device, n_sm, cells, Nmax, Smax, Fmax, out)); break;
+    case 2: AFE_CUDA(afe::pc_plan<2>(device, n_sm, cells, Nmax, Smax, Fmax, out)); break;
+    case 3: AFE_CUDA(afe::pc_plan<3>(device, n_sm, cells, Nmax, Smax, Fmax, out)); break;
+    default: break;
+  }
+  return AFE_OK;
+}
+
 template <int N, typename Real>
 void launch_predictor(const StepPlan& P) {
   if constexpr (N <= 3) {  // the shared-memory FP32 predictor exists for N <= 3 (cells up to 640 nodes)
+    if (sizeof(Real) == 4 && P.f32_ok && P.pc.blocks && !P.f32_tc) {
+      afe::pc_launch<N>(P.pc, *P.b, P.pref, P.inviscid, P.viscous, P.diag, P.n_sm, P.st);
+      return;
+    }
     if (sizeof(Real) == 4 && P.f32_ok) {
       if (P.f32_tc)
         afe::predictor_f32_kernel<N, true><<<P.n_sm, afe::kF32Threads, P.f32_smem, P.st>>>(*P.b, P.d_ref, P.diag,
@@ -281,9 +318,12 @@ afe_status record(const StepPlan& P) {
   return AFE_OK;
 }
 
-// kernels per step: begin + [means + limiter] + (set_dt | cfl + finalize) + predictor + face
-// + corrector + clock
-int launches_per_step(const StepPlan& P, double dt) { return 1 + (P.limiter ? 2 : 0) + (dt > 0 ? 1 : 2) + 3 + 1; }
+// kernels per step: begin + [means + limiter] + (set_dt | cfl + finalize) + predictor (one for
+// each kind of cell) + face + corrector + clock
+int launches_per_step(const StepPlan& P, double dt) {
+  const int both = P.fp32 && P.pc.blocks && !P.f32_tc && P.inviscid && P.viscous;
+  return 1 + (P.limiter ? 2 : 0) + (dt > 0 ? 1 : 2) + 3 + both + 1;
+}
 
 afe_status enqueue_step(const StepPlan& P, double dt) {
   NvtxRange step_range("afe step");
@@ -350,6 +390,35 @@ void sync_self(afe_mesh* m) {
   b.gpre[0] = 0;
   b.gpre[1] = m->topo.n_groups;
   b.tab[0] = m->dm;
+}
+
+// What predictor_cells_kernel needs beside the one-block form's data: the split copy of M_i^-1
+// and the gather blocks.  A handle whose cells do not fit the plan, or for which the device
+// has no room left, keeps the one-block form.
+afe_status set_up_cells(afe_mesh* m, int64_t nminv) {
+  const afe::Topology& T = m->topo;
+  const afe::RefData& R = m->ref;
+  for (int s = 0; s < R.Nt; ++s) {
+    double sum = 0;
+    m->pref.w[s] = (float)R.w[s];
+    for (int t = 0; t < R.Nt; ++t) {
+      m->pref.kw[s][t] = (float)(R.K1tinv[s][t] * R.w[t]);
+      sum += R.K1tinv[s][t] * R.w[t];
+    }
+    m->pref.kws[s] = (float)sum;
+  }
+  afe::PcPlan pc;
+  AFE_TRY(plan_cells(m->p.order, m->device, m->n_sm, T.C, T.Nmax, T.Smax, T.slots_max, &pc));
+  if (!pc.blocks) return AFE_OK;
+  if (m->alloc(&m->dm.m16, (size_t)nminv) != AFE_OK ||
+      m->alloc(&m->dm.gat, afe::pc_gather_bytes(m->dm, T.T, R.Np, R.Nf)) != AFE_OK) {
+    (void)cudaGetLastError();  // out of memory: the one-block form needs neither
+    return AFE_OK;
+  }
+  afe::pc_set_up(m->dm, R.Np, R.Nf, (int)std::min<int64_t>(T.C, (int64_t)m->n_sm * 8), m->stream);
+  AFE_CUDA(cudaGetLastError());
+  m->pc = pc;
+  return AFE_OK;
 }
 
 afe_status check_params(const afe_params* p) {
@@ -551,7 +620,7 @@ afe_status afe_mesh_create(const afe_params* p, int64_t n_vertices, const double
   AFE_TRY(M->alloc(&d.tacc, 1));
   AFE_TRY(M->alloc(&d.maxbits, 1));
   AFE_TRY(M->alloc(&d.flags, afe::F_COUNT));
-  AFE_TRY(M->alloc(&d.work, 1));
+  AFE_TRY(M->alloc(&d.work, 2));
   AFE_TRY(M->alloc(&M->d_ref, 1));
 
   AFE_TRY(M->alloc(&M->d_totals_partial, (size_t)M->totals_blocks * 5));
@@ -619,6 +688,7 @@ afe_status afe_mesh_create(const afe_params* p, int64_t n_vertices, const double
         d.minv64 = nullptr;
         break;
       }
+    if (M->f32_ok) AFE_TRY(set_up_cells(M, nminv));
   }
   sync_self(M);
   *out = m.release();
@@ -870,7 +940,7 @@ afe_status afe_plan_info(const afe_mesh* m, afe_plan* out) {
   out->fp32_shared = (fp32 && m->f32_ok) ? 1 : 0;
   out->corrector_block = (fp32 && corrector_f32_fits(T.Nmax)) ? 1 : 0;
   if (!out->fp32_shared) return AFE_OK;
-  out->smem_bytes = (int64_t)m->f32_smem;
+  out->smem_bytes = (int64_t)(m->pc.blocks && !m->f32_tc ? m->pc.smem : m->f32_smem);
   out->tcgen05 = m->f32_tc;
   int rmin = afe::kF32MaxStages, rmax = 0, hmin = afe::kF32Rows;
   for (int64_t c = 0; c < T.C; ++c) {
@@ -1052,7 +1122,7 @@ afe_status afe_batch_create(afe_mesh* const* members, int n_members, void* cuda_
   if (dev != m0->device) return fail(AFE_EINVAL, "the current device is not the members' device");
   {
     void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, sizeof(int));
+    cudaError_t e = cudaMalloc(&p, 2 * sizeof(int));
     if (e != cudaSuccess) return fail(AFE_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
     b->d_work = (int*)p;
   }
@@ -1075,6 +1145,17 @@ afe_status afe_batch_create(afe_mesh* const* members, int n_members, void* cuda_
   P.diag = 0;
   P.f32_ok = 1;
   P.f32_smem = m0->f32_smem;
+  P.pref = m0->pref;
+  for (afe_mesh* m : b->mem) add_kinds(&P, m);
+  {
+    int Fmax = 0;
+    bool all = true;  // every member holds the data of the several-cells form
+    for (afe_mesh* m : b->mem) {
+      Fmax = std::max(Fmax, m->topo.slots_max);
+      all = all && m->pc.blocks > 0;
+    }
+    if (all) AFE_TRY(plan_cells(P.order, m0->device, m0->n_sm, C, Nmax, Smax, Fmax, &P.pc));
+  }
   b->tc_fits = afe::tc_cell_plan(P.order, P.f32_smem, Smax, Nmax).ok ? 1 : 0;
   P.f32_tc = b->tc_fits;
   for (afe_mesh* m : b->mem)
@@ -1197,11 +1278,15 @@ afe_status autotune_impl(const std::string& sig, int order, bool tc_fits, int* w
   cudaEvent_t e0, e1;
   AFE_CUDA(cudaEventCreate(&e0));
   AFE_CUDA(cudaEventCreate(&e1));
+  // several cells per SM: only the order of the cells is a choice (ring_cap and narrow belong to the
+  // one-block form, which with either apply is the slower one for these cells)
+  const bool one_block = plan().pc.blocks == 0;
   std::vector<afe_schedule> cand;
   for (int co = 0; co < 2; ++co)
-    for (int va = 0; va < (tc_fits ? 2 : 1); ++va)
-      for (int rc : {0, 2})
-        for (int na = 0; na < (afe::f32_ntp(order) == 4 ? 2 : 1); ++na) cand.push_back(afe_schedule{co, va, rc, na});
+    for (int va = 0; va < (one_block && tc_fits ? 2 : 1); ++va)
+      for (int rc = 0; rc <= (one_block ? 2 : 0); rc += 2)
+        for (int na = 0; na < (one_block && afe::f32_ntp(order) == 4 ? 2 : 1); ++na)
+          cand.push_back(afe_schedule{co, va, rc, na});
   double tbest = 1e300, tdef = -1.0;
   afe_schedule sbest = cand[0];
   afe_status status = AFE_OK;
@@ -1212,7 +1297,7 @@ afe_status autotune_impl(const std::string& sig, int order, bool tc_fits, int* w
     float ms = 0.f;
     for (int r = 0; r <= trials && status == AFE_OK; ++r) {
       if (r == 1) cudaEventRecord(e0, st);
-      cudaMemsetAsync(work, 0, sizeof(int), st);
+      cudaMemsetAsync(work, 0, 2 * sizeof(int), st);
       status = stage(P, 0);
     }
     if (status != AFE_OK) break;

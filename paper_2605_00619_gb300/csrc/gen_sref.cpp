@@ -17,6 +17,7 @@
 #include <cmath>
 #include <cstdio>
 #include <string>
+#include <vector>
 
 #include "refelem.hpp"
 
@@ -56,6 +57,33 @@ void emit_body(FILE* f, int np, Coef coef) {
     }
     std::fprintf(f, "    }\n");
   }
+}
+
+// out[d Np + j] = sum_l D[d][j][l] x[l]: the reference gradient of a nodal polynomial.
+void emit_gradient(FILE* f, const afe::RefData& r) {
+  const int np = r.Np;
+  double dmax = 0.0;
+  for (int d = 0; d < 3; ++d)
+    for (int j = 0; j < np; ++j)
+      for (int l = 0; l < np; ++l) dmax = std::fmax(dmax, std::fabs(r.D[d][j][l]));
+  std::fprintf(f,
+               "  // out[d Np + j] = sum_l D[d][j][l] x[l]: reference gradient of a sub-tet polynomial\n"
+               "  static __device__ __forceinline__ void gradient(const float (&x)[%d], float* out) {\n"
+               "    float a[%d];\n",
+               np, np);
+  for (int d = 0; d < 3; ++d) {
+    std::vector<bool> seen(np, false);
+    for (int l = 0; l < np; ++l)
+      for (int j = 0; j < np; ++j) {
+        const double c = r.D[d][j][l];
+        if (std::fabs(c) < 1e-13 * dmax) continue;
+        if (seen[j]) std::fprintf(f, "    a[%d] = fmaf(%s, x[%d], a[%d]);\n", j, lit((float)c).c_str(), l, j);
+        else std::fprintf(f, "    a[%d] = %s * x[%d];\n", j, lit((float)c).c_str(), l);
+        seen[j] = true;
+      }
+    for (int j = 0; j < np; ++j) std::fprintf(f, "    out[%d] = %s;\n", d * np + j, seen[j] ? ("a[" + std::to_string(j) + "]").c_str() : "0.f");
+  }
+  std::fprintf(f, "  }\n");
 }
 
 }  // namespace
@@ -117,7 +145,9 @@ int main(int argc, char** argv) {
                  "  static __device__ __forceinline__ void contract_t(const float* __restrict__ b, float (&acc)[%d]) {\n",
                  np);
     emit_body(f, np, [&](int m, int kk) { return (float)r.S[kk / np][kk % np][m]; });
-    std::fprintf(f, "  }\n};\n\n");
+    std::fprintf(f, "  }\n");
+    emit_gradient(f, r);
+    std::fprintf(f, "};\n\n");
   }
   std::fprintf(f, "}  // namespace afe\n");
   std::fclose(f);

@@ -55,6 +55,8 @@ struct DevMesh {
   double* wvec;
   double* minv64;
   float* minv32;
+  uint32_t* m16;       // M_i^-1 as pairs of FP16 values in matrix-fragment order (reduced precision)
+  unsigned char* gat;  // per cell: gather lists and face data of the reduced-precision predictor
   double* u;
   void* vol;
   void* slot_q;
@@ -179,7 +181,7 @@ __device__ __forceinline__ void block_max2(double& a, double& b, double* sh /* >
 // Set-up (FP64): cell mass matrices M_i = sum_k |J_ik| A_k^T M^ A_k (Sec. 4.4), written
 // into the per-cell dense blocks, and w_i = M_i 1.  One block per cell; sub-tets are added
 // in order (within one sub-tet the gather A_k is injective, so there is no write conflict).
-__global__ void assemble_mass_kernel(DevMesh m, const RefData* __restrict__ ref) {
+static __global__ void assemble_mass_kernel(DevMesh m, const RefData* __restrict__ ref) {
   const int Np = ref->Np;
   for (int64_t c = blockIdx.x; c < m.C; c += gridDim.x) {
     const int64_t n0 = m.node_ptr[c];
@@ -210,7 +212,7 @@ __global__ void assemble_mass_kernel(DevMesh m, const RefData* __restrict__ ref)
 // (no pivoting is needed for SPD matrices; every pivot block is a Schur complement of an
 // SPD matrix).  One block of 256 threads per cell, 32 x 32 tiles staged in shared memory.
 // A non-positive pivot raises flags[F_NONFINITE].
-__global__ void __launch_bounds__(256) invert_spd_kernel(DevMesh m) {
+static __global__ void __launch_bounds__(256) invert_spd_kernel(DevMesh m) {
   constexpr int B = 32;
   __shared__ double sD[B][B + 1];
   __shared__ double sX[B][B + 1];
@@ -329,7 +331,7 @@ __global__ void __launch_bounds__(256) invert_spd_kernel(DevMesh m) {
 }
 
 // Symmetrise in FP64 and keep the FP32 copy used by the reduced-precision path.
-__global__ void symmetrize_kernel(DevMesh m, int make32) {
+static __global__ void symmetrize_kernel(DevMesh m, int make32) {
   for (int64_t c = blockIdx.x; c < m.C; c += gridDim.x) {
     const int n = (int)(m.node_ptr[c + 1] - m.node_ptr[c]);
     const int LD = minv_ld(n);
@@ -356,22 +358,22 @@ __global__ void symmetrize_kernel(DevMesh m, int make32) {
 //
 // Start of a series of steps: clear every member's status flags (they then accumulate over
 // the steps until the host reads them).
-__global__ void flags_clear_kernel(const __grid_constant__ Batch bt) {
+static __global__ void flags_clear_kernel(const __grid_constant__ Batch bt) {
   for (int h = threadIdx.x; h < bt.nh; h += blockDim.x) {
 #pragma unroll
     for (int f = 0; f < F_COUNT; ++f) bt.tab[h].flags[f] = 0;
   }
 }
 
-// Start of a step: clear every member's CFL maximum and the shared work counter of the
+// Start of a step: clear every member's CFL maximum and the shared work counters of the
 // persistent predictor.
-__global__ void step_begin_kernel(const __grid_constant__ Batch bt) {
+static __global__ void step_begin_kernel(const __grid_constant__ Batch bt) {
   for (int h = threadIdx.x; h < bt.nh; h += blockDim.x) *bt.tab[h].maxbits = 0ull;
-  if (threadIdx.x == 0) *bt.work = 0;
+  if (threadIdx.x < 2) bt.work[threadIdx.x] = 0;
 }
 
 // Sec. 4.5: cell means u_bar_i = w_i . u_i / |P_i|  (w_i = M_i 1), one block per cell at a time.
-__global__ void cell_means_kernel(const __grid_constant__ Batch bt) {
+static __global__ void cell_means_kernel(const __grid_constant__ Batch bt) {
   __shared__ double sh[5][256];
   const int64_t total = bt.cpre[bt.nh];
   for (int64_t gc = blockIdx.x; gc < total; gc += gridDim.x) {
@@ -402,7 +404,7 @@ __global__ void cell_means_kernel(const __grid_constant__ Batch bt) {
 
 // Artificial-viscosity limiter (Sec. 4.5, Eq. beta3D): beta_i from the discrete velocity
 // divergence of the cell means over the faces of P_i, mu_i = mu + beta_i rho_i lambda_i h_i/(2N+1).
-__global__ void limiter_kernel(const __grid_constant__ Batch bt) {
+static __global__ void limiter_kernel(const __grid_constant__ Batch bt) {
   const int64_t gc = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (gc >= bt.cpre[bt.nh]) return;
   const int hh = batch_find(bt.cpre, bt.nh, gc);
@@ -439,7 +441,7 @@ __global__ void limiter_kernel(const __grid_constant__ Batch bt) {
 // CFL bound (Sec. 4.6): max over nodes of lambda + 2 lambda_v (2N+1)/h_i, one warp per cell,
 // folded into the member's maximum by an integer atomicMax on the bits of a non-negative
 // double (order-independent, hence deterministic).
-__global__ void cfl_kernel(const __grid_constant__ Batch bt) {
+static __global__ void cfl_kernel(const __grid_constant__ Batch bt) {
   const int64_t gc = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (gc >= bt.cpre[bt.nh]) return;
@@ -470,7 +472,7 @@ __global__ void cfl_kernel(const __grid_constant__ Batch bt) {
 }
 
 // dt = CFL h_min / ((2N+1) max_bound) per member (Sec. 4.6)
-__global__ void dt_finalize_kernel(const __grid_constant__ Batch bt) {
+static __global__ void dt_finalize_kernel(const __grid_constant__ Batch bt) {
   for (int h = threadIdx.x; h < bt.nh; h += blockDim.x) {
     const DevMesh& m = bt.tab[h];
     const double mx = __longlong_as_double((long long)*m.maxbits);
@@ -480,11 +482,11 @@ __global__ void dt_finalize_kernel(const __grid_constant__ Batch bt) {
   }
 }
 
-__global__ void set_dt_kernel(const __grid_constant__ Batch bt, double dt) {
+static __global__ void set_dt_kernel(const __grid_constant__ Batch bt, double dt) {
   for (int h = threadIdx.x; h < bt.nh; h += blockDim.x) *bt.tab[h].dt = dt;
 }
 
-__global__ void advance_time_kernel(const __grid_constant__ Batch bt) {
+static __global__ void advance_time_kernel(const __grid_constant__ Batch bt) {
   for (int h = threadIdx.x; h < bt.nh; h += blockDim.x) *bt.tab[h].tacc += *bt.tab[h].dt;
 }
 
@@ -999,7 +1001,7 @@ __global__ void __launch_bounds__(256) corrector_kernel(DevMesh m, const RefData
 
 // FP64 conserved totals sum_i w_i . u_i: per-block partials over a fixed cell partition,
 // then a single block sums the partials in order (bitwise reproducible).
-__global__ void totals_partial_kernel(DevMesh m, double* partial) {
+static __global__ void totals_partial_kernel(DevMesh m, double* partial) {
   __shared__ double sh[5][256];
   double acc[5] = {0, 0, 0, 0, 0};
   const int64_t per = (m.n_nodes + gridDim.x - 1) / gridDim.x;
@@ -1021,7 +1023,7 @@ __global__ void totals_partial_kernel(DevMesh m, double* partial) {
   if (threadIdx.x < 5) partial[blockIdx.x * 5 + threadIdx.x] = sh[threadIdx.x][0];
 }
 
-__global__ void totals_final_kernel(const double* partial, int nblk, double* out) {
+static __global__ void totals_final_kernel(const double* partial, int nblk, double* out) {
   if (threadIdx.x < 5) {
     double s = 0.0;
     for (int b = 0; b < nblk; ++b) s += partial[b * 5 + threadIdx.x];

@@ -1,0 +1,191 @@
+// Kernels, plans and launches of predictor_cells.cuh for one order (AFE_ORDER), and, with the
+// first, the set-up of the data they read.
+#include "predictor_cells.cuh"
+
+#include <algorithm>
+
+namespace afe {
+namespace {
+
+// Block shapes by order: warps per block and blocks per SM at most.  Shape 1 serves meshes with
+// many cells (us per step of the predictor, 24^3 P1 / 8^3 P2 / 32^3 P3 meshes), shape 0 those whose
+// cells all run at once with more warps each, where the slowest cell's latency is the time
+// (4^3 P1: 41 us with 8 warps, 58 with 2).
+template <int N, int SHAPE, bool VISC>
+struct PcShape;
+template <bool V> struct PcShape<1, 0, V> { static constexpr int W = 8, MB = 2; };
+template <bool V> struct PcShape<1, 1, V> { static constexpr int W = 2, MB = 10; };
+template <bool V> struct PcShape<2, 0, V> { static constexpr int W = 8, MB = 2; };
+template <bool V> struct PcShape<2, 1, V> { static constexpr int W = 4, MB = 4; };
+template <bool V> struct PcShape<3, 0, V> { static constexpr int W = 16, MB = 1; };
+template <bool V> struct PcShape<3, 1, V> { static constexpr int W = 8, MB = 2; };
+
+template <int N, int SHAPE, bool VISC>
+constexpr auto pc_kernel = predictor_cells_kernel<N, PcShape<N, SHAPE, VISC>::W, PcShape<N, SHAPE, VISC>::MB, VISC>;
+
+template <int N, int SHAPE>
+cudaError_t plan_shape(int device, int Nmax, int Smax, int Fmax, PcPlan* out) {
+  constexpr int W = PcShape<N, SHAPE, false>::W, MB = PcShape<N, SHAPE, false>::MB, THR = 32 * W;
+  *out = PcPlan{};
+  if (pc_slots(Nmax, THR) > (kPcOver + 1) * THR || Smax > kPcMaxSub) return cudaSuccess;
+  cudaFuncAttributes fa, fv;
+  cudaError_t e = cudaFuncGetAttributes(&fa, pc_kernel<N, SHAPE, false>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fv, pc_kernel<N, SHAPE, true>);
+  int per_sm = 0, optin = 0;
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+  if (e != cudaSuccess) return e;
+  const int stat = (int)std::max(fa.sharedSizeBytes, fv.sharedSizeBytes);
+  for (int nb = MB; nb >= std::min(MB, 2); --nb) {
+    // 1 KB of every block's share is the system's
+    const int64_t share = std::min<int64_t>(per_sm / nb - 1024, optin) - stat;
+    const size_t smem = share > 0 ? (size_t)share / 128 * 128 : 0;
+    if (pc_need<N>(Nmax, Smax, Fmax, THR) > smem) continue;
+    // the limit is the function's, shared by every handle: the most any plan may ask for
+    e = cudaFuncSetAttribute(pc_kernel<N, SHAPE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - stat);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(pc_kernel<N, SHAPE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - stat);
+    out->shape = SHAPE;
+    out->blocks = nb;
+    out->smem = smem;
+    return e;
+  }
+  return cudaSuccess;
+}
+
+template <int N, int SHAPE>
+void launch_shape(const PcPlan& p, const Batch& b, const PcRef& ref, bool inviscid, bool viscous, int diag, int n_sm,
+                  cudaStream_t st) {
+  constexpr int THR = 32 * PcShape<N, SHAPE, false>::W;
+  static_assert(PcShape<N, SHAPE, true>::W == PcShape<N, SHAPE, false>::W, "one plan serves both kinds");
+  const int grid = (int)std::min<int64_t>(b.cpre[b.nh], (int64_t)n_sm * p.blocks);
+  const int smem = (int)p.smem, mixed = inviscid && viscous;
+  if (inviscid) pc_kernel<N, SHAPE, false><<<grid, THR, smem, st>>>(b, ref, diag, smem, mixed);
+  if (viscous) pc_kernel<N, SHAPE, true><<<grid, THR, smem, st>>>(b, ref, diag, smem, mixed);
+}
+
+}  // namespace
+
+template <int N>
+cudaError_t pc_plan(int device, int n_sm, int64_t cells, int Nmax, int Smax, int Fmax, PcPlan* out) {
+  // the largest cell has to leave room for two blocks per SM (shape 1) in any case: meshes beyond
+  // that take the one-block form whatever their size
+  PcPlan many;
+  cudaError_t e = plan_shape<N, 1>(device, Nmax, Smax, Fmax, &many);
+  *out = many;
+  if (e != cudaSuccess || !many.blocks || cells > (int64_t)n_sm * PcShape<N, 0, false>::MB) return e;
+  PcPlan few;
+  e = plan_shape<N, 0>(device, Nmax, Smax, Fmax, &few);
+  if (few.blocks) *out = few;
+  return e;
+}
+
+template <int N>
+void pc_launch(const PcPlan& p, const Batch& b, const PcRef& ref, bool inviscid, bool viscous, int diag, int n_sm,
+               cudaStream_t st) {
+  if (p.shape) launch_shape<N, 1>(p, b, ref, inviscid, viscous, diag, n_sm, st);
+  else launch_shape<N, 0>(p, b, ref, inviscid, viscous, diag, n_sm, st);
+}
+
+template cudaError_t pc_plan<AFE_ORDER>(int, int, int64_t, int, int, int, PcPlan*);
+template void pc_launch<AFE_ORDER>(const PcPlan&, const Batch&, const PcRef&, bool, bool, int, int, cudaStream_t);
+
+#if AFE_ORDER == 1
+// The split copy of M_i^-1 (see minv_split_words), from its FP32 rows; one block per cell at a time.
+static __global__ void __launch_bounds__(256) split_minv_kernel(DevMesh m) {
+  __shared__ uint32_t smax;
+  for (int64_t c = blockIdx.x; c < m.C; c += gridDim.x) {
+    const int n = (int)(m.node_ptr[c + 1] - m.node_ptr[c]), LD = minv_ld(n);
+    const float* A = m.minv32 + m.minv_ptr[c];
+    uint32_t* out = m.m16 + m.minv_ptr[c];
+    if (threadIdx.x == 0) smax = 0;
+    __syncthreads();
+    uint32_t mx = 0;
+    for (int e = threadIdx.x; e < n * LD; e += blockDim.x) mx = max(mx, __float_as_uint(fabsf(A[e])));
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0) atomicMax(&smax, mx);
+    __syncthreads();
+    const int e = f16_scale_exp(smax);
+    const float s = __uint_as_float((uint32_t)e << 23);
+    if (threadIdx.x == 0) out[0] = (uint32_t)(254 - e) << 23;
+    const int nt = (n + 15) / 16;
+    // word (tile, part, lane, i): entries (row, col), (row, col + 1) with row = 16 ti + lane / 4 + 8 (i & 1),
+    // col = 16 tj + 2 (lane & 3) + 8 (i >> 1)
+    for (int w = threadIdx.x; w < nt * nt * 128; w += blockDim.x) {
+      const int i = w & 3, lane = (w >> 2) & 31, blk = w >> 7, ti = blk / nt, tj = blk - ti * nt;
+      if (tj > ti) continue;
+      const int row = 16 * ti + (lane >> 2) + 8 * (i & 1), col = 16 * tj + 2 * (lane & 3) + 8 * (i >> 1);
+      uint32_t hi = 0, lo = 0;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const float x = (row < n && col + q < n) ? s * A[(int64_t)row * LD + col + q] : 0.f;
+        const __half h = __float2half_rn(x), l = __float2half_rn(x - __half2float(h));
+        hi |= (uint32_t)__half_as_ushort(h) << (16 * q);
+        lo |= (uint32_t)__half_as_ushort(l) << (16 * q);
+      }
+      uint32_t* o = out + 32 + tri_tile(ti, tj) * 256 + lane * 4 + i;
+      o[0] = hi;
+      o[128] = lo;
+    }
+    __syncthreads();
+  }
+}
+
+// The gather blocks (see gat_bytes), one block per cell at a time.
+static __global__ void __launch_bounds__(256) gather_lists_kernel(DevMesh m, int np, int nf) {
+  for (int64_t c = blockIdx.x; c < m.C; c += gridDim.x) {
+    const int64_t n0 = m.node_ptr[c], k0 = m.sub_ptr[c], s0 = m.slot_ptr[c];
+    const int n = (int)(m.node_ptr[c + 1] - n0), S = (int)(m.sub_ptr[c + 1] - k0), ns = (int)(m.slot_ptr[c + 1] - s0);
+    unsigned char* blk = m.gat + gat_start(n0, k0, s0, c, np, nf);
+    uint16_t* list = reinterpret_cast<uint16_t*>(blk);
+    uint16_t* inc = reinterpret_cast<uint16_t*>(blk + gat_up(2 * (size_t)(2 * n + 3)));
+    float* face = reinterpret_cast<float*>(blk + gat_up(2 * (size_t)(2 * n + 3)) + gat_up(2 * (size_t)S * np));
+    uint16_t* info = reinterpret_cast<uint16_t*>(face + ns);
+    uint8_t* loc = reinterpret_cast<uint8_t*>(info + ns);
+    // nodes by decreasing list length (equal lengths in node order): a node's place and the
+    // offset of its list are sums over the nodes ahead of it
+    auto len = [&](int i) { return (int)(m.inc_ptr[n0 + i + 1] - m.inc_ptr[n0 + i]); };
+    int longs = 0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const int li = len(i);
+      int place = 0, off = 0;
+      for (int q = 0; q < n; ++q) {
+        const int lq = len(q);
+        if (lq > li || (lq == li && q < i)) {
+          ++place;
+          off += lq;
+        }
+      }
+      list[1 + 2 * place] = (uint16_t)i;
+      list[2 + 2 * place] = (uint16_t)off;
+      for (int e = 0; e < li; ++e) inc[off + e] = (uint16_t)m.inc[m.inc_ptr[n0 + i] + e];
+    }
+    if (threadIdx.x == 0) {
+      for (int i = 0; i < n; ++i) longs += len(i) > kLongList;
+      list[0] = (uint16_t)min(longs, kMaxLong);
+        list[2 + 2 * n] = (uint16_t)(S * np);
+    }
+    for (int s = threadIdx.x; s < ns; s += blockDim.x) {
+      int o = 6;  // local nodes 0 .. 3 are the sub-tet's vertices: the one missing lies opposite
+      for (int a = 0; a < nf; ++a) {
+        const int j = m.slot_loc[(s0 + s) * nf + a];
+        loc[s * nf + a] = (uint8_t)j;
+        if (j < 4) o -= j;
+      }
+      face[s] = (float)(0.5 / m.slot_geo[(s0 + s) * 4 + 3]);
+      info[s] = (uint16_t)(m.slot_sub[s0 + s] << 2 | o);
+    }
+  }
+}
+
+size_t pc_gather_bytes(const DevMesh& m, int64_t n_subtets, int np, int nf) {
+  return gat_start(m.n_nodes, n_subtets, m.n_slots, m.C, np, nf);
+}
+
+void pc_set_up(const DevMesh& m, int np, int nf, int grid, cudaStream_t st) {
+  split_minv_kernel<<<grid, 256, 0, st>>>(m);
+  gather_lists_kernel<<<grid, 256, 0, st>>>(m, np, nf);
+}
+#endif
+
+}  // namespace afe

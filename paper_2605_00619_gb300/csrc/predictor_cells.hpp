@@ -1,0 +1,40 @@
+// Host interface of the FP32 predictor with several cells in flight per SM (predictor_cells.cuh):
+// its plan, its launches and the set-up of the data it reads.  The kernels of each order are a
+// translation unit of their own (predictor_cells.cu compiled with AFE_ORDER = 1, 2, 3).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "kernels.cuh"
+
+namespace afe {
+
+// Time-basis constants.
+struct PcRef {
+  float w[4];       // Gauss-Legendre weights
+  float kw[4][4];   // K1t^-1[s][t] w_t
+  float kws[4];     // sum_t K1t^-1[s][t] w_t
+};
+
+// Launch plan: block shape (0: few cells, more warps each; 1: many cells), blocks per SM and
+// dynamic shared memory of a block.  blocks = 0: the cells do not fit.
+struct PcPlan {
+  int shape = 0;
+  int blocks = 0;
+  size_t smem = 0;
+};
+
+// Plan for `cells` cells of up to Nmax nodes, Smax sub-tets and Fmax face slots on n_sm SMs.
+template <int N>
+cudaError_t pc_plan(int device, int n_sm, int64_t cells, int Nmax, int Smax, int Fmax, PcPlan* out);
+
+// Launches the kernels of the kinds of cells that may be present.
+template <int N>
+void pc_launch(const PcPlan& plan, const Batch& b, const PcRef& ref, bool inviscid, bool viscous, int diag, int n_sm,
+               cudaStream_t st);
+
+// Bytes of the gather blocks of a mesh, and the set-up of m.m16 and m.gat.
+size_t pc_gather_bytes(const DevMesh& m, int64_t n_subtets, int np, int nf);
+void pc_set_up(const DevMesh& m, int np, int nf, int grid, cudaStream_t st);
+
+}  // namespace afe

@@ -18,6 +18,13 @@ namespace afe {
 // four consecutive rows hit 32 different shared-memory banks.
 inline constexpr int minv_ld(int n) { return (n + 15) / 16 * 16 + 8; }
 
+// Words (32 bits) of a cell's block of split M_i^-1 (pairs of 16-bit values): a 32-word header
+// (word 0: 1 / s), then the 16 x 16 tiles (i, j), j <= i, of the lower triangle at i (i + 1) / 2 + j,
+// 128 words of hi and 128 of lo each.
+inline constexpr int64_t minv_split_words(int n) {
+  return 32 + (int64_t)((n + 15) / 16) * ((n + 15) / 16 + 1) / 2 * 256;
+}
+
 struct Topology {
   int N = 0, Np = 0, Nt = 0, Nf = 0;
   int64_t C = 0, T = 0, n_nodes = 0, n_slots = 0, n_groups = 0;
@@ -26,7 +33,7 @@ struct Topology {
   std::vector<int64_t> node_ptr;   // [C+1] global node offset of each cell
   std::vector<int64_t> sub_ptr;    // [C+1] sub-tet offset of each cell
   std::vector<int64_t> slot_ptr;   // [C+1] face-slot offset of each cell
-  std::vector<int64_t> minv_ptr;   // [C+1] offset of the dense N_i x minv_ld(N_i) block of each cell
+  std::vector<int64_t> minv_ptr;   // [C+1] offset of each cell's block: dense N_i x minv_ld(N_i) rows, or the split form
 
   std::vector<uint16_t> A;         // [T*Np] cell-local node of sub-tet node j
   std::vector<double> geo;         // [T*10] adj(J) row-major (adj = det(J) J^-1), det(J)
@@ -34,7 +41,7 @@ struct Topology {
 
   // node -> (sub-tet, local node) incidences, cell-local sub-tet index, fixed order
   std::vector<int64_t> inc_ptr;    // [n_nodes+1]
-  std::vector<uint32_t> inc;       // (k_local << 5) | j
+  std::vector<uint32_t> inc;       // (k_local << 6) | j
 
   // face slots: one per cell-boundary sub-triangle, grouped by cell
   std::vector<int32_t> slot_cell;  // [n_slots]
