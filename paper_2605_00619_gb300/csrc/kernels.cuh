@@ -438,23 +438,81 @@ static __global__ void limiter_kernel(const __grid_constant__ Batch bt) {
   if (b > 0.0) atomicAdd(&m.flags[F_TROUBLED], 1);
 }
 
+// FP32 value of x by truncation, from its bits (integer instructions: the FP64 pipe, conversions
+// included, takes one lane or two per cycle and SM).  Relative error below 2^-23 when the result is
+// true in `ok`: x is zero or its exponent lies within +-100.
+__device__ __forceinline__ float f32_head(double x, bool& ok) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int e = (hi >> 20) & 0x7ff;
+  const bool zero = ((hi << 1) | lo) == 0;
+  ok = ok && (zero || (unsigned)(e - 923) <= 200u);
+  const unsigned bits = (unsigned)(hi & 0x80000000) | (unsigned)((e - 896) << 23) |
+                        (__funnelshift_l((unsigned)lo, (unsigned)hi, 3) & 0x7fffffu);
+  return zero ? 0.f : __uint_as_float(bits);
+}
+
 // CFL bound (Sec. 4.6): max over nodes of lambda + 2 lambda_v (2N+1)/h_i, one warp per cell,
 // folded into the member's maximum by an integer atomicMax on the bits of a non-negative
 // double (order-independent, hence deterministic).
-static __global__ void cfl_kernel(const __grid_constant__ Batch bt) {
+// The bound itself is FP64 arithmetic (a division and two square roots per node), and the FP64
+// pipe is what the kernel would wait for: on the 10.2 M nodes of a 32^3 P3 mesh 890 us, and 120 us as
+// it stands (62 us for the state's bytes at the copy rate); 24^3 P1 95 -> 38 us.  So every node first gets an interval around its bound in FP32; only nodes
+// whose upper end reaches the largest lower end seen (of the cell's nodes, and the maximum folded
+// so far) can be the maximum and are evaluated in FP64.  A node whose interval is in doubt (an
+// exponent out of range, a pressure that is not positive beyond its error) always is, so that
+// the maximum and the report of inadmissible states are those of evaluating every node.
+static __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__ Batch bt) {
   const int64_t gc = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (gc >= bt.cpre[bt.nh]) return;
   const int hh = batch_find(bt.cpre, bt.nh, gc);
   const DevMesh& m = bt.tab[hh];
   const int64_t c = gc - bt.cpre[hh];
-  const double mu_i = m.mu[c], kap = cell_kappa(m, mu_i), h = m.cell_hv[c];
+  const int64_t n0 = m.node_ptr[c], n1 = m.node_ptr[c + 1];
+  const double mu_i = m.mu[c], kap = cell_kappa(m, mu_i);
   // per cell: lambda_v = max(4 mu / 3, kappa / c_v) / rho, weighted by 2 (2N+1) / h
-  const double gam = m.gamma, visc = fmax(4.0 * mu_i / 3.0, kap / m.cv) * (2.0 * (2 * m.N + 1) / h);
+  const double gam = m.gamma;
+  const double visc =
+      mu_i == 0.0 && kap == 0.0 ? 0.0 : fmax(4.0 * mu_i / 3.0, kap / m.cv) * (2.0 * (2 * m.N + 1) / m.cell_hv[c]);
+  const float vf = (float)visc, gf = (float)gam, gg = gf * (gf - 1.f);
+  // interval of a node's bound: relative errors are a few 2^-23 of each term, kEps covers them
+  constexpr float kEps = 0x1p-18f;
+  auto interval = [&](const double (&q)[5], float& lower) {
+    bool ok = true;
+    const float r = f32_head(q[0], ok), a = f32_head(q[1], ok), b = f32_head(q[2], ok), d = f32_head(q[3], ok),
+                e = f32_head(q[4], ok);
+    const float ir = 1.f / r, m2 = (a * a + b * b + d * d) * ir;
+    const float c2 = gg * ir * (e - 0.5f * m2), err = kEps * gg * ir * (fabsf(e) + m2);
+    const float s = sqrtf(m2 * ir) + vf * ir;
+    const float lo = sqrtf(c2 - err), up = s + sqrtf(c2 + err);
+    // rho > 0, a pressure that is positive whatever the error, everything in range
+    ok = ok && r > 0.f && c2 > err && up < 1e30f && s >= 0.f;
+    lower = ok ? (s + lo) * (1.f - kEps) : 0.f;
+    return ok ? up * (1.f + kEps) : __int_as_float(0x7f800000);
+  };
+  auto load = [&](int64_t n, double (&q)[5]) {
+#pragma unroll
+    for (int v = 0; v < 5; ++v) q[v] = m.u[n * 5 + v];
+  };
+  float most = 0.f, least = 0.f;  // largest upper and lower end of this lane's nodes
+  for (int64_t n = n0 + lane; n < n1; n += 32) {
+    double q[5];
+    load(n, q);
+    float lower;
+    most = fmaxf(most, interval(q, lower));
+    least = fmaxf(least, lower);
+  }
+  least = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(least)));
+  const double seen = __longlong_as_double((long long)*(volatile unsigned long long*)m.maxbits);
+  const float floor_ = fmaxf(least, (float)seen * (1.f - kEps));
+  if (!__any_sync(0xffffffffu, most >= floor_)) return;
   double best = 0.0;
   bool bad = false;
-  for (int64_t n = m.node_ptr[c] + lane; n < m.node_ptr[c + 1]; n += 32) {
-    const double* q = m.u + n * 5;
+  for (int64_t n = n0 + lane; n < n1; n += 32) {
+    double q[5];
+    load(n, q);
+    float lower;
+    if (interval(q, lower) < floor_) continue;
     const double rho = q[0], ir = 1.0 / rho;  // one division per node
     const double m2 = q[1] * q[1] + q[2] * q[2] + q[3] * q[3];
     const double p = (gam - 1.0) * (q[4] - 0.5 * m2 * ir);

@@ -1,0 +1,68 @@
+"""The small kernels of a step at the states and sizes where they can go wrong."""
+import numpy as np
+import pytest
+
+from inputs import states
+from inputs.lattice import split_cube_lattice
+from inputs.voronoi import periodic_voronoi
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def afe():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2605_00619_gb300 import afe as a
+    a.lib()
+    return a
+
+
+def _bound(u, gamma=1.4):
+    u = u[np.isfinite(u[:, 0])]
+    rho, v, p = states.conserved_to_primitive(u, gamma)
+    return (np.linalg.norm(v, axis=1) + np.sqrt(gamma * p / rho)).max()
+
+
+# density scale, velocity scale, pressure scale: from rest to a kinetic energy that leaves the
+# pressure 1e-13 of the total, and values outside FP32's range
+@pytest.mark.parametrize("scales", [(1, 0, 1), (1, 1, 1), (1, 1e3, 1), (1, 1e5, 1e-3), (1e-9, 10, 1e-6), (1e40, 1, 1e41),
+                                    (1, 1e-40, 1), (1e-42, 1, 1e-42)])
+@pytest.mark.parametrize("N", [1, 3])
+def test_time_step_is_the_fp64_maximum(afe, N, scales):
+    """dt is inversely proportional to the largest bound over all nodes, evaluated in FP64: on one
+    mesh dt times the bound is the same for every state (to the rounding of its operations)."""
+    pm = periodic_voronoi(3)
+    h = afe.create_from_polymesh(pm, afe.afe_default_params(N, precision=afe.AFE_FP32, picard_tol=1e-6))
+    n = afe.afe_num_nodes(h)
+    rng = np.random.default_rng(3)
+
+    def dt_times_bound(u):
+        afe.afe_set_state(h, u)
+        return afe.afe_compute_dt(h) * _bound(u)
+
+    ref = dt_times_bound(states.primitive_to_conserved(np.ones(n), np.zeros((n, 3)), np.ones(n)))
+    for _ in range(3):
+        r, s, q = scales
+        u = states.primitive_to_conserved(r * rng.uniform(0.5, 2, n), s * rng.normal(size=(n, 3)), q * rng.uniform(0.5, 2, n))
+        p = states.conserved_to_primitive(u)[2]
+        if (p <= 0).any():  # rounding of the total energy: inadmissible, and reported
+            with pytest.raises(afe.AfeError):
+                dt_times_bound(u)
+            continue
+        # p = (gamma - 1) (E - m^2 / 2 rho) is rounded to 2^-52 of E on either side (products may be
+        # fused), which moves c = sqrt(gamma p / rho) by up to sqrt(gamma 2^-51 E / rho)
+        tol = 1e-12 + np.sqrt(1.4 * 2.0 ** -51 * u[:, 4] / u[:, 0]).max() / _bound(u)
+        assert abs(dt_times_bound(u) / ref - 1) <= tol
+    u = states.primitive_to_conserved(np.ones(n), rng.normal(size=(n, 3)), np.ones(n))
+    for bad in (np.nan, -1.0, np.inf):
+        w = u.copy()
+        w[n // 2, 0] = bad
+        if bad == np.inf:  # the bound as it is written is 0 there: no report, the other nodes decide
+            assert abs(dt_times_bound(w) / ref - 1) <= 1e-12
+            continue
+        afe.afe_set_state(h, w)
+        with pytest.raises(afe.AfeError):
+            afe.afe_compute_dt(h)
+    afe.afe_mesh_destroy(h)
