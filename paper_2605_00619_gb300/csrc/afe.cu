@@ -233,9 +233,14 @@ afe_status plan_f32(afe_mesh* m) {
 
 template <int N, typename Real>
 void launch_face(const StepPlan& P) {
-  const int64_t threads = P.b->gpre[P.b->nh] * 32;
-  const int blocks = (int)((threads + 255) / 256);
-  if (blocks > 0) afe::face_kernel<N, Real><<<blocks, 256, 0, P.st>>>(*P.b);
+  const int64_t faces = P.b->gpre[P.b->nh];
+  if (faces <= 0) return;
+  if constexpr (sizeof(Real) == 4) {
+    const int per_block = N == 1 ? 32 : (N == 2 ? 16 : 8);  // 8, 16 or 32 lanes per face
+    afe::face_f32_kernel<N><<<(unsigned)((faces + per_block - 1) / per_block), 256, 0, P.st>>>(*P.b);
+  } else {
+    afe::face_kernel<N, Real><<<(unsigned)((faces + 7) / 8), 256, 0, P.st>>>(*P.b);
+  }
 }
 
 template <int N, typename Real>
@@ -541,6 +546,8 @@ afe_status afe_mesh_create(const afe_params* p, int64_t n_vertices, const double
     if (rc) return fail(rc == 2 ? AFE_EMESH : AFE_EINVAL, err);
   }
 
+  if (m->topo.n_slots > (int64_t)INT32_MAX) return fail(AFE_EINVAL, "too many cell-boundary triangles");
+
   // ---- GPU part
   int ndev = 0;
   if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev == 0) return fail(AFE_ECUDA, "no CUDA device");
@@ -585,12 +592,16 @@ afe_status afe_mesh_create(const afe_params* p, int64_t n_vertices, const double
   AFE_TRY(M->upload((uint8_t**)&d.slot_loc, T.slot_loc));
   AFE_TRY(M->upload((uint16_t**)&d.slot_node, T.slot_node));
   AFE_TRY(M->upload((double**)&d.slot_geo, T.slot_geo));
-  AFE_TRY(M->upload((int64_t**)&d.slot_partner, T.slot_partner));
   AFE_TRY(M->upload((int32_t**)&d.slot_nbr, T.slot_nbr));
   AFE_TRY(M->upload((int64_t**)&d.finc_ptr, T.finc_ptr));
   AFE_TRY(M->upload((uint32_t**)&d.finc, T.finc));
   AFE_TRY(M->upload((int64_t**)&d.group_ptr, T.group_ptr));
-  AFE_TRY(M->upload((int64_t**)&d.group_slot, T.group_slot));
+  {
+    std::vector<int2> pairs(T.group_slot.size());
+    for (size_t i = 0; i < pairs.size(); ++i)
+      pairs[i] = make_int2((int)T.group_slot[i], (int)T.slot_partner[T.group_slot[i]]);
+    AFE_TRY(M->upload((int2**)&d.group_pair, pairs));
+  }
   AFE_TRY(M->upload((double**)&d.cell_vol, T.cell_vol));
   AFE_TRY(M->upload((double**)&d.cell_h, hcell));
   if (p->visc_dt_subtet) AFE_TRY(M->upload((double**)&d.cell_hv, T.cell_hsub));

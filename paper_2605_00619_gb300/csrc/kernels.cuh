@@ -43,12 +43,11 @@ struct DevMesh {
   const uint8_t* slot_loc;
   const uint16_t* slot_node;
   const double* slot_geo;
-  const int64_t* slot_partner;
   const int32_t* slot_nbr;
   const int64_t* finc_ptr;
   const uint32_t* finc;
   const int64_t* group_ptr;
-  const int64_t* group_slot;
+  const int2* group_pair;  // own-side slot and its partner (-1: domain boundary) of every sub-triangle
   const double* cell_vol;
   const double* cell_h;
   const double* cell_hv;  // length in the viscous term of the time step (cell_h or the sub-tet length)
@@ -861,7 +860,7 @@ __global__ void __launch_bounds__(256) predictor_kernel(DevMesh m, const RefData
 }
 
 // ----------------------------------------------------------------------------------------
-// Rusanov fluxes (Eq. 3.33) on the face nodes; one warp per polygonal face (all its
+// Rusanov fluxes (Eq. 3.33) on the face nodes, FP64 form; one warp per polygonal face (all its
 // sub-triangles, both sides).  The wave speeds are reduced over the face with warp
 // shuffles; G is written for the own side and, negated, for the matched side.
 template <int N, typename Real>
@@ -881,9 +880,9 @@ __global__ void face_kernel(const __grid_constant__ Batch bt) {
   const double dt = *m.dt;
   const Real idt = Real(1.0 / dt);
   const Real gam = (Real)m.gamma;
-  const int64_t s_first = m.group_slot[g0];
-  const int32_t ci = m.slot_cell[s_first];
-  const int32_t cj = m.slot_nbr[s_first];
+  const int2 p_first = m.group_pair[g0];
+  const int32_t ci = m.slot_cell[p_first.x];
+  const int32_t cj = p_first.y >= 0 ? m.slot_cell[p_first.y] : -1;
   const double mu_i = m.mu[ci], kap_i = cell_kappa(m, mu_i);
   const double mu_j = cj >= 0 ? m.mu[cj] : mu_i, kap_j = cell_kappa(m, mu_j);
   const double h_i = m.cell_h[ci], h_j = cj >= 0 ? m.cell_h[cj] : h_i;
@@ -893,9 +892,9 @@ __global__ void face_kernel(const __grid_constant__ Batch bt) {
   const Real rdt = (Real)dt;
   Real smax = 0, vmax = 0;
   for (int e = lane; e < nitems; e += 32) {
-    const int64_t s = m.group_slot[g0 + e / NF];
+    const int2 pair = m.group_pair[g0 + e / NF];
+    const int64_t s = pair.x, ps = pair.y;
     const int a = e % NF;
-    const int64_t ps = m.slot_partner[s];
     const double* g = m.slot_geo + s * 4;
     for (int side = 0; side < 2; ++side) {
       const int64_t ss = side == 0 ? s : ps;
@@ -920,9 +919,9 @@ __global__ void face_kernel(const __grid_constant__ Batch bt) {
   const Real diss = Real(0.5) * (smax + Real(2) * eps * vmax);
   for (int e = lane; e < nitems * 5; e += 32) {
     const int item = e / 5, v = e % 5;
-    const int64_t s = m.group_slot[g0 + item / NF];
+    const int2 pair = m.group_pair[g0 + item / NF];
+    const int64_t s = pair.x, ps = pair.y;
     const int a = item % NF;
-    const int64_t ps = m.slot_partner[s];
     const int64_t io = (s * NF + a) * 5 + v;
     if (ps < 0) {  // transmissive boundary: q+ = q-, F+ = F-
       sG[io] = sfn[io];
@@ -933,6 +932,128 @@ __global__ void face_kernel(const __grid_constant__ Batch bt) {
     const Real G = Real(0.5) * (sfn[io] - sfn[ip]) - diss * (sq[ip] - sq[io]);
     sG[io] = G;
     sG[ip] = -G;
+  }
+}
+
+// FP32 value of x to nearest, by integer instructions where x is zero or normal in FP32.
+__device__ __forceinline__ float f32_of(double x) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int e = (hi >> 20) & 0x7ff;
+  if (((hi << 1) | lo) == 0) return 0.f;
+  if ((unsigned)(e - 898) > 250u) return (float)x;
+  unsigned bits = (unsigned)(hi & 0x80000000) | (unsigned)((e - 896) << 23) |
+                  (__funnelshift_l((unsigned)lo, (unsigned)hi, 3) & 0x7fffffu);
+  const unsigned rest = (unsigned)lo & 0x1fffffffu;  // the 29 bits dropped
+  if (rest > 0x10000000u || (rest == 0x10000000u && (bits & 1u))) ++bits;
+  return __uint_as_float(bits);
+}
+
+// The FP32 form's fluxes: L lanes per polygonal face (8, 16, 32 at N = 1, 2, 3: about the face nodes of
+// three sub-triangles), the states and fluxes of a lane's first two face nodes held in registers
+// from the wave speeds to the fluxes.  What it waited for before: the FP64 pipe (1 / dt, eps and the
+// conversions of mu, h and the normals, per lane), then chains of dependent loads; the
+// conversions are integer instructions now and slots and partners come as one pair.
+// us per launch before and after: 32^3 P3 1,177 and 493 (127 for the bytes at
+// the copy rate), 21^3 P2 258 and 98, 24^3 P1 479 and 82, 4^3 P1 18 and 14.
+template <int N>
+__global__ void __launch_bounds__(256) face_f32_kernel(const __grid_constant__ Batch bt) {
+  constexpr int NF = nf_of(N), L = N == 1 ? 8 : (N == 2 ? 16 : 32), R = 2;
+  const int64_t ggw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / L;
+  const int lane = threadIdx.x % L;
+  const bool on = ggw < bt.gpre[bt.nh];  // whole groups of lanes; the others only take part in the shuffles
+  const int h = batch_find(bt.gpre, bt.nh, on ? ggw : 0);
+  const DevMesh& m = bt.tab[h];
+  const int64_t gw = on ? ggw - bt.gpre[h] : 0;
+  const int64_t g0 = m.group_ptr[gw], g1 = on ? m.group_ptr[gw + 1] : g0;
+  const int nitems = (int)(g1 - g0) * NF;
+  const float* sq = (const float*)m.slot_q;
+  const float* sfn = (const float*)m.slot_fn;
+  float* sG = (float*)m.slot_G;
+  const int2* pairs = m.group_pair + g0;
+  const float rdt = f32_of(*m.dt), idt = 1.f / rdt, gam = f32_of(m.gamma);
+  const int2 first = pairs[0];
+  const int32_t ci = m.slot_cell[first.x];
+  const int32_t cj = first.y >= 0 ? m.slot_cell[first.y] : ci;
+  // |lambda_v| = max(4 mu / 3, kappa / c_v) / rho: the coefficient per side
+  const float icv = 1.f / f32_of(m.cv), k0 = f32_of(m.kappa0), gcp = f32_of(m.gamma * m.cv / m.Pr);
+  const float mu_i = f32_of(m.mu[ci]), mu_j = f32_of(m.mu[cj]);
+  const bool given = m.kappa0 >= 0.0;
+  const float cvis_i = fmaxf(4.f / 3.f * mu_i, (given ? k0 : mu_i * gcp) * icv);
+  const float cvis_j = fmaxf(4.f / 3.f * mu_j, (given ? k0 : mu_j * gcp) * icv);
+  const float hsum = f32_of(m.cell_h[ci]) + f32_of(m.cell_h[cj]);
+  float smax = 0.f, vmax = 0.f;
+  auto speeds = [&](const float* Q, const float (&n)[3], float cvis) {
+    const float ir = 1.f / Q[0], rho = Q[0] * idt;
+    const float v0 = Q[1] * ir, v1 = Q[2] * ir, v2 = Q[3] * ir;  // q_bar / dt ratios
+    const float p = (gam - 1.f) * (Q[4] * idt - 0.5f * rho * (v0 * v0 + v1 * v1 + v2 * v2));
+    const float irho = ir * rdt;  // 1 / rho
+    smax = fmaxf(smax, fabsf(v0 * n[0] + v1 * n[1] + v2 * n[2]) + sqrtf(gam * p * irho));
+    vmax = fmaxf(vmax, cvis * irho);
+  };
+  auto load = [&](int e, int2& ps, int& a, float (&qo)[5], float (&qp)[5]) {
+    const int k = e / NF;
+    a = e - k * NF;
+    ps = pairs[k];
+    const double* g = m.slot_geo + (int64_t)ps.x * 4;
+    const float n[3] = {f32_of(g[0]), f32_of(g[1]), f32_of(g[2])};
+    const float* po = sq + ((int64_t)ps.x * NF + a) * 5;
+    const float* pp = sq + ((int64_t)max(ps.y, 0) * NF + a) * 5;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) qo[v] = po[v], qp[v] = pp[v];
+    speeds(qo, n, cvis_i);
+    if (ps.y >= 0) speeds(qp, n, cvis_j);
+  };
+  int2 ps[R];
+  int a[R];
+  float qo[R][5], qp[R][5], fo[R][5], fp[R][5];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int e = lane + r * L;
+    if (e >= nitems) continue;
+    load(e, ps[r], a[r], qo[r], qp[r]);
+    const float* po = sfn + ((int64_t)ps[r].x * NF + a[r]) * 5;
+    const float* pp = sfn + ((int64_t)max(ps[r].y, 0) * NF + a[r]) * 5;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) fo[r][v] = po[v], fp[r][v] = pp[v];
+  }
+  for (int e = lane + R * L; e < nitems; e += L) {
+    int2 p2;
+    int a2;
+    float q1[5], q2[5];
+    load(e, p2, a2, q1, q2);
+  }
+#pragma unroll
+  for (int o = L / 2; o > 0; o >>= 1) {
+    smax = fmaxf(smax, __shfl_xor_sync(0xffffffffu, smax, o));
+    vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
+  }
+  // eps = (2N+1) / ((h_i + h_j) sqrt(pi / 2))
+  const float eps = (2 * N + 1) * 0.797884560802865f / hsum;
+  const float diss = 0.5f * (smax + 2.f * eps * vmax);
+  auto flux = [&](int2 p, int a1, const float* q1, const float* q2, const float* f1, const float* f2) {
+    float* go = sG + ((int64_t)p.x * NF + a1) * 5;
+    if (p.y < 0) {  // transmissive boundary: q+ = q-, F+ = F-
+#pragma unroll
+      for (int v = 0; v < 5; ++v) go[v] = f1[v];
+      return;
+    }
+    float* gp = sG + ((int64_t)p.y * NF + a1) * 5;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      // the matched side stores F_bar . (its own normal) = -F_bar+ . n
+      const float G = 0.5f * (f1[v] - f2[v]) - diss * (q2[v] - q1[v]);
+      go[v] = G;
+      gp[v] = -G;
+    }
+  };
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+    if (lane + r * L < nitems) flux(ps[r], a[r], qo[r], qp[r], fo[r], fp[r]);
+  for (int e = lane + R * L; e < nitems; e += L) {
+    const int k = e / NF, a2 = e - k * NF;
+    const int2 p2 = pairs[k];
+    const int64_t io = ((int64_t)p2.x * NF + a2) * 5, ip = ((int64_t)max(p2.y, 0) * NF + a2) * 5;
+    flux(p2, a2, sq + io, sq + ip, sfn + io, sfn + ip);
   }
 }
 
