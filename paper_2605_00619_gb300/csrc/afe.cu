@@ -298,9 +298,8 @@ afe_status stage(const StepPlan& P, int s) { return P.fp32 ? dispatch_stage<floa
 afe_status enqueue_dt(const StepPlan& P, double dt) {
   const int64_t C = P.b->cpre[P.b->nh];
   if (P.limiter) {
-    const int cgrid = (int)std::min<int64_t>(C, (int64_t)P.n_sm * 8);
-    afe::cell_means_kernel<<<cgrid, 256, 0, P.st>>>(*P.b);
-    afe::limiter_kernel<<<(int)((C + 127) / 128), 128, 0, P.st>>>(*P.b);
+    afe::cell_means_kernel<<<(int)((C + 7) / 8), 256, 0, P.st>>>(*P.b);
+    afe::limiter_kernel<<<(int)((C + 7) / 8), 256, 0, P.st>>>(*P.b);
   }
   if (dt > 0) {
     afe::set_dt_kernel<<<1, 64, 0, P.st>>>(*P.b, dt);
@@ -801,8 +800,8 @@ afe_status afe_cfl_pieces(afe_mesh* m, int64_t n_cells, double* bracket_max, dou
   afe::step_begin_kernel<<<1, 64, 0, P.st>>>(*P.b);
   if (P.limiter) {  // the viscosity of every cell of the handle
     const int64_t C = m->topo.C;
-    afe::cell_means_kernel<<<(int)std::min<int64_t>(C, (int64_t)P.n_sm * 8), 256, 0, P.st>>>(*P.b);
-    afe::limiter_kernel<<<(int)((C + 127) / 128), 128, 0, P.st>>>(*P.b);
+    afe::cell_means_kernel<<<(int)((C + 7) / 8), 256, 0, P.st>>>(*P.b);
+    afe::limiter_kernel<<<(int)((C + 7) / 8), 256, 0, P.st>>>(*P.b);
   }
   afe::Batch sub = m->self;  // the bracket over the first n_cells cells only
   sub.cpre[1] = n_cells;

@@ -64,7 +64,7 @@ struct DevMesh {
   int32_t* iters;
   double* beta;
   double* mu;     // per-cell dynamic viscosity mu_i (physical + artificial)
-  double* means;  // [C][5] cell means
+  double* means;  // [C][5] density, velocity and sound speed of the cell means
   double* dt;     // device scalar: time step of the current step
   double* tacc;   // device scalar: accumulated time
   unsigned long long* maxbits;
@@ -371,69 +371,78 @@ static __global__ void step_begin_kernel(const __grid_constant__ Batch bt) {
   if (threadIdx.x < 2) bt.work[threadIdx.x] = 0;
 }
 
-// Sec. 4.5: cell means u_bar_i = w_i . u_i / |P_i|  (w_i = M_i 1), one block per cell at a time.
-static __global__ void cell_means_kernel(const __grid_constant__ Batch bt) {
-  __shared__ double sh[5][256];
-  const int64_t total = bt.cpre[bt.nh];
-  for (int64_t gc = blockIdx.x; gc < total; gc += gridDim.x) {
-    const int hh = batch_find(bt.cpre, bt.nh, gc);
-    const DevMesh& m = bt.tab[hh];
-    if (!m.limiter) continue;  // block-uniform
-    const int64_t c = gc - bt.cpre[hh];
-    const int64_t n0 = m.node_ptr[c], n1 = m.node_ptr[c + 1];
-    double acc[5] = {0, 0, 0, 0, 0};
-    for (int64_t n = n0 + threadIdx.x; n < n1; n += blockDim.x) {
-      const double w = m.wvec[n];
+// Sec. 4.5: cell means u_bar_i = w_i . u_i / |P_i| (w_i = M_i 1), one warp per cell, kept as what the
+// detector reads of them, once per cell instead of once per neighbour: density, velocity and
+// sound speed.
+static __global__ void __launch_bounds__(256) cell_means_kernel(const __grid_constant__ Batch bt) {
+  const int64_t gc = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (gc >= bt.cpre[bt.nh]) return;
+  const int hh = batch_find(bt.cpre, bt.nh, gc);
+  const DevMesh& m = bt.tab[hh];
+  if (!m.limiter) return;  // warp-uniform
+  const int64_t c = gc - bt.cpre[hh];
+  double acc[5] = {0, 0, 0, 0, 0};
+  for (int64_t n = m.node_ptr[c] + lane; n < m.node_ptr[c + 1]; n += 32) {
+    const double w = m.wvec[n];
 #pragma unroll
-      for (int v = 0; v < 5; ++v) acc[v] += w * m.u[n * 5 + v];
-    }
-#pragma unroll
-    for (int v = 0; v < 5; ++v) sh[v][threadIdx.x] = acc[v];
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-      if (threadIdx.x < s)
-#pragma unroll
-        for (int v = 0; v < 5; ++v) sh[v][threadIdx.x] += sh[v][threadIdx.x + s];
-      __syncthreads();
-    }
-    if (threadIdx.x < 5) m.means[c * 5 + threadIdx.x] = sh[threadIdx.x][0] / m.cell_vol[c];
-    __syncthreads();
+    for (int v = 0; v < 5; ++v) acc[v] += w * m.u[n * 5 + v];
   }
+#pragma unroll
+  for (int v = 0; v < 5; ++v)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc[v] += __shfl_xor_sync(0xffffffffu, acc[v], o);
+  if (lane) return;
+  const double vol = m.cell_vol[c];
+  double q[5], vel[3];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) q[v] = acc[v] / vol;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) vel[d] = q[1 + d] / q[0];
+  const double p = (m.gamma - 1.0) * (q[4] - 0.5 * q[0] * (vel[0] * vel[0] + vel[1] * vel[1] + vel[2] * vel[2]));
+  double* out = m.means + c * 5;
+  out[0] = q[0];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) out[1 + d] = vel[d];
+  out[4] = sqrt(m.gamma * p / q[0]);
 }
 
 // Artificial-viscosity limiter (Sec. 4.5, Eq. beta3D): beta_i from the discrete velocity
 // divergence of the cell means over the faces of P_i, mu_i = mu + beta_i rho_i lambda_i h_i/(2N+1).
-static __global__ void limiter_kernel(const __grid_constant__ Batch bt) {
-  const int64_t gc = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+// One warp per cell, its lanes on the face slots: with a thread per cell the some 45 slots, each with
+// its neighbour's divisions and square root in FP64, were one serial chain (limiter stage 270 us
+// whatever the size of the mesh; before and after with the time step: 15^3 P3 338 and 165 us, batch of ten P2 3,676 and 3,077 us per pass).
+static __global__ void __launch_bounds__(256) limiter_kernel(const __grid_constant__ Batch bt) {
+  const int64_t gc = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
   if (gc >= bt.cpre[bt.nh]) return;
   const int hh = batch_find(bt.cpre, bt.nh, gc);
   const DevMesh& m = bt.tab[hh];
   if (!m.limiter) return;  // a batch member without the limiter keeps beta = 0, mu_i = mu
   const int64_t c = gc - bt.cpre[hh];
-  auto prim = [&](int64_t i, double v[3], double& rho, double& cs) {
-    const double* q = m.means + i * 5;
-    rho = q[0];
-    for (int d = 0; d < 3; ++d) v[d] = q[1 + d] / rho;
-    const double p = (m.gamma - 1.0) * (q[4] - 0.5 * rho * (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]));
-    cs = sqrt(m.gamma * p / rho);
-  };
-  double vi[3], rhoi, ci;
-  prim(c, vi, rhoi, ci);
-  double div = 0.0, cmin = ci;
-  for (int64_t s = m.slot_ptr[c]; s < m.slot_ptr[c + 1]; ++s) {
+  double own[5];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) own[v] = m.means[c * 5 + v];
+  double div = 0.0, cmin = own[4];
+  for (int64_t s = m.slot_ptr[c] + lane; s < m.slot_ptr[c + 1]; s += 32) {
     const int32_t nb = m.slot_nbr[s];
     if (nb < 0) continue;
-    double vj[3], rj, cj;
-    prim(nb, vj, rj, cj);
+    const double* q = m.means + (int64_t)nb * 5;
     const double* g = m.slot_geo + s * 4;
-    div += g[3] * ((vj[0] - vi[0]) * g[0] + (vj[1] - vi[1]) * g[1] + (vj[2] - vi[2]) * g[2]);
-    cmin = fmin(cmin, cj);
+    div += g[3] * ((q[1] - own[1]) * g[0] + (q[2] - own[2]) * g[1] + (q[3] - own[3]) * g[2]);
+    cmin = fmin(cmin, q[4]);
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    div += __shfl_xor_sync(0xffffffffu, div, o);
+    cmin = fmin(cmin, __shfl_xor_sync(0xffffffffu, cmin, o));
+  }
+  if (lane) return;
   div /= m.cell_vol[c];
   const double b = fmin(1.0, fmax(0.0, -(div + m.m1 * cmin) / (m.m1 * cmin)));
   m.beta[c] = b;
-  const double lam = sqrt(vi[0] * vi[0] + vi[1] * vi[1] + vi[2] * vi[2]) + ci;
-  m.mu[c] = m.mu0 + b * rhoi * lam * m.cell_h[c] / (2 * m.N + 1);
+  const double lam = sqrt(own[1] * own[1] + own[2] * own[2] + own[3] * own[3]) + own[4];
+  m.mu[c] = m.mu0 + b * own[0] * lam * m.cell_h[c] / (2 * m.N + 1);
   if (b > 0.0) atomicAdd(&m.flags[F_TROUBLED], 1);
 }
 
@@ -505,13 +514,23 @@ static __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__
   const double seen = __longlong_as_double((long long)*(volatile unsigned long long*)m.maxbits);
   const float floor_ = fmaxf(least, (float)seen * (1.f - kEps));
   if (!__any_sync(0xffffffffu, most >= floor_)) return;
-  double best = 0.0;
-  bool bad = false;
+  double best = 0.0, last[5] = {0, 0, 0, 0, 0};
+  bool bad = false, any = false;
   for (int64_t n = n0 + lane; n < n1; n += 32) {
     double q[5];
     load(n, q);
     float lower;
     if (interval(q, lower) < floor_) continue;
+    // in a uniform region every node is a candidate: a state equal to the lane's last, bit for
+    // bit, has its bound already
+    bool same = any;
+    any = true;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      same = same && __double_as_longlong(q[v]) == __double_as_longlong(last[v]);
+      last[v] = q[v];
+    }
+    if (same) continue;
     const double rho = q[0], ir = 1.0 / rho;  // one division per node
     const double m2 = q[1] * q[1] + q[2] * q[2] + q[3] * q[3];
     const double p = (gam - 1.0) * (q[4] - 0.5 * m2 * ir);
