@@ -67,6 +67,7 @@ struct afe_mesh {
   afe_schedule sched{};  // predictor schedule (cost order, ring cap, narrow chunks; variant above)
   int32_t* d_order = nullptr;  // the cells in decreasing cost (allocated when first asked for)
   size_t f32_smem = 0;
+  afe::CorrRef cref{};   // ... and the face mass of its corrector
   afe::PcRef pref{};     // time-basis constants of the predictor with several cells per SM
   afe::PcPlan pc{};           // its plan for this mesh's cells (blocks = 0: not used)
   double* d_totals_partial = nullptr;
@@ -126,6 +127,7 @@ struct StepPlan {
   size_t f32_smem = 0;
   afe::PcPlan pc;
   afe::PcRef pref{};
+  afe::CorrRef cref{};
   int inviscid = 0, viscous = 0;  // cells without / with viscous fluxes may be present
   const afe::RefData* d_ref = nullptr;
   afe_mesh* single = nullptr;  // nullptr for a batch (FP32 shared-memory kernels only)
@@ -159,6 +161,7 @@ StepPlan plan_of(afe_mesh* m) {
   P.f32_smem = m->f32_smem;
   P.pc = m->pc;
   P.pref = m->pref;
+  P.cref = m->cref;
   P.d_ref = m->d_ref;
   P.single = m;
   P.prof = m;
@@ -245,6 +248,11 @@ void launch_face(const StepPlan& P) {
 
 template <int N, typename Real>
 afe_status launch_corrector(const StepPlan& P) {
+  if constexpr (N <= 3)
+    if (sizeof(Real) == 4 && P.pc.blocks) {  // the cells' split M_i^-1 is there
+      afe::pc_correct<N>(*P.b, P.cref, P.b->Nmax, P.pc.Fmax, P.st);
+      return AFE_OK;
+    }
   if (sizeof(Real) == 4 && corrector_f32_fits(P.b->Nmax)) {
     const size_t smem = (size_t)P.b->Nmax * 10 * sizeof(float);
     if (smem > 48 * 1024)
@@ -411,6 +419,11 @@ afe_status set_up_cells(afe_mesh* m, int64_t nminv) {
     }
     m->pref.kws[s] = (float)sum;
   }
+  for (int a = 0; a < R.Nf && R.Nf <= 10; ++a)
+    for (int b = 0; b < R.Nf; ++b) {
+      m->cref.Z[a][b] = (float)R.Z[a][b];
+      m->cref.zs[b] += R.Z[a][b];
+    }
   afe::PcPlan pc;
   AFE_TRY(plan_cells(m->p.order, m->device, m->n_sm, T.C, T.Nmax, T.Smax, T.slots_max, &pc));
   if (!pc.blocks) return AFE_OK;
@@ -1156,6 +1169,7 @@ afe_status afe_batch_create(afe_mesh* const* members, int n_members, void* cuda_
   P.f32_ok = 1;
   P.f32_smem = m0->f32_smem;
   P.pref = m0->pref;
+  P.cref = m0->cref;
   for (afe_mesh* m : b->mem) add_kinds(&P, m);
   {
     int Fmax = 0;

@@ -23,6 +23,14 @@ template <bool V> struct PcShape<3, 1, V> { static constexpr int W = 8, MB = 2; 
 template <int N, int SHAPE, bool VISC>
 constexpr auto pc_kernel = predictor_cells_kernel<N, PcShape<N, SHAPE, VISC>::W, PcShape<N, SHAPE, VISC>::MB, VISC>;
 
+// Warps per block of the corrector.
+template <int N>
+constexpr int corr_warps = N == 3 ? 8 : (N == 2 ? 4 : 1);
+
+size_t corr_smem(int n, int ns, int nf) {
+  return (size_t)(n + 15) / 16 * 320 + (size_t)((n * 5 + 3) & ~3) * 4 + (size_t)ns * nf * 20;
+}
+
 template <int N, int SHAPE>
 cudaError_t plan_shape(int device, int Nmax, int Smax, int Fmax, PcPlan* out) {
   constexpr int W = PcShape<N, SHAPE, false>::W, MB = PcShape<N, SHAPE, false>::MB, THR = 32 * W;
@@ -45,6 +53,13 @@ cudaError_t plan_shape(int device, int Nmax, int Smax, int Fmax, PcPlan* out) {
     e = cudaFuncSetAttribute(pc_kernel<N, SHAPE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - stat);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(pc_kernel<N, SHAPE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - stat);
+    auto* corr = corrector_cells_kernel<N, corr_warps<N>>;
+    cudaFuncAttributes fc;
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fc, corr);
+    if (e != cudaSuccess) return e;
+    if (corr_smem(Nmax, Fmax, nf_of(N)) > optin - fc.sharedSizeBytes) return cudaSuccess;
+    e = cudaFuncSetAttribute(corr, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fc.sharedSizeBytes);
+    out->Fmax = Fmax;
     out->shape = SHAPE;
     out->blocks = nb;
     out->smem = smem;
@@ -87,6 +102,13 @@ void pc_launch(const PcPlan& p, const Batch& b, const PcRef& ref, bool inviscid,
   else launch_shape<N, 0>(p, b, ref, inviscid, viscous, diag, n_sm, st);
 }
 
+template <int N>
+void pc_correct(const Batch& b, const CorrRef& ref, int Nmax, int Fmax, cudaStream_t st) {
+  corrector_cells_kernel<N, corr_warps<N>>
+      <<<(unsigned)b.cpre[b.nh], 32 * corr_warps<N>, corr_smem(Nmax, Fmax, nf_of(N)), st>>>(b, ref);
+}
+
+template void pc_correct<AFE_ORDER>(const Batch&, const CorrRef&, int, int, cudaStream_t);
 template cudaError_t pc_plan<AFE_ORDER>(int, int, int64_t, int, int, int, PcPlan*);
 template void pc_launch<AFE_ORDER>(const PcPlan&, const Batch&, const PcRef&, bool, bool, int, int, cudaStream_t);
 

@@ -1033,4 +1033,234 @@ __global__ void __launch_bounds__(32 * W, MB) predictor_cells_kernel(const __gri
   }
 }
 
+// ----------------------------------------------------------------------------------------
+// FP32 corrector on the split M_i^-1 (Sec. 4.4), one block of W warps per cell.
+//   f[slot][a] = 2 area sum_b Z^[a][b] G[b]     (a thread per slot and variable, once per slot)
+//   r = vol - sum over the node's face incidences of f   (fixed order)
+//   du = M_i^-1 r on the tensor cores: the operands, tiles and products of the predictor's first
+//        iteration (5 columns)
+//   u += du + (T - w_i . du) / |P_i|            (FP64: T = exact cell total of r, see
+//                                                corrector_f32_kernel)
+// What bounds it: M_i^-1 from HBM, once per step.  The lower triangle in 16-bit pairs is 53 % of the
+// FP32 rows that corrector_f32_kernel streams (75 % of the copy rate there); each tile is read a
+// second time for its mirror, from L2, which holds the cells in flight as long as few blocks
+// share an SM (three: 2,210 us at 32^3 P3, two 2,841).  FP64 work per node is kept to the update
+// itself and conversions are integer instructions: with ten FP64 reductions per warp and FP64
+// admissibility tests the launch took 3,017 us.
+// us per launch, corrector_f32_kernel and here: 32^3 P3 3,155 and 2,210 (1,500 for the bytes at the copy
+// rate), 16^3 P3 465 and 310, 21^3 P2 432 and 200, 24^3 P1 436 and 121, 8^3 P2 49 and 26.
+__device__ __forceinline__ double f64_of(float x) {
+  const unsigned b = __float_as_uint(x), e = b >> 23 & 255u;
+  if (e - 1u >= 254u) return (double)x;  // zero, denormal, infinity, NaN
+  return __hiloint2double((int)((b & 0x80000000u) | ((b & 0x7fffffffu) >> 3) + 0x38000000u), (int)(b << 29));
+}
+
+template <int N, int W>
+__global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) corrector_cells_kernel(
+    const __grid_constant__ Batch bt, const __grid_constant__ CorrRef ref) {
+  constexpr int NF = nf_of(N), THR = 32 * W, DP = N == 1 ? 2 : kPcDeep;
+  extern __shared__ __align__(128) unsigned char pc_smem[];
+  __shared__ double sred[10][W];
+  __shared__ float smax[5][W];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t gc = blockIdx.x;
+  const int h = batch_find(bt.cpre, bt.nh, gc);
+  const DevMesh& m = bt.tab[h];
+  const int64_t c = gc - bt.cpre[h];
+  const int64_t n0 = m.node_ptr[c], s0 = m.slot_ptr[c];
+  const int Ni = (int)(m.node_ptr[c + 1] - n0), ns = (int)(m.slot_ptr[c + 1] - s0), nks = (Ni + 15) / 16;
+  const uint32_t* const m16 = m.m16 + m.minv_ptr[c];
+  unsigned char* const frag = pc_smem;                                   // [nks][320] split right-hand side
+  float* const sr = reinterpret_cast<float*>(pc_smem + nks * 320);       // [N_i][5] r, then du
+  float* const sf = sr + ((Ni * 5 + 3) & ~3);                            // [ns][NF][5] face integrals
+  const float* const vol = (const float*)m.vol;
+  const float* const sG = (const float*)m.slot_G;
+  if (warp == W - 1) {  // M_i^-1 on its way into L2
+    const uint32_t bytes = (uint32_t)(minv_split_words(Ni) - 32) * 4u;
+    for (uint32_t o = lane * 8192u; o < bytes; o += 32 * 8192u)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<const unsigned char*>(m16 + 32) + o),
+                   "r"(min(8192u, bytes - o))
+                   : "memory");
+  }
+  // face integrals and the FP64 cell total of the update, item (slot, variable)
+  double tot = 0.0;  // of variable tid % 5 (the stride keeps it)
+  constexpr int FS = THR / 5 * 5;
+  for (int e = tid; e < ns * 5 && tid < FS; e += FS) {
+    const int sl = e / 5, v = e - sl * 5;
+    const float* g = sG + (s0 + sl) * NF * 5 + v;
+    const double twoA = 2.0 * m.slot_geo[(s0 + sl) * 4 + 3];
+    const float tA = f32_of(twoA);
+    float x[NF];
+#pragma unroll
+    for (int b = 0; b < NF; ++b) x[b] = g[b * 5];
+    double z = 0.0;
+#pragma unroll
+    for (int b = 0; b < NF; ++b) z += ref.zs[b] * f64_of(x[b]);
+    tot -= twoA * z;
+#pragma unroll
+    for (int a = 0; a < NF; ++a) {
+      float f = 0.f;
+#pragma unroll
+      for (int b = 0; b < NF; ++b) f += ref.Z[a][b] * x[b];
+      sf[(sl * NF + a) * 5 + v] = tA * f;
+    }
+  }
+  __syncthreads();
+  float mx[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+  for (int n = tid; n < Ni; n += THR) {
+    float acc[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) acc[v] = vol[(n0 + n) * 5 + v];
+    const int64_t p1 = m.finc_ptr[n0 + n + 1];
+    for (int64_t p = m.finc_ptr[n0 + n]; p < p1; ++p) {
+      const uint32_t w = m.finc[p];
+      const float* f = sf + ((w >> 4) * NF + (w & 15)) * 5;
+#pragma unroll
+      for (int v = 0; v < 5; ++v) acc[v] -= f[v];
+    }
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      sr[n * 5 + v] = acc[v];
+      mx[v] = fmaxf(mx[v], fabsf(acc[v]));
+    }
+  }
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    const float x = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx[v])));
+    if (lane == 0) smax[v][warp] = x;
+  }
+  __syncthreads();
+  // split right-hand side in fragment order, a power of two per variable
+  float sc[5], isc[5];
+  const float is0 = __uint_as_float(m16[0]);
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    float x = smax[v][0];
+#pragma unroll
+    for (int w = 1; w < W; ++w) x = fmaxf(x, smax[v][w]);
+    const int e = f16_scale_exp(__float_as_uint(x));
+    sc[v] = __uint_as_float((uint32_t)e << 23);
+    isc[v] = __uint_as_float((uint32_t)(254 - e) << 23);
+  }
+  for (int n = tid; n < 16 * nks; n += THR) {
+    unsigned char* b = frag + (n >> 4) * 320 + ((n & 7) >> 1) * 16 + ((n >> 3) & 1) * 4 + (n & 1) * 2;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      const float y = n < Ni ? sr[n * 5 + v] * sc[v] : 0.f;
+      const __half hi = __float2half_rn(y);
+      *reinterpret_cast<__half*>(b + v * 64) = hi;
+      *reinterpret_cast<__half*>(b + v * 64 + 8) = __float2half_rn(y - __half2float(hi));
+    }
+  }
+  __syncthreads();
+  for (int mt = warp; mt < nks; mt += W) {
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    const uint32_t* const a0 = m16 + 32 + lane * 4;
+    uint4 ah[DP], al[DP];
+    auto load = [&](int s, int ks) {
+      const uint32_t* t = a0 + tri_tile(mt, min(ks, nks - 1)) * 256;
+      ah[s] = ldg_stream(t);
+      al[s] = ldg_stream(t + 128);
+    };
+    auto step = [&](int s, int ks) {
+      const uint4 b = lane < 20 ? *reinterpret_cast<const uint4*>(frag + ks * 320 + lane * 16) : make_uint4(0, 0, 0, 0);
+      uint4 x = ah[s], l = al[s];
+      if (ks > mt) {  // above the diagonal: the mirrored tile
+        x = transpose16(x);
+        l = transpose16(l);
+      }
+      mma_f16(acc, l, b.x, b.y);
+      mma_f16(acc, x, b.z, b.w);
+      mma_f16(acc, x, b.x, b.y);
+    };
+#pragma unroll
+    for (int s = 0; s < DP; ++s) load(s, s);
+    int ks = 0;
+    for (; ks + DP <= nks; ks += DP) {
+#pragma unroll
+      for (int s = 0; s < DP; ++s) {
+        step(s, ks + s);
+        load(s, ks + s + DP);
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < DP - 1; ++s)
+      if (ks + s < nks) step(s, ks + s);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int v = 2 * (lane & 3) + (i & 1), n = mt * 16 + (lane >> 2) + (i >> 1) * 8;
+      if (v < 5 && n < Ni) {
+        float si = isc[0];
+#pragma unroll
+        for (int q = 1; q < 5; ++q)
+          if (v == q) si = isc[q];
+        sr[n * 5 + v] = (acc[i] * is0) * si;
+      }
+    }
+  }
+  __syncthreads();
+  // FP64 totals: target (per thread one variable) minus w . du, in a fixed order.  The FP64 pipe takes
+  // 64 cycles per warp instruction and scheduler: the five sums share their shuffles (lanes 0-15
+  // keep one sum, 16-31 another, and so on), one warp adds up the warps' parts.
+  double d[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  for (int n = tid; n < Ni; n += THR) {
+    const double w = -m.wvec[n0 + n];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) d[v] += w * f64_of(sr[n * 5 + v]);
+  }
+  if (tid < FS && tid < ns * 5) {
+    const int tv = tid % 5;
+#pragma unroll
+    for (int v = 0; v < 5; ++v)
+      if (tv == v) d[v] += tot;
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {  // 8 sums over 32 lanes -> one sum per lane, over 4 lanes
+    const int half = 4 >> k, o = 16 >> k;
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < half; ++i) {
+      const double send = up ? d[i] : d[i + half], keep = up ? d[i + half] : d[i];
+      d[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  d[0] += __shfl_xor_sync(0xffffffffu, d[0], 2);
+  d[0] += __shfl_xor_sync(0xffffffffu, d[0], 1);
+  if ((lane & 3) == 0 && lane < 20) sred[lane >> 2][warp] = d[0];  // lanes 4 v .. 4 v + 3 hold sum v
+  __syncthreads();
+  if (warp == 0) {
+    double x = 0.0;
+    if (lane < 5) {
+#pragma unroll
+      for (int w = 0; w < W; ++w) x += sred[lane][w];
+      sred[5 + lane][0] = x / m.cell_vol[c];
+    }
+  }
+  __syncthreads();
+  double corr[5];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) corr[v] = sred[5 + v][0];
+  for (int n = tid; n < Ni; n += THR) {
+    double* un = m.u + (n0 + n) * 5;
+    double x[5];
+    bool ok = true;
+    float xf[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      x[v] = un[v] + (f64_of(sr[n * 5 + v]) + corr[v]);
+      un[v] = x[v];
+      xf[v] = f32_head(x[v], ok);
+    }
+    // rho > 0 and p > 0, with p > 0 tested as rho E > |rho u|^2 / 2 (no division): in FP32 where the
+    // margin is beyond its error, else in FP64, which also sees infinities and NaN
+    const float a = xf[0] * xf[4], b = 0.5f * (xf[1] * xf[1] + xf[2] * xf[2] + xf[3] * xf[3]);
+    if (ok && xf[0] > 0.f && xf[4] > 0.f && a > 1e-30f && a < 1e37f && a - b > 0x1p-18f * (a + b)) continue;
+    bool bad = false;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) bad |= !isfinite(x[v]);
+    const double pr = x[0] * x[4] - 0.5 * (x[1] * x[1] + x[2] * x[2] + x[3] * x[3]);
+    if (bad || !(x[0] > 0.0) || !(pr > 0.0)) atomicOr(&m.flags[F_NONFINITE], 8);
+  }
+}
+
 }  // namespace afe

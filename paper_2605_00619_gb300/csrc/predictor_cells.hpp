@@ -16,12 +16,19 @@ struct PcRef {
   float kws[4];     // sum_t K1t^-1[s][t] w_t
 };
 
+// Constants of the corrector on the split M_i^-1.
+struct CorrRef {
+  float Z[10][10];   // face mass on the unit right triangle
+  double zs[10];     // its column sums
+};
+
 // Launch plan: block shape (0: few cells, more warps each; 1: many cells), blocks per SM and
-// dynamic shared memory of a block.  blocks = 0: the cells do not fit.
+// dynamic shared memory of a block; most face slots of a cell.  blocks = 0: the cells do not fit.
 struct PcPlan {
   int shape = 0;
   int blocks = 0;
   size_t smem = 0;
+  int Fmax = 0;
 };
 
 // Plan for `cells` cells of up to Nmax nodes, Smax sub-tets and Fmax face slots on n_sm SMs.
@@ -32,6 +39,10 @@ cudaError_t pc_plan(int device, int n_sm, int64_t cells, int Nmax, int Smax, int
 template <int N>
 void pc_launch(const PcPlan& plan, const Batch& b, const PcRef& ref, bool inviscid, bool viscous, int diag, int n_sm,
                cudaStream_t st);
+
+// The corrector on the split M_i^-1 for cells of up to Nmax nodes and Fmax face slots.
+template <int N>
+void pc_correct(const Batch& b, const CorrRef& ref, int Nmax, int Fmax, cudaStream_t st);
 
 // Bytes of the gather blocks of a mesh, and the set-up of m.m16 and m.gat.
 size_t pc_gather_bytes(const DevMesh& m, int64_t n_subtets, int np, int nf);
