@@ -54,9 +54,10 @@ def build(verbose: bool = False, extra_flags=None) -> str:
         obj = os.path.join(objdir, src + ".o")
         jobs.append([os.environ.get("CXX", "g++"), *common, "-fPIC", "-Wall", "-c",
                      os.path.join(CSRC, src), "-o", obj])
-    # the CUDA translation units: the library, and one per order of predictor_cells
+    # the CUDA translation units: the library, and one per order of the predictors
     units = [("afe.cu", "afe.cu.o", [])]
     units += [("predictor_cells.cu", f"predictor_cells_{n}.o", [f"-DAFE_ORDER={n}"]) for n in (1, 2, 3)]
+    units += [("predictor_f64.cu", f"predictor_f64_{n}.o", [f"-DAFE_ORDER={n}"]) for n in (1, 2, 3)]
     for src, obj, flags in units:
         jobs.append([nvcc, *common, *ARCH, "-lineinfo", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
                      *flags, *extra, "-c", os.path.join(CSRC, src), "-o", os.path.join(objdir, obj)])

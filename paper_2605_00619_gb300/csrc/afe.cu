@@ -17,6 +17,7 @@
 #include "kernels.cuh"
 #include "predictor_cells.hpp"
 #include "predictor_f32.cuh"
+#include "predictor_f64.hpp"
 #include "refelem.hpp"
 #include "topology.hpp"
 
@@ -70,6 +71,8 @@ struct afe_mesh {
   afe::CorrRef cref{};   // ... and the face mass of its corrector
   afe::PcRef pref{};     // time-basis constants of the predictor with several cells per SM
   afe::PcPlan pc{};           // its plan for this mesh's cells (blocks = 0: not used)
+  afe::PdRef dref{};     // the same for the FP64 predictor with its product on the tensor cores
+  afe::PdPlan pd{};
   double* d_totals_partial = nullptr;
   double* d_totals = nullptr;
   int totals_blocks = 256;
@@ -128,18 +131,20 @@ struct StepPlan {
   afe::PcPlan pc;
   afe::PcRef pref{};
   afe::CorrRef cref{};
+  afe::PdPlan pd;
+  afe::PdRef dref{};
   int inviscid = 0, viscous = 0;  // cells without / with viscous fluxes may be present
   const afe::RefData* d_ref = nullptr;
   afe_mesh* single = nullptr;  // nullptr for a batch (FP32 shared-memory kernels only)
   afe_mesh* prof = nullptr;    // stage events are recorded on this mesh when profiling
 };
 
-// Adds the kinds of cells a mesh may hold: with mu or kappa every cell is viscous (in FP32, as
-// the predictor tests it), with the limiter any cell may be.
+// Adds the kinds of cells a mesh may hold: with mu or kappa every cell is viscous (in the
+// precision the predictor tests it in), with the limiter any cell may be.
 void add_kinds(StepPlan* P, const afe_mesh* m) {
   const afe::DevMesh& d = m->dm;
   const double kap = d.kappa0 >= 0.0 ? d.kappa0 : d.mu0 * d.gamma * d.cv / d.Pr;
-  const bool visc = (float)d.mu0 != 0.f || (float)kap != 0.f;
+  const bool visc = m->p.precision == AFE_FP32 ? (float)d.mu0 != 0.f || (float)kap != 0.f : d.mu0 != 0.0 || kap != 0.0;
   if (visc || m->p.limiter) P->viscous = 1;
   if (!visc) P->inviscid = 1;
   // a limiter may undo a viscosity below FP32's range: both kinds are possible
@@ -162,6 +167,8 @@ StepPlan plan_of(afe_mesh* m) {
   P.pc = m->pc;
   P.pref = m->pref;
   P.cref = m->cref;
+  P.pd = m->pd;
+  P.dref = m->dref;
   P.d_ref = m->d_ref;
   P.single = m;
   P.prof = m;
@@ -196,6 +203,12 @@ void launch_predictor(const StepPlan& P) {
       else
         afe::predictor_f32_kernel<N, false><<<P.n_sm, afe::kF32Threads, P.f32_smem, P.st>>>(*P.b, P.d_ref, P.diag,
                                                                                           (int)P.f32_smem);
+      return;
+    }
+  }
+  if constexpr (N <= 3) {
+    if (sizeof(Real) == 8 && P.pd.blocks) {
+      afe::pd_launch<N>(P.pd, *P.b, P.dref, P.inviscid, P.viscous, P.diag, P.n_sm, P.st);
       return;
     }
   }
@@ -333,7 +346,7 @@ afe_status record(const StepPlan& P) {
 // kernels per step: begin + [means + limiter] + (set_dt | cfl + finalize) + predictor (one for
 // each kind of cell) + face + corrector + clock
 int launches_per_step(const StepPlan& P, double dt) {
-  const int both = P.fp32 && P.pc.blocks && !P.f32_tc && P.inviscid && P.viscous;
+  const int both = (P.fp32 ? P.pc.blocks && !P.f32_tc : P.pd.blocks) && P.inviscid && P.viscous;
   return 1 + (P.limiter ? 2 : 0) + (dt > 0 ? 1 : 2) + 3 + both + 1;
 }
 
@@ -435,6 +448,48 @@ afe_status set_up_cells(afe_mesh* m, int64_t nminv) {
   afe::pc_set_up(m->dm, R.Np, R.Nf, (int)std::min<int64_t>(T.C, (int64_t)m->n_sm * 8), m->stream);
   AFE_CUDA(cudaGetLastError());
   m->pc = pc;
+  return AFE_OK;
+}
+
+// What the FP64 predictor of predictor_f64.cuh needs: the digits of M_i^-1 and the gather blocks.  A
+// handle whose cells do not fit its plan, or for which the device has no room left, keeps
+// predictor_kernel and its scratch.
+afe_status set_up_f64(afe_mesh* m, int64_t nminv) {
+  const afe::Topology& T = m->topo;
+  const afe::RefData& R = m->ref;
+  if (R.N > 3) return AFE_OK;
+  for (int s = 0; s < R.Nt; ++s) {
+    m->dref.w[s] = R.w[s];
+    for (int t = 0; t < R.Nt; ++t) {
+      m->dref.kw[s][t] = R.K1tinv[s][t] * R.w[t];
+      m->dref.kws[s] += R.K1tinv[s][t] * R.w[t];
+    }
+  }
+  afe::PdPlan pd;
+  switch (R.N) {
+    case 1: AFE_CUDA(afe::pd_plan<1>(m->device, T.Nmax, T.Smax, T.slots_max, &pd)); break;
+    case 2: AFE_CUDA(afe::pd_plan<2>(m->device, T.Nmax, T.Smax, T.slots_max, &pd)); break;
+    default: AFE_CUDA(afe::pd_plan<3>(m->device, T.Nmax, T.Smax, T.slots_max, &pd)); break;
+  }
+  if (!pd.blocks) return AFE_OK;
+  if (m->alloc(&m->dm.m16, 2 * (size_t)afe::pd_start(nminv, T.n_nodes, T.C)) != AFE_OK ||
+      m->alloc(&m->dm.gat, afe::pc_gather_bytes(m->dm, T.T, R.Np, R.Nf)) != AFE_OK) {
+    (void)cudaGetLastError();
+    return AFE_OK;
+  }
+  const int grid = (int)std::min<int64_t>(T.C, (int64_t)m->n_sm * 8);
+  afe::pd_set_up(m->dm, grid, m->stream);
+  afe::pc_gather_set_up(m->dm, R.Np, R.Nf, grid, m->stream);
+  AFE_CUDA(cudaGetLastError());
+  m->pd = pd;
+  for (size_t i = 0; i < m->allocs.size(); ++i)  // predictor_kernel's scratch is not needed then
+    if (m->allocs[i] == m->scratch) {
+      cudaFree(m->scratch);
+      m->allocs.erase(m->allocs.begin() + i);
+      m->bytes -= m->scratch_stride * m->pred_grid * 8;
+      m->scratch = nullptr;
+      break;
+    }
   return AFE_OK;
 }
 
@@ -712,6 +767,8 @@ afe_status afe_mesh_create(const afe_params* p, int64_t n_vertices, const double
         break;
       }
     if (M->f32_ok) AFE_TRY(set_up_cells(M, nminv));
+  } else {
+    AFE_TRY(set_up_f64(M, nminv));
   }
   sync_self(M);
   *out = m.release();

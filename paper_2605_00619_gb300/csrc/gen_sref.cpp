@@ -86,6 +86,75 @@ void emit_gradient(FILE* f, const afe::RefData& r) {
   std::fprintf(f, "  }\n");
 }
 
+// Entries of S^ that vanish in exact arithmetic are set to the zeros they are.
+void drop_zeros(afe::RefData* r) {
+  const int np = r->Np;
+  double smax = 0.0;
+  for (int d = 0; d < 3; ++d)
+    for (int m = 0; m < np; ++m)
+      for (int j = 0; j < np; ++j) smax = std::fmax(smax, std::fabs(r->S[d][m][j]));
+  for (int d = 0; d < 3; ++d)
+    for (int m = 0; m < np; ++m)
+      for (int j = 0; j < np; ++j)
+        if (std::fabs(r->S[d][m][j]) < 1e-13 * smax) r->S[d][m][j] = 0.0;
+}
+
+// The same contractions for the FP64 form: the entries sit in constant memory and reach the
+// multiply-adds as constant operands (immediates hold 32 bits).
+void emit_f64(FILE* f, const afe::RefData& r) {
+  const int np = r.Np;
+  double dmax = 0.0;
+  for (int d = 0; d < 3; ++d)
+    for (int j = 0; j < np; ++j)
+      for (int l = 0; l < np; ++l) dmax = std::fmax(dmax, std::fabs(r.D[d][j][l]));
+  auto put = [&](const char* name, bool transposed) {
+    std::vector<double> c;
+    std::string body;
+    char buf[160];
+    for (int kk = 0; kk < 3 * np; ++kk) {
+      std::snprintf(buf, sizeof buf, "    {\n      const double x = b[%d];\n", kk);
+      body += buf;
+      for (int m = 0; m < np; ++m) {
+        const double s = transposed ? r.S[kk / np][kk % np][m] : r.S[kk / np][m][kk % np];
+        if (s == 0.0) continue;
+        std::snprintf(buf, sizeof buf, "      acc[%d] = fma(k%s%d[%d], x, acc[%d]);\n", m, name, r.N, (int)c.size(), m);
+        body += buf;
+        c.push_back(s);
+      }
+      body += "    }\n";
+    }
+    std::fprintf(f, "static __device__ __constant__ double k%s%d[%d] = {", name, r.N, (int)c.size());
+    for (size_t i = 0; i < c.size(); ++i) std::fprintf(f, "%s%a", i ? ", " : "", c[i]);
+    std::fprintf(f, "};\n");
+    return body;
+  };
+  const std::string a = put("Contract", false), t = put("ContractT", true);
+  std::vector<double> c;
+  std::string g;
+  char buf[160];
+  for (int d = 0; d < 3; ++d) {
+    g += "    for (int j = 0; j < " + std::to_string(np) + "; ++j) a[j] = 0.0;\n";
+    for (int l = 0; l < np; ++l)
+      for (int j = 0; j < np; ++j) {
+        if (std::fabs(r.D[d][j][l]) < 1e-13 * dmax) continue;
+        std::snprintf(buf, sizeof buf, "    a[%d] = fma(kGradient%d[%d], x[%d], a[%d]);\n", j, r.N, (int)c.size(), l, j);
+        g += buf;
+        c.push_back(r.D[d][j][l]);
+      }
+    for (int j = 0; j < np; ++j) {
+      std::snprintf(buf, sizeof buf, "    out[%d] = a[%d];\n", d * np + j, j);
+      g += buf;
+    }
+  }
+  std::fprintf(f, "static __device__ __constant__ double kGradient%d[%d] = {", r.N, (int)c.size());
+  for (size_t i = 0; i < c.size(); ++i) std::fprintf(f, "%s%a", i ? ", " : "", c[i]);
+  std::fprintf(f, "};\n");
+  std::fprintf(f, "template <>\nstruct SrefFP64<%d> {\n", r.N);
+  std::fprintf(f, "  static __device__ __forceinline__ void contract(const double* b, double (&acc)[%d]) {\n%s  }\n", np, a.c_str());
+  std::fprintf(f, "  static __device__ __forceinline__ void contract_t(const double* b, double (&acc)[%d]) {\n%s  }\n", np, t.c_str());
+  std::fprintf(f, "  static __device__ __forceinline__ void gradient(const double (&x)[%d], double* out) {\n    double a[%d];\n%s  }\n};\n\n", np, np, g.c_str());
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -103,6 +172,7 @@ int main(int argc, char** argv) {
                "// reference-stiffness contractions with S^ as immediates.  Do not edit.\n"
                "#pragma once\n\nnamespace afe {\n\n"
                "template <int N>\nstruct SrefFP32;\n\n");
+  // the FP64 contractions follow in a section of their own, for the translation units that ask
   for (int N = 1; N <= 3; ++N) {
     static afe::RefData r;
     if (!afe::build_ref(N, &r)) {
@@ -110,14 +180,7 @@ int main(int argc, char** argv) {
       return 1;
     }
     const int np = r.Np, kk_n = 3 * np;
-    double smax = 0.0;
-    for (int d = 0; d < 3; ++d)
-      for (int m = 0; m < np; ++m)
-        for (int j = 0; j < np; ++j) smax = std::fmax(smax, std::fabs(r.S[d][m][j]));
-    for (int d = 0; d < 3; ++d)
-      for (int m = 0; m < np; ++m)
-        for (int j = 0; j < np; ++j)
-          if (std::fabs(r.S[d][m][j]) < 1e-13 * smax) r.S[d][m][j] = 0.0;
+    drop_zeros(&r);
     int nz_p = 0, nz_v = 0;
     for (int d = 0; d < 3; ++d)
       for (int m = 0; m < np; ++m)
@@ -149,6 +212,14 @@ int main(int argc, char** argv) {
     emit_gradient(f, r);
     std::fprintf(f, "};\n\n");
   }
+  std::fprintf(f, "#ifdef AFE_SREF_F64\ntemplate <int N>\nstruct SrefFP64;\n\n");
+  for (int N = 1; N <= 3; ++N) {
+    static afe::RefData r;
+    if (!afe::build_ref(N, &r)) return 1;
+    drop_zeros(&r);
+    emit_f64(f, r);
+  }
+  std::fprintf(f, "#endif\n\n");
   std::fprintf(f, "}  // namespace afe\n");
   std::fclose(f);
   return 0;

@@ -206,6 +206,10 @@ size_t pc_gather_bytes(const DevMesh& m, int64_t n_subtets, int np, int nf) {
 
 void pc_set_up(const DevMesh& m, int np, int nf, int grid, cudaStream_t st) {
   split_minv_kernel<<<grid, 256, 0, st>>>(m);
+  pc_gather_set_up(m, np, nf, grid, st);
+}
+
+void pc_gather_set_up(const DevMesh& m, int np, int nf, int grid, cudaStream_t st) {
   gather_lists_kernel<<<grid, 256, 0, st>>>(m, np, nf);
 }
 #endif

@@ -44,8 +44,9 @@ void pc_launch(const PcPlan& plan, const Batch& b, const PcRef& ref, bool invisc
 template <int N>
 void pc_correct(const Batch& b, const CorrRef& ref, int Nmax, int Fmax, cudaStream_t st);
 
-// Bytes of the gather blocks of a mesh, and the set-up of m.m16 and m.gat.
+// Bytes of the gather blocks of a mesh, and the set-up of m.m16 and m.gat (of m.gat alone).
 size_t pc_gather_bytes(const DevMesh& m, int64_t n_subtets, int np, int nf);
 void pc_set_up(const DevMesh& m, int np, int nf, int grid, cudaStream_t st);
+void pc_gather_set_up(const DevMesh& m, int np, int nf, int grid, cudaStream_t st);
 
 }  // namespace afe
