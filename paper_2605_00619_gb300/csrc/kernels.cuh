@@ -596,7 +596,21 @@ __global__ void __launch_bounds__(256) predictor_kernel(DevMesh m, const RefData
   __shared__ Real sW[NT];
   __shared__ double sred[64];
   __shared__ int64_t sCell;
+  // FP32 at N = 4: the stiffness with its rows innermost, and a tile of right-hand-side rows, both read as
+  // vectors (what the scalar loads of the general form are bound by; us per launch at 8^3: 11,770
+  // without, 6,680 with both)
+  constexpr bool kTiled = N == 4 && sizeof(Real) == 4;
+  constexpr int MP = (NP + 3) / 4 * 4, CP = (NT * 5 + 3) / 4 * 4, LT = 32;
+  __shared__ __align__(16) float sST[kTiled ? 3 * NP : 1][MP];
+  __shared__ __align__(16) float sRT[kTiled ? LT : 1][CP];
   const int tid = threadIdx.x, nthr = blockDim.x;
+  if constexpr (kTiled) {
+    for (int e = tid; e < 3 * NP * MP; e += nthr) {
+      const int kk = e / MP, r = e % MP;
+      sST[kk][r] = r < NP ? (float)ref->S[kk / NP][r][kk % NP] : 0.f;
+    }
+    for (int e = tid; e < LT * CP; e += nthr) sRT[e / CP][e % CP] = 0.f;
+  }
   for (int e = tid; e < 3 * NP * NP; e += nthr) {
     const int d = e / (NP * NP), r = (e / NP) % NP, q = e % NP;
     sS[d][r][q] = (Real)ref->S[d][r][q];
@@ -701,7 +715,27 @@ __global__ void __launch_bounds__(256) predictor_kernel(DevMesh m, const RefData
       }
       __syncthreads();
       // B: R[k][t][m][v] = w_t sum_d sum_j S[d][m][j] B[k][t][d][j][v]
-      for (int e = tid; e < S * NT * NP * 5; e += nthr) {
+      if constexpr (kTiled) {  // a column (k, t, v) per thread, all rows m in registers
+        for (int e = tid; e < S * NT * 5; e += nthr) {
+          const int kt = e / 5, v = e % 5;
+          const Real* src = Bf + (int64_t)kt * 3 * NP * 5 + v;
+          float acc[MP];
+#pragma unroll
+          for (int i = 0; i < MP; ++i) acc[i] = 0.f;
+#pragma unroll 3
+          for (int kk = 0; kk < 3 * NP; ++kk) {
+            const float x = src[kk * 5];
+#pragma unroll
+            for (int i = 0; i < MP; i += 4) {
+              const float4 c = *reinterpret_cast<const float4*>(&sST[kk][i]);
+              acc[i] += c.x * x, acc[i + 1] += c.y * x, acc[i + 2] += c.z * x, acc[i + 3] += c.w * x;
+            }
+          }
+          const float wt = sW[kt % NT];
+#pragma unroll
+          for (int i = 0; i < NP; ++i) Rb[((int64_t)kt * NP + i) * 5 + v] = wt * acc[i];
+        }
+      } else for (int e = tid; e < S * NT * NP * 5; e += nthr) {
         const int k = e / (NT * NP * 5), t = (e / (NP * 5)) % NT, mm = (e / 5) % NP, v = e % 5;
         const Real* src = Bf + ((int64_t)(k * NT + t) * 3) * NP * 5 + v;
         Real acc = 0;
@@ -725,7 +759,49 @@ __global__ void __launch_bounds__(256) predictor_kernel(DevMesh m, const RefData
       }
       __syncthreads();
       // D: Y = M_i^-1 RHS (M_i^-1 symmetric: row n read as column n, coalesced)
-      for (int n = tid; n < Ni; n += nthr) {
+      if constexpr (kTiled) {  // four nodes per thread against tiles of 32 right-hand-side rows
+        const int LD = minv_ld(Ni);
+        for (int g0 = 0; 4 * g0 < Ni; g0 += nthr) {
+          const int g = g0 + tid;
+          float acc[4][NT * 5];
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int c2 = 0; c2 < NT * 5; ++c2) acc[i][c2] = 0.f;
+          for (int l0 = 0; l0 < Ni; l0 += LT) {
+            __syncthreads();
+            for (int e = tid; e < LT * NT * 5; e += nthr) {
+              const int l = e / (NT * 5);
+              sRT[l][e - l * NT * 5] = l0 + l < Ni ? RHS[l0 * NT * 5 + e] : 0.f;
+            }
+            __syncthreads();
+            if (4 * g >= Ni) continue;
+            const float* col = (const float*)minv + 4 * g;
+#pragma unroll 2
+            for (int l = 0; l < min(LT, Ni - l0); ++l) {
+              const float4 a = *reinterpret_cast<const float4*>(col + (int64_t)(l0 + l) * LD);
+#pragma unroll
+              for (int q = 0; q < CP; q += 4) {
+                const float4 r = *reinterpret_cast<const float4*>(&sRT[l][q]);
+                const float rv[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                  if (q + u < NT * 5) {
+                    acc[0][q + u] += a.x * rv[u];
+                    acc[1][q + u] += a.y * rv[u];
+                    acc[2][q + u] += a.z * rv[u];
+                    acc[3][q + u] += a.w * rv[u];
+                  }
+              }
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (4 * g + i < Ni)
+#pragma unroll
+              for (int c2 = 0; c2 < NT * 5; ++c2) Y[(4 * g + i) * NT * 5 + c2] = acc[i][c2];
+        }
+      } else for (int n = tid; n < Ni; n += nthr) {
         Real acc[NT * 5];
 #pragma unroll
         for (int c2 = 0; c2 < NT * 5; ++c2) acc[c2] = 0;
