@@ -472,6 +472,13 @@ afe_status set_up_f64(afe_mesh* m, int64_t nminv) {
     default: AFE_CUDA(afe::pd_plan<3>(m->device, T.Nmax, T.Smax, T.slots_max, &pd)); break;
   }
   if (!pd.blocks) return AFE_OK;
+  std::vector<uint32_t> table(2 * afe::pd_stiffness_words(R.N));
+  m->dref.sexp = afe::pd_stiffness_digits(R, false, table.data());
+  (void)afe::pd_stiffness_digits(R, true, table.data() + table.size() / 2);
+  uint32_t* dtab = nullptr;
+  AFE_TRY(m->upload(&dtab, table));
+  m->dref.sdig = dtab;
+  m->dref.sdig_t = dtab + table.size() / 2;
   if (m->alloc(&m->dm.m16, 2 * (size_t)afe::pd_start(nminv, T.n_nodes, T.C)) != AFE_OK ||
       m->alloc(&m->dm.gat, afe::pc_gather_bytes(m->dm, T.T, R.Np, R.Nf)) != AFE_OK) {
     (void)cudaGetLastError();

@@ -99,7 +99,7 @@ void drop_zeros(afe::RefData* r) {
         if (std::fabs(r->S[d][m][j]) < 1e-13 * smax) r->S[d][m][j] = 0.0;
 }
 
-// The same contractions for the FP64 form: the entries sit in constant memory and reach the
+// The reference gradient (and S^ at N = 1) for the FP64 form: the entries sit in constant memory and reach the
 // multiply-adds as constant operands (immediates hold 32 bits).
 void emit_f64(FILE* f, const afe::RefData& r) {
   const int np = r.Np;
@@ -107,28 +107,23 @@ void emit_f64(FILE* f, const afe::RefData& r) {
   for (int d = 0; d < 3; ++d)
     for (int j = 0; j < np; ++j)
       for (int l = 0; l < np; ++l) dmax = std::fmax(dmax, std::fabs(r.D[d][j][l]));
-  auto put = [&](const char* name, bool transposed) {
-    std::vector<double> c;
-    std::string body;
-    char buf[160];
-    for (int kk = 0; kk < 3 * np; ++kk) {
-      std::snprintf(buf, sizeof buf, "    {\n      const double x = b[%d];\n", kk);
-      body += buf;
+  // S^ itself at N = 1 only (above, the FP64 form's contraction runs on the tensor cores)
+  std::string contract[2];
+  for (int tr = 0; tr < 2 && r.N == 1; ++tr) {
+    std::vector<double> k;
+    char line[160];
+    for (int kk = 0; kk < 3 * np; ++kk)
       for (int m = 0; m < np; ++m) {
-        const double s = transposed ? r.S[kk / np][kk % np][m] : r.S[kk / np][m][kk % np];
-        if (s == 0.0) continue;
-        std::snprintf(buf, sizeof buf, "      acc[%d] = fma(k%s%d[%d], x, acc[%d]);\n", m, name, r.N, (int)c.size(), m);
-        body += buf;
-        c.push_back(s);
+        const double v = tr ? r.S[kk / np][kk % np][m] : r.S[kk / np][m][kk % np];
+        if (v == 0.0) continue;
+        std::snprintf(line, sizeof line, "    acc[%d] = fma(kStiffness%d[%d], b[%d], acc[%d]);\n", m, tr, (int)k.size(), kk, m);
+        contract[tr] += line;
+        k.push_back(v);
       }
-      body += "    }\n";
-    }
-    std::fprintf(f, "static __device__ __constant__ double k%s%d[%d] = {", name, r.N, (int)c.size());
-    for (size_t i = 0; i < c.size(); ++i) std::fprintf(f, "%s%a", i ? ", " : "", c[i]);
+    std::fprintf(f, "static __device__ __constant__ double kStiffness%d[%d] = {", tr, (int)k.size());
+    for (size_t i = 0; i < k.size(); ++i) std::fprintf(f, "%s%a", i ? ", " : "", k[i]);
     std::fprintf(f, "};\n");
-    return body;
-  };
-  const std::string a = put("Contract", false), t = put("ContractT", true);
+  }
   std::vector<double> c;
   std::string g;
   char buf[160];
@@ -150,8 +145,10 @@ void emit_f64(FILE* f, const afe::RefData& r) {
   for (size_t i = 0; i < c.size(); ++i) std::fprintf(f, "%s%a", i ? ", " : "", c[i]);
   std::fprintf(f, "};\n");
   std::fprintf(f, "template <>\nstruct SrefFP64<%d> {\n", r.N);
-  std::fprintf(f, "  static __device__ __forceinline__ void contract(const double* b, double (&acc)[%d]) {\n%s  }\n", np, a.c_str());
-  std::fprintf(f, "  static __device__ __forceinline__ void contract_t(const double* b, double (&acc)[%d]) {\n%s  }\n", np, t.c_str());
+  if (r.N == 1)
+    for (int tr = 0; tr < 2; ++tr)
+      std::fprintf(f, "  static __device__ __forceinline__ void %s(const double* b, double (&acc)[%d]) {\n%s  }\n",
+                   tr ? "contract_t" : "contract", np, contract[tr].c_str());
   std::fprintf(f, "  static __device__ __forceinline__ void gradient(const double (&x)[%d], double* out) {\n    double a[%d];\n%s  }\n};\n\n", np, np, g.c_str());
 }
 
@@ -172,7 +169,7 @@ int main(int argc, char** argv) {
                "// reference-stiffness contractions with S^ as immediates.  Do not edit.\n"
                "#pragma once\n\nnamespace afe {\n\n"
                "template <int N>\nstruct SrefFP32;\n\n");
-  // the FP64 contractions follow in a section of their own, for the translation units that ask
+  // the FP64 gradients follow in a section of their own, for the translation units that ask
   for (int N = 1; N <= 3; ++N) {
     static afe::RefData r;
     if (!afe::build_ref(N, &r)) {

@@ -3,6 +3,7 @@
 #include "predictor_f64.cuh"
 
 #include <algorithm>
+#include <cmath>
 
 namespace afe {
 namespace {
@@ -93,6 +94,34 @@ static __global__ void __launch_bounds__(256) digits_kernel(DevMesh m) {
     }
     __syncthreads();
   }
+}
+
+int pd_stiffness_words(int N) { return (np_of(N) + 15) / 16 * ((3 * np_of(N) + 15) / 16) * 512; }
+
+int pd_stiffness_digits(const RefData& r, bool transposed, uint32_t* out) {
+  const int np = r.Np, kst = (3 * np + 15) / 16, mts = (np + 15) / 16;
+  double smax = 0.0;
+  for (int d = 0; d < 3; ++d)
+    for (int m = 0; m < np; ++m)
+      for (int j = 0; j < np; ++j) smax = std::max(smax, std::fabs(r.S[d][m][j]));
+  int e = 0;
+  (void)std::frexp(smax, &e);
+  for (int mt = 0; mt < mts; ++mt)
+    for (int ks = 0; ks < kst; ++ks)
+      for (int lane = 0; lane < 32; ++lane)
+        for (int half = 0; half < 2; ++half)
+          for (int s = 0; s < 8; ++s) {
+            uint32_t v = 0;
+            for (int i = 0; i < 4; ++i) {
+              const int row = 16 * mt + (lane >> 2) + 8 * (i >> 1), kk = 16 * ks + 2 * (lane & 3) + 8 * half + (i & 1);
+              double x = 0.0;
+              if (row < np && kk < 3 * np) x = transposed ? r.S[kk / np][kk % np][row] : r.S[kk / np][row][kk % np];
+              if (std::fabs(x) < 1e-13 * smax) x = 0.0;  // zeros of the exact matrix
+              v |= (uint32_t)(digits(x, e) >> (56 - 8 * s) & 255u) << (8 * i);
+            }
+            out[(size_t)(mt * kst + ks) * 512 + (s >> 1) * 128 + lane * 4 + (s & 1) * 2 + half] = v;
+          }
+  return e;
 }
 
 void pd_set_up(const DevMesh& m, int grid, cudaStream_t st) { digits_kernel<<<grid, 256, 0, st>>>(m); }

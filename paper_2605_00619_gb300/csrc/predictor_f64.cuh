@@ -15,17 +15,21 @@
 //     instructions (77 cycles) replace 64 warp FMAs (1,088 cycles) per 16 x 16 x 8 block.
 //   - The first iteration starts from q^0 = u^ at every time node: one time slice serves all.
 //   - The flux goes straight to its contravariant form (half the arithmetic), with one
-//     reciprocal refined by Newton steps; entries of the stiffness that vanish are skipped.
+//     reciprocal refined by Newton steps.
+//   - The stiffness contractions are digit products too, with the digits of S^ from a table.
 // Error of the product against 64 bits on random rows of 320 entries: 1e-18 to 2e-16 of the sum of
 // magnitudes, FP64 summation 6e-18 to 8e-16; of the whole step the same as before (3.3e-16 at 8^3 P3).
-// us per launch, predictor_kernel and here: 8^3 P3 31,240 and 11,430, 10^3 P2 12,740 and 5,650, 6^3 P1 984 and
-// 456.  What bounds it now: the stiffness contraction's FP64 multiply-adds (65 % of the FP64
-// instructions at N = 3), at P1 the latency of an iteration's eight barriers.
+// us per launch, predictor_kernel and here: 8^3 P3 31,240 and 7,865 (11,430 with the contraction in FP64),
+// 10^3 P2 12,740 and 5,390 (5,650), 6^3 P1 984 and 450.  What bounds it now, per cell-iteration at P3: the
+// digit products' tensor instructions (160 k of 545 k cycles) and the integer work around them, the
+// fluxes' FP64 instructions (100 k); at P2 the fluxes; at P1 the latency of an iteration's barriers.
 // One block per cell, persistent; the cell's q, u^ and lists in shared memory; data flow, lists
 // and gather order as in predictor_cells.cuh.
 #pragma once
 
 #include <cuda_fp16.h>
+
+#include <cstring>
 
 #define AFE_SREF_F64 1
 #include "predictor_cells.cuh"
@@ -38,6 +42,10 @@ struct Pd {
   static constexpr int NP = np_of(N), NT = N + 1, NF = nf_of(N), NTP = f32_ntp(N);
   static constexpr int SQ = 5 * NT;              // doubles of q per node, time innermost
   static constexpr int KKS = (3 * NP) | 1;       // column of pre-contracted fluxes (odd: conflict-free)
+  static constexpr int KST = (3 * NP + 15) / 16;  // its 16-row steps
+  static constexpr int MT = (NP + 15) / 16;       // 16-row tiles of its contraction's result
+  // bytes of a chunk per column: FP64 values, and their digits (1 KB per eight columns and step)
+  static constexpr int CB = KKS * 8 + (N == 1 ? 0 : KST * 128);  // (P1 contracts in FP64)
   static constexpr int NNT = N == 1 ? 2 : 3;     // 8-column tiles of RHS / Y: column v NTP + t
   // bytes of the digit fragments per 16 rows: 32 per lane in use of every column tile
   static constexpr int FB = 20 * NTP * 32, FB1 = 20 * 32;
@@ -55,6 +63,7 @@ struct PdShared {
   int ired[5][16];
   long long red[2][16];
   PdRef ref;
+  double dkw[4][4], dkws[4];  // dt times the time-basis constants
 };
 constexpr int kPdNone = 20000;  // exponent of a variable with an infinite or NaN entry
 constexpr int kPdGat = (int)((sizeof(PdShared) + 127) / 128 * 128);  // the gather block follows
@@ -73,7 +82,7 @@ template <int N>
 __host__ __device__ constexpr size_t pd_need(int n, int s, int ns, int thr) {
   // the fragments beside the sums past the second slot; two sub-tets beside all sums
   const size_t frag = (size_t)((n + 15) / 16) * Pd<N>::FB + pd_over<N>(pc_slots(n, thr), 2 * thr);
-  const size_t chunk = (size_t)2 * 5 * Pd<N>::NT * Pd<N>::KKS * 8 + pd_over<N>(pc_slots(n, thr), thr);
+  const size_t chunk = (size_t)(2 * 5 * Pd<N>::NT + 8) * (Pd<N>::CB + 4) + pd_over<N>(pc_slots(n, thr), thr);
   return pd_fixed<N>(n, s, ns) + (frag > chunk ? frag : chunk);
 }
 
@@ -88,12 +97,17 @@ __device__ __forceinline__ double recip(double x) {
 
 // x 2^(62 - e) to nearest as a 64-bit integer plus 128 in every byte, for |x| < 2^e: the bytes are the
 // balanced base-256 digits plus 128.
-__device__ __forceinline__ unsigned long long digits(double x, int e) {
+__host__ __device__ __forceinline__ unsigned long long digits(double x, int e) {
+#ifdef __CUDA_ARCH__
   const long long b = __double_as_longlong(x);
+#else
+  long long b;
+  std::memcpy(&b, &x, 8);
+#endif
   const int ex = (int)(b >> 52) & 0x7ff;
   unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | (ex ? 1ull << 52 : 0ull);
   const int sh = (ex ? ex : 1) - 1075 + 62 - e;  // value = m 2^(ex - 1075)
-  if (sh >= 0) m <<= min(sh, 10);
+  if (sh >= 0) m <<= sh < 10 ? sh : 10;
   else if (sh > -63) m = (m + (1ull << (-sh - 1))) >> -sh;
   else m = 0;
   const long long v = b < 0 ? -(long long)m : (long long)m;
@@ -105,8 +119,70 @@ __device__ __forceinline__ uint32_t digit_pair(uint32_t w, uint32_t sel) {
   const __half2 r = __hsub2(*reinterpret_cast<const __half2*>(&h), __half2half2(__ushort_as_half(0x6480)));  // 1152
   return *reinterpret_cast<const uint32_t*>(&r);
 }
-// 2^k for |k| < 1022
-__device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
+// The exact product of digit tiles: a 16 x (16 steps) row of tiles at `at` (16-byte groups of this
+// lane, 512 words per step) with an 8-column operand at `bt` (this lane's 32 bytes, `stride` bytes per
+// step; the digit zero where !on).  The product is hi 2^32 + lo, times 2^56 of the factors' units.
+__device__ __forceinline__ void digit_product(const uint32_t* at, const unsigned char* bt, int stride, bool on, int steps,
+                                              long long (&hi)[4], long long (&lo)[4]) {
+  uint4 nx[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) nx[q] = ldg_stream(at + q * 128);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) hi[i] = lo[i] = 0;
+  for (int k0 = 0; k0 < steps; k0 += 7) {  // 112 columns: what the FP32 accumulators hold exactly
+    float acc[8][4];
+#pragma unroll
+    for (int l = 0; l < 8; ++l)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[l][i] = 0.f;
+    const int k1 = min(k0 + 7, steps);
+#pragma unroll 1
+    for (int ks = k0; ks < k1; ++ks) {
+      uint4 A[8];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t w[4] = {nx[q].x, nx[q].y, nx[q].z, nx[q].w};
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+          A[2 * q + s] = make_uint4(digit_pair(w[2 * s], 0x4140), digit_pair(w[2 * s], 0x4342),
+                                    digit_pair(w[2 * s + 1], 0x4140), digit_pair(w[2 * s + 1], 0x4342));
+      }
+      const uint32_t* t = at + (size_t)min(ks + 1, steps - 1) * 512;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) nx[q] = ldg_stream(t + q * 128);
+      const uint4 z4 = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
+      const uint4 b0 = on ? *reinterpret_cast<const uint4*>(bt + ks * stride) : z4;
+      const uint4 b1 = on ? *reinterpret_cast<const uint4*>(bt + ks * stride + 16) : z4;
+      const uint32_t b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const uint32_t c0 = digit_pair(b[u], 0x4140), c1 = digit_pair(b[u], 0x4342);
+#pragma unroll
+        for (int s = 0; s + u < 8; ++s) mma_f16(acc[s + u], A[s], c0, c1);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      int a[8];
+#pragma unroll
+      for (int l = 0; l < 8; ++l) a[l] = __float2int_rn(acc[l][i]);
+      hi[i] += ((long long)a[0] << 24) + ((long long)a[1] << 16) + ((long long)a[2] << 8) + a[3];
+      lo[i] += ((long long)a[4] << 24) + ((long long)a[5] << 16) + ((long long)a[6] << 8) + a[7];
+    }
+  }
+}
+// (hi 2^32 + lo) 2^k, rounded once, for |hi|, |lo| < 2^51; none: a factor was infinite or NaN.  The integers
+// enter as the last bits of 1.5 2^52 + integer, because the conversion instructions go through
+// the FP64 pipe too.
+__device__ __forceinline__ double digit_value(long long hi, long long lo, int k, bool none) {
+  const double h = fma(__longlong_as_double(hi + 0x4338000000000000ll), 0x1p32, -0x1.8p84);  // hi 2^32, exact
+  const double s = h + (__longlong_as_double(lo + 0x4338000000000000ll) - 0x1.8p52);
+  if (none) return __hiloint2double(0x7ff80000, 0);
+  if ((unsigned)(k + 900) <= 1800u) return s * __hiloint2double((1023 + k) << 20, 0);
+  k = max(-2000, min(2000, k));
+  const int k2 = k / 2;
+  return s * __hiloint2double((1023 + k2) << 20, 0) * __hiloint2double((1023 + k - k2) << 20, 0);
+}
 
 __device__ __forceinline__ void contravariant_flux(const double (&Q)[5], const double (&g)[9], double gm1,
                                                    double out[3][5]) {
@@ -181,6 +257,120 @@ __device__ __forceinline__ void contract_adj(const double (&g)[9], double scale,
       out[d][v] = scale * (g[d * 3] * F[0][v] + g[d * 3 + 1] * F[1][v] + g[d * 3 + 2] * F[2][v]);
 }
 
+// Contraction of `cols` columns (`cstride` doubles apart) with S^ or its transpose, in place:
+// four lanes per column find its power of two and write its digits as fragments behind the columns
+// and their exponents behind those, then (row tile, 8 columns) pairs go over the warps.  A column's
+// 882 FP64 multiply-adds at N = 3 would take 15 k cycles per warp of columns, this 2.5 k.
+template <int N, int W>
+__device__ __forceinline__ void pd_contract(const PdRef& ref, bool transposed, int cols, int cstride) {
+  using P = Pd<N>;
+  constexpr int NP = P::NP, KK = 3 * NP, KST = P::KST, THR = 32 * W, QN = KST * 4;  // values per lane
+  double* const col0 = PdView<N>().region;
+  if constexpr (N == 1) {  // 12 values per column: 36 multiply-adds are less than the digits' own work
+    for (int c = threadIdx.x; c < cols; c += THR) {
+      double acc[NP];
+#pragma unroll
+      for (int i = 0; i < NP; ++i) acc[i] = 0.0;
+      double* b = col0 + (size_t)c * cstride;
+      if (transposed) SrefFP64<N>::contract_t(b, acc);
+      else SrefFP64<N>::contract(b, acc);
+      asm volatile("" ::: "memory");  // the results replace the column
+#pragma unroll
+      for (int i = 0; i < NP; ++i) b[i] = acc[i];
+    }
+    return;
+  }
+  unsigned char* const dig = reinterpret_cast<unsigned char*>(col0) + pc_up((size_t)cols * cstride * 8);
+  const int tiles = (cols + 7) / 8;
+  int* const dex = reinterpret_cast<int*>(dig + (size_t)tiles * KST * 1024);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // digits: lane quarter u of a column takes rows 16 ks + 2 u, + 1, + 8, + 9 of every step, the two 16-bit
+  // halves of a fragment word
+  for (int e = tid; e < tiles * 32; e += THR) {
+    const int c = e >> 2, u = e & 3;
+    const double* b = col0 + (size_t)c * cstride;
+    double val[QN];
+    int ex = 1;
+#pragma unroll
+    for (int q = 0; q < QN; ++q) {
+      const int kk = (q >> 2) * 16 + 2 * u + (q & 1) + 8 * ((q >> 1) & 1);
+      val[q] = c < cols && kk < KK ? b[kk] : 0.0;
+      ex = max(ex, __double2hiint(val[q]) >> 20 & 0x7ff);
+    }
+    ex = max(ex, __shfl_xor_sync(0xffffffffu, ex, 1));
+    ex = max(ex, __shfl_xor_sync(0xffffffffu, ex, 2));
+    if (u == 0) dex[c] = ex == 0x7ff ? kPdNone : ex - 1022;
+#pragma unroll
+    for (int ks = 0; ks < KST; ++ks) {
+      unsigned long long d[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) d[i] = digits(val[ks * 4 + i], ex - 1022);
+      uint32_t w[8];
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        w[s] = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[s] |= (uint32_t)(d[i] >> (56 - 8 * s) & 255u) << (8 * i);
+      }
+      uint4* o = reinterpret_cast<uint4*>(dig + ((size_t)(c >> 3) * KST + ks) * 1024 + ((c & 7) * 4 + u) * 32);
+      o[0] = make_uint4(w[0], w[1], w[2], w[3]);
+      o[1] = make_uint4(w[4], w[5], w[6], w[7]);
+    }
+  }
+  __syncthreads();
+  for (int job = warp; job < tiles * P::MT; job += W) {
+    const int ct = job / P::MT, mt = job - ct * P::MT;
+    long long hi[4], lo[4];
+    digit_product((transposed ? ref.sdig_t : ref.sdig) + (size_t)mt * KST * 512 + lane * 4, dig + (size_t)ct * KST * 1024 + lane * 32, 1024, true, KST, hi, lo);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int c = ct * 8 + 2 * (lane & 3) + (i & 1), row = mt * 16 + (lane >> 2) + 8 * (i >> 1);
+      if (c < cols && row < NP) {
+        const int ec = dex[c];
+        col0[(size_t)c * cstride + row] = digit_value(hi[i], lo[i], 56 - 124 + ref.sexp + ec, ec >= kPdNone);
+      }
+    }
+  }
+}
+
+// Sums of V values over the lanes of a warp, in a fixed order, to lane 0: every step halves the values
+// a lane holds (V - 1 + a few additions per lane instead of 5 V), then the lanes hand theirs over.
+template <int V>
+__device__ __forceinline__ void lane_sums(double* r, int lane) {
+  double d[V + 1];
+#pragma unroll
+  for (int i = 0; i < V; ++i) d[i] = r[i];
+  d[V] = 0.0;
+  constexpr int n1 = (V + 1) / 2, n2 = (n1 + 1) / 2, n3 = (n2 + 1) / 2, n4 = (n3 + 1) / 2, n5 = (n4 + 1) / 2;
+  static_assert(n5 == 1, "up to 32 values");
+  auto fold = [&](auto have, auto half, int o) {
+    constexpr int n = decltype(have)::value, h = decltype(half)::value;
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const double hi = i + h < n ? d[i + h] : 0.0;
+      const double send = up ? d[i] : hi, keep = up ? hi : d[i];
+      d[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  };
+  fold(std::integral_constant<int, V>{}, std::integral_constant<int, n1>{}, 16);
+  fold(std::integral_constant<int, n1>{}, std::integral_constant<int, n2>{}, 8);
+  fold(std::integral_constant<int, n2>{}, std::integral_constant<int, n3>{}, 4);
+  fold(std::integral_constant<int, n3>{}, std::integral_constant<int, n4>{}, 2);
+  if constexpr (n4 > 1) fold(std::integral_constant<int, n4>{}, std::integral_constant<int, n5>{}, 1);
+  else d[0] += __shfl_xor_sync(0xffffffffu, d[0], 1);
+#pragma unroll
+  for (int i = 0; i < V; ++i) {  // value i sits in the lane its halves lead to
+    int k = i, src = 0;
+    if (k >= n1) k -= n1, src |= 16;
+    if (k >= n2) k -= n2, src |= 8;
+    if (k >= n3) k -= n3, src |= 4;
+    if (k >= n4) k -= n4, src |= 2;
+    if (k >= n5) k -= n5, src |= 1;
+    r[i] = __shfl_sync(0xffffffffu, d[0], src);
+  }
+}
+
 // ---- 1. Right-hand side, left in the region as digit fragments.
 template <int N, int W, bool VISC>
 __device__ __forceinline__ void pd_rhs(bool first) {
@@ -192,7 +382,8 @@ __device__ __forceinline__ void pd_rhs(bool first) {
   const int S = x.S, over = max(x.slots - THR, 0);
   double* const sover = V.region + x.room / 8 - over * SQ;
   const int nte = first ? 1 : NT;
-  const int cap = (x.room - over * SQ * 8) / (5 * nte * KKS * 8);
+  // (the columns' tiles of eight and their exponents take part of a tile more)
+  const int cap = (x.room - over * SQ * 8 - 8 * P::CB) / (5 * nte * (P::CB + 4));
   const int nch = (S + cap - 1) / cap, CH = (S + nch - 1) / nch;
   double racc[5][NT];
   int cur, cend, cstep;
@@ -234,16 +425,7 @@ __device__ __forceinline__ void pd_rhs(bool first) {
         for (int d = 0; d < 3; ++d) dst[v * vs + d * NP] = out[d][v];
     }
     __syncthreads();
-    for (int col = tid; col < nk * 5 * nte; col += THR) {
-      double acc[NP];
-#pragma unroll
-      for (int i = 0; i < NP; ++i) acc[i] = 0.0;
-      double* b = V.region + col * KKS;
-      SrefFP64<N>::contract(b, acc);
-      asm volatile("" ::: "memory");  // the results replace the column
-#pragma unroll
-      for (int i = 0; i < NP; ++i) b[i] = acc[i];
-    }
+    pd_contract<N, W>(x.ref, false, nk * 5 * nte, KKS);
     __syncthreads();
     auto gather = [&](int& c1, int end, int step, double (&acc)[5][NT]) {
       const int lim = (kc + nk) << 6;
@@ -275,16 +457,7 @@ __device__ __forceinline__ void pd_rhs(bool first) {
     }
     if (kc + CH < S) __syncthreads();
   }
-  if (warp < x.nlong) {  // the lanes' shares of a long list, in a fixed order
-#pragma unroll
-    for (int v = 0; v < 5; ++v)
-#pragma unroll
-      for (int t = 0; t < NT; ++t) {
-        if (first && t > 0) continue;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) racc[v][t] += __shfl_xor_sync(0xffffffffu, racc[v][t], o);
-      }
-  }
+  if (warp < x.nlong) lane_sums<SQ>(&racc[0][0], lane);  // the lanes' shares of a long list
   // per variable the exponent e with |r 2^-p| < 2^e over the nodes (p: the row's exponent)
   // (infinities and NaN: kPdNone, the product is NaN then)
   auto expo = [&](double r, int p) {
@@ -383,7 +556,6 @@ __device__ __forceinline__ longlong2 pd_apply() {
   constexpr int NT1 = FIRST ? 1 : P::NNT, QL = FIRST ? 20 : 20 * NTP;
   const PdView<N> V;
   const PdShared& x = pd_shared();
-  const PdRef& ref = x.ref;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gq = lane >> 2, tq = lane & 3;
   const int Ni = x.Ni, nks = x.nks;
   long long res = 0, qmax = 0;
@@ -394,10 +566,10 @@ __device__ __forceinline__ longlong2 pd_apply() {
     for (int s = 0; s < NT; ++s) {
       double z = uh;
       if constexpr (FIRST) {
-        z -= ref.kws[s] * y[0];
+        z -= x.dkws[s] * y[0];
       } else {
 #pragma unroll
-        for (int t = 0; t < NT; ++t) z -= ref.kw[s][t] * y[t];
+        for (int t = 0; t < NT; ++t) z -= x.dkw[s][t] * y[t];
       }
       const double old = FIRST ? uh : qp[s];
       // maxima of magnitudes as integers: non-negative doubles order as their bits
@@ -411,68 +583,21 @@ __device__ __forceinline__ longlong2 pd_apply() {
   };
   for (int job = warp; job < nks * NT1; job += W) {
     const int mt = job / NT1, nt = job - mt * NT1;
-    long long hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
-    const uint32_t* const at = x.dig + (size_t)mt * nks * 512 + lane * 4;
-    const unsigned char* const bt = reinterpret_cast<const unsigned char*>(V.region) + nt * 1024 + lane * 32;
-    const bool on = nt * 32 + lane < QL;
-    uint4 nx[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) nx[q] = ldg_stream(at + q * 128);
-    for (int k0 = 0; k0 < nks; k0 += 7) {  // 112 columns: what the FP32 accumulators hold exactly
-      float acc[8][4];
-#pragma unroll
-      for (int l = 0; l < 8; ++l)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) acc[l][i] = 0.f;
-      const int k1 = min(k0 + 7, nks);
-#pragma unroll 1
-      for (int ks = k0; ks < k1; ++ks) {
-        uint4 A[8];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const uint32_t w[4] = {nx[q].x, nx[q].y, nx[q].z, nx[q].w};
-#pragma unroll
-          for (int s = 0; s < 2; ++s)
-            A[2 * q + s] = make_uint4(digit_pair(w[2 * s], 0x4140), digit_pair(w[2 * s], 0x4342),
-                                      digit_pair(w[2 * s + 1], 0x4140), digit_pair(w[2 * s + 1], 0x4342));
-        }
-        const uint32_t* t = at + (size_t)min(ks + 1, nks - 1) * 512;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) nx[q] = ldg_stream(t + q * 128);
-        const uint4 z4 = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
-        const uint4 b0 = on ? *reinterpret_cast<const uint4*>(bt + ks * fb) : z4;
-        const uint4 b1 = on ? *reinterpret_cast<const uint4*>(bt + ks * fb + 16) : z4;
-        const uint32_t b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const uint32_t c0 = digit_pair(b[u], 0x4140), c1 = digit_pair(b[u], 0x4342);
-#pragma unroll
-          for (int s = 0; s + u < 8; ++s) mma_f16(acc[s + u], A[s], c0, c1);
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        int a[8];
-#pragma unroll
-        for (int l = 0; l < 8; ++l) a[l] = __float2int_rn(acc[l][i]);
-        hi[i] += ((long long)a[0] << 24) + ((long long)a[1] << 16) + ((long long)a[2] << 8) + a[3];
-        lo[i] += ((long long)a[4] << 24) + ((long long)a[5] << 16) + ((long long)a[6] << 8) + a[7];
-      }
-    }
+    long long hi[4], lo[4];
+    digit_product(x.dig + (size_t)mt * nks * 512 + lane * 4,
+                  reinterpret_cast<const unsigned char*>(V.region) + nt * 1024 + lane * 32, fb, nt * 32 + lane < QL, nks, hi,
+                  lo);
     // digit s of one factor weighs 2^(56 - 8 s): level l 2^(112 - 8 l); the factors are scaled by 2^62
     // (over the row's, column's and right-hand side's powers)
     auto value = [&](int i, int n, int v) {
-      if (x.ev[v] >= kPdNone) return __hiloint2double(0x7ff80000, 0);
-      const double s = fma((double)hi[i], 4294967296.0, (double)lo[i]);
-      const int k = max(-2000, min(2000, 56 - 124 + x.ev[v] - V.sexp[n]));
-      return s * pow2(k / 2) * pow2(k - k / 2);
+      return digit_value(hi[i], lo[i], 56 - 124 + x.ev[v] - V.sexp[n], x.ev[v] >= kPdNone);
     };
     if constexpr (FIRST) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int v = 2 * tq + (i & 1), n = mt * 16 + gq + (i >> 1) * 8;
         if (v < 5 && n < Ni) {
-          const double y[NT] = {value(i, n, v) * x.dt};
+          const double y[NT] = {value(i, n, v)};
           update(n, v, y);
         }
       }
@@ -481,7 +606,7 @@ __device__ __forceinline__ longlong2 pd_apply() {
       for (int h = 0; h < 2; ++h) {
         const int v = nt * 4 + tq, n = mt * 16 + gq + 8 * h;
         if (v < 5 && n < Ni) {
-          const double y[2] = {value(2 * h, n, v) * x.dt, value(2 * h + 1, n, v) * x.dt};
+          const double y[2] = {value(2 * h, n, v), value(2 * h + 1, n, v)};
           update(n, v, y);
         }
       }
@@ -502,7 +627,7 @@ __device__ __forceinline__ longlong2 pd_apply() {
       if (v < 5 && n < Ni) {
         double y[NT];
 #pragma unroll
-        for (int t = 0; t < NT; ++t) y[t] = value(t, n, v) * x.dt;
+        for (int t = 0; t < NT; ++t) y[t] = value(t, n, v);
         update(n, v, y);
       }
     }
@@ -532,7 +657,7 @@ __device__ __forceinline__ void pd_epilogue() {
     for (int v = 0; v < 5; ++v) vacc[r][v] = 0.0;
     node[r] = slot_list(V.slist, x.Ni, x.nlong, tid + r * THR, cur[r], cend[r], cstep[r]);
   }
-  const int cap = x.room / (5 * cv * 8), nch = (S + cap - 1) / cap, CH = (S + nch - 1) / nch;
+  const int cap = (x.room - 8 * P::CB) / (5 * (cv * 8 + P::CB - KKS * 8 + 4)), nch = (S + cap - 1) / cap, CH = (S + nch - 1) / nch;
   const double gm1 = m.gamma - 1.0, dt = x.dt;
   for (int kc = 0; kc < S; kc += CH) {
     const int nk = min(CH, S - kc);
@@ -619,16 +744,7 @@ __device__ __forceinline__ void pd_epilogue() {
       }
     }
     __syncthreads();
-    for (int col = tid; col < nk * 5; col += THR) {
-      double acc[NP];
-#pragma unroll
-      for (int i = 0; i < NP; ++i) acc[i] = 0.0;
-      double* b = V.region + col * cv;
-      SrefFP64<N>::contract_t(b, acc);
-      asm volatile("" ::: "memory");
-#pragma unroll
-      for (int i = 0; i < NP; ++i) b[i] = acc[i];
-    }
+    pd_contract<N, W>(ref, true, nk * 5, cv);
     __syncthreads();
 #pragma unroll
     for (int r = 0; r <= kPcOver; ++r) {
@@ -644,10 +760,7 @@ __device__ __forceinline__ void pd_epilogue() {
     }
   }
   if (warp < x.nlong) {
-#pragma unroll
-    for (int v = 0; v < 5; ++v)
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) vacc[0][v] += __shfl_xor_sync(0xffffffffu, vacc[0][v], o);
+    lane_sums<5>(vacc[0], lane);
     if (lane) node[0] = -1;
   }
   double* const vol = (double*)m.vol;
@@ -732,6 +845,10 @@ __global__ void __launch_bounds__(32 * W, MB) predictor_f64_kernel(const __grid_
       x.o_q = o_q;
       x.o_region = o_region;
       x.dt = *m.dt;
+      for (int s = 0; s < NT; ++s) {
+        x.dkws[s] = x.dt * ref.kws[s];
+        for (int t = 0; t < NT; ++t) x.dkw[s][t] = x.dt * ref.kw[s][t];
+      }
       x.mu = m.mu[c];
       x.kap = cell_kappa(m, x.mu);
       x.nlong = min((int)*reinterpret_cast<const uint16_t*>(m.gat + gat_start(n0, k0, s0, c, NP, NF)), W);

@@ -14,7 +14,15 @@ struct PdRef {
   double w[4];      // Gauss-Legendre weights
   double kw[4][4];  // K1t^-1[s][t] w_t
   double kws[4];    // sum_t K1t^-1[s][t] w_t
+  // digits of S^ and of S^ transposed (rows m, columns (d, j)), 16 x 16 tiles of 512 words, for
+  // |entries| < 2^sexp
+  const uint32_t *sdig, *sdig_t;
+  int sexp;
 };
+
+// Words of one of the two digit tables of S^, and the tables (host).
+int pd_stiffness_words(int N);
+int pd_stiffness_digits(const RefData& ref, bool transposed, uint32_t* out);  // returns the exponent
 
 // Blocks per SM (0: the cells do not fit) and dynamic shared memory of a block.
 struct PdPlan {
