@@ -178,12 +178,12 @@ StepPlan plan_of(afe_mesh* m) {
 bool corrector_f32_fits(int Nmax) { return Nmax <= 2 * 4 * afe::kCorrThreads; }
 
 // Plan of the FP32 predictor with several cells per SM (blocks = 0: the one-block form runs).
-afe_status plan_cells(int order, int device, int n_sm, int64_t cells, int Nmax, int Smax, int Fmax, afe::PcPlan* out) {
+afe_status plan_cells(int order, int device, int n_sm, int64_t cells, bool viscous, int Nmax, int Smax, int Fmax, afe::PcPlan* out) {
   *out = afe::PcPlan{};
   switch (order) {
-    case 1: AFE_CUDA(afe::pc_plan<1>(device, n_sm, cells, Nmax, Smax, Fmax, out)); break;
-    case 2: AFE_CUDA(afe::pc_plan<2>(device, n_sm, cells, Nmax, Smax, Fmax, out)); break;
-    case 3: AFE_CUDA(afe::pc_plan<3>(device, n_sm, cells, Nmax, Smax, Fmax, out)); break;
+    case 1: AFE_CUDA(afe::pc_plan<1>(device, n_sm, cells, viscous, Nmax, Smax, Fmax, out)); break;
+    case 2: AFE_CUDA(afe::pc_plan<2>(device, n_sm, cells, viscous, Nmax, Smax, Fmax, out)); break;
+    case 3: AFE_CUDA(afe::pc_plan<3>(device, n_sm, cells, viscous, Nmax, Smax, Fmax, out)); break;
     default: break;
   }
   return AFE_OK;
@@ -438,7 +438,9 @@ afe_status set_up_cells(afe_mesh* m, int64_t nminv) {
       m->cref.zs[b] += R.Z[a][b];
     }
   afe::PcPlan pc;
-  AFE_TRY(plan_cells(m->p.order, m->device, m->n_sm, T.C, T.Nmax, T.Smax, T.slots_max, &pc));
+  StepPlan kinds;
+  add_kinds(&kinds, m);
+  AFE_TRY(plan_cells(m->p.order, m->device, m->n_sm, T.C, !kinds.inviscid, T.Nmax, T.Smax, T.slots_max, &pc));
   if (!pc.blocks) return AFE_OK;
   if (m->alloc(&m->dm.m16, (size_t)nminv) != AFE_OK ||
       m->alloc(&m->dm.gat, afe::pc_gather_bytes(m->dm, T.T, R.Np, R.Nf)) != AFE_OK) {
@@ -1242,7 +1244,7 @@ afe_status afe_batch_create(afe_mesh* const* members, int n_members, void* cuda_
       Fmax = std::max(Fmax, m->topo.slots_max);
       all = all && m->pc.blocks > 0;
     }
-    if (all) AFE_TRY(plan_cells(P.order, m0->device, m0->n_sm, C, Nmax, Smax, Fmax, &P.pc));
+    if (all) AFE_TRY(plan_cells(P.order, m0->device, m0->n_sm, C, !P.inviscid, Nmax, Smax, Fmax, &P.pc));
   }
   b->tc_fits = afe::tc_cell_plan(P.order, P.f32_smem, Smax, Nmax).ok ? 1 : 0;
   P.f32_tc = b->tc_fits;

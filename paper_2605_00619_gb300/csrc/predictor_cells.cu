@@ -82,13 +82,16 @@ void launch_shape(const PcPlan& p, const Batch& b, const PcRef& ref, bool invisc
 }  // namespace
 
 template <int N>
-cudaError_t pc_plan(int device, int n_sm, int64_t cells, int Nmax, int Smax, int Fmax, PcPlan* out) {
+cudaError_t pc_plan(int device, int n_sm, int64_t cells, bool viscous, int Nmax, int Smax, int Fmax, PcPlan* out) {
   // the largest cell has to leave room for two blocks per SM (shape 1) in any case: meshes beyond
   // that take the one-block form whatever their size
   PcPlan many;
   cudaError_t e = plan_shape<N, 1>(device, Nmax, Smax, Fmax, &many);
   *out = many;
-  if (e != cudaSuccess || !many.blocks || cells > (int64_t)n_sm * PcShape<N, 0, false>::MB) return e;
+  // at P2 the viscous fluxes' registers make eight warps per cell the better shape for any number of
+  // cells (21^3 Navier-Stokes: 1,345 us per launch against 1,565)
+  const bool wide = cells <= (int64_t)n_sm * PcShape<N, 0, false>::MB || (N == 2 && viscous);
+  if (e != cudaSuccess || !many.blocks || !wide) return e;
   PcPlan few;
   e = plan_shape<N, 0>(device, Nmax, Smax, Fmax, &few);
   if (few.blocks) *out = few;
@@ -109,7 +112,7 @@ void pc_correct(const Batch& b, const CorrRef& ref, int Nmax, int Fmax, cudaStre
 }
 
 template void pc_correct<AFE_ORDER>(const Batch&, const CorrRef&, int, int, cudaStream_t);
-template cudaError_t pc_plan<AFE_ORDER>(int, int, int64_t, int, int, int, PcPlan*);
+template cudaError_t pc_plan<AFE_ORDER>(int, int, int64_t, bool, int, int, int, PcPlan*);
 template void pc_launch<AFE_ORDER>(const PcPlan&, const Batch&, const PcRef&, bool, bool, int, int, cudaStream_t);
 
 #if AFE_ORDER == 1

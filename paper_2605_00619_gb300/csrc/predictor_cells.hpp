@@ -31,9 +31,9 @@ struct PcPlan {
   int Fmax = 0;
 };
 
-// Plan for `cells` cells of up to Nmax nodes, Smax sub-tets and Fmax face slots on n_sm SMs.
+// Plan for `cells` cells (`viscous`: every one with viscous fluxes) of up to Nmax nodes, Smax sub-tets and Fmax face slots on n_sm SMs.
 template <int N>
-cudaError_t pc_plan(int device, int n_sm, int64_t cells, int Nmax, int Smax, int Fmax, PcPlan* out);
+cudaError_t pc_plan(int device, int n_sm, int64_t cells, bool viscous, int Nmax, int Smax, int Fmax, PcPlan* out);
 
 // Launches the kernels of the kinds of cells that may be present.
 template <int N>
