@@ -70,6 +70,7 @@ struct afe_mesh {
   size_t f32_smem = 0;
   afe::CorrRef cref{};   // ... and the face mass of its corrector
   afe::PcRef pref{};     // time-basis constants of the predictor with several cells per SM
+  afe::PcCells pcells{}; // what its plan needs to know of the cells
   afe::PcPlan pc{};           // its plan for this mesh's cells (blocks = 0: not used)
   afe::PdRef dref{};     // the same for the FP64 predictor with its product on the tensor cores
   afe::PdPlan pd{};
@@ -124,6 +125,10 @@ namespace {
 // for shared memory) take the single mesh's record directly.
 struct StepPlan {
   const afe::Batch* b = nullptr;
+  // the members on the form with several cells per SM, and those on the one-block form (FP32), which keep
+  // their form in any batch, so that a member's result does not depend on its neighbours
+  const afe::Batch* cells = nullptr;
+  const afe::Batch* one = nullptr;
   cudaStream_t st = nullptr;
   int order = 1, fp32 = 0, limiter = 0, n_sm = 1, diag = 0;
   int f32_ok = 0, f32_tc = 0;
@@ -165,6 +170,7 @@ StepPlan plan_of(afe_mesh* m) {
   P.f32_tc = m->f32_tc;
   P.f32_smem = m->f32_smem;
   P.pc = m->pc;
+  (m->pc.blocks ? P.cells : P.one) = &m->self;
   P.pref = m->pref;
   P.cref = m->cref;
   P.pd = m->pd;
@@ -178,12 +184,13 @@ StepPlan plan_of(afe_mesh* m) {
 bool corrector_f32_fits(int Nmax) { return Nmax <= 2 * 4 * afe::kCorrThreads; }
 
 // Plan of the FP32 predictor with several cells per SM (blocks = 0: the one-block form runs).
-afe_status plan_cells(int order, int device, int n_sm, int64_t cells, bool viscous, int Nmax, int Smax, int Fmax, afe::PcPlan* out) {
+afe_status plan_cells(int order, int device, int n_sm, int64_t cells, bool viscous, const afe::PcCells& q,
+                      afe::PcPlan* out) {
   *out = afe::PcPlan{};
   switch (order) {
-    case 1: AFE_CUDA(afe::pc_plan<1>(device, n_sm, cells, viscous, Nmax, Smax, Fmax, out)); break;
-    case 2: AFE_CUDA(afe::pc_plan<2>(device, n_sm, cells, viscous, Nmax, Smax, Fmax, out)); break;
-    case 3: AFE_CUDA(afe::pc_plan<3>(device, n_sm, cells, viscous, Nmax, Smax, Fmax, out)); break;
+    case 1: AFE_CUDA(afe::pc_plan<1>(device, n_sm, cells, viscous, q, out)); break;
+    case 2: AFE_CUDA(afe::pc_plan<2>(device, n_sm, cells, viscous, q, out)); break;
+    case 3: AFE_CUDA(afe::pc_plan<3>(device, n_sm, cells, viscous, q, out)); break;
     default: break;
   }
   return AFE_OK;
@@ -192,16 +199,15 @@ afe_status plan_cells(int order, int device, int n_sm, int64_t cells, bool visco
 template <int N, typename Real>
 void launch_predictor(const StepPlan& P) {
   if constexpr (N <= 3) {  // the shared-memory FP32 predictor exists for N <= 3 (cells up to 640 nodes)
-    if (sizeof(Real) == 4 && P.f32_ok && P.pc.blocks && !P.f32_tc) {
-      afe::pc_launch<N>(P.pc, *P.b, P.pref, P.inviscid, P.viscous, P.diag, P.n_sm, P.st);
-      return;
-    }
     if (sizeof(Real) == 4 && P.f32_ok) {
-      if (P.f32_tc)
+      if (P.f32_tc) {
         afe::predictor_f32_kernel<N, true><<<P.n_sm, afe::kF32Threads, P.f32_smem, P.st>>>(*P.b, P.d_ref, P.diag,
                                                                                          (int)P.f32_smem);
-      else
-        afe::predictor_f32_kernel<N, false><<<P.n_sm, afe::kF32Threads, P.f32_smem, P.st>>>(*P.b, P.d_ref, P.diag,
+        return;
+      }
+      if (P.cells) afe::pc_launch<N>(P.pc, *P.cells, P.pref, P.inviscid, P.viscous, P.diag, P.n_sm, P.st);
+      if (P.one)
+        afe::predictor_f32_kernel<N, false><<<P.n_sm, afe::kF32Threads, P.f32_smem, P.st>>>(*P.one, P.d_ref, P.diag,
                                                                                           (int)P.f32_smem);
       return;
     }
@@ -261,17 +267,19 @@ void launch_face(const StepPlan& P) {
 
 template <int N, typename Real>
 afe_status launch_corrector(const StepPlan& P) {
-  if constexpr (N <= 3)
-    if (sizeof(Real) == 4 && P.pc.blocks) {  // the cells' split M_i^-1 is there
-      afe::pc_correct<N>(*P.b, P.cref, P.b->Nmax, P.pc.Fmax, P.st);
-      return AFE_OK;
+  if constexpr (N <= 3 && sizeof(Real) == 4) {
+    if (P.cells) {  // the cells' split M_i^-1 is there
+      afe::pc_correct<N>(*P.cells, P.cref, P.cells->Nmax, P.pc.Fmax, P.st);
+      if (!P.one) return AFE_OK;
     }
-  if (sizeof(Real) == 4 && corrector_f32_fits(P.b->Nmax)) {
-    const size_t smem = (size_t)P.b->Nmax * 10 * sizeof(float);
-    if (smem > 48 * 1024)
+  }
+  const afe::Batch& b = sizeof(Real) == 4 && P.one ? *P.one : *P.b;
+  if (sizeof(Real) == 4 && corrector_f32_fits(b.Nmax)) {
+    const size_t smem = (size_t)b.Nmax * 10 * sizeof(float);
+    if (smem > 32 * 1024)  // the static part (11 KB) counts against the 48 KB that need no opt-in
       AFE_CUDA(cudaFuncSetAttribute(afe::corrector_f32_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)smem));
-    afe::corrector_f32_kernel<N><<<(unsigned)P.b->cpre[P.b->nh], afe::kCorrThreads, smem, P.st>>>(*P.b, P.d_ref);
+    afe::corrector_f32_kernel<N><<<(unsigned)b.cpre[b.nh], afe::kCorrThreads, smem, P.st>>>(b, P.d_ref);
     return AFE_OK;
   }
   afe_mesh* m = P.single;
@@ -346,8 +354,9 @@ afe_status record(const StepPlan& P) {
 // kernels per step: begin + [means + limiter] + (set_dt | cfl + finalize) + predictor (one for
 // each kind of cell) + face + corrector + clock
 int launches_per_step(const StepPlan& P, double dt) {
-  const int both = (P.fp32 ? P.pc.blocks && !P.f32_tc : P.pd.blocks) && P.inviscid && P.viscous;
-  return 1 + (P.limiter ? 2 : 0) + (dt > 0 ? 1 : 2) + 3 + both + 1;
+  const int both = (P.fp32 ? P.cells && !P.f32_tc : P.pd.blocks > 0) && P.inviscid && P.viscous;
+  const int groups = P.cells && P.one ? (P.f32_tc ? 1 : 2) : 0;  // predictor and corrector once per form
+  return 1 + (P.limiter ? 2 : 0) + (dt > 0 ? 1 : 2) + 3 + both + groups + 1;
 }
 
 afe_status enqueue_step(const StepPlan& P, double dt) {
@@ -440,9 +449,16 @@ afe_status set_up_cells(afe_mesh* m, int64_t nminv) {
   afe::PcPlan pc;
   StepPlan kinds;
   add_kinds(&kinds, m);
-  AFE_TRY(plan_cells(m->p.order, m->device, m->n_sm, T.C, !kinds.inviscid, T.Nmax, T.Smax, T.slots_max, &pc));
+  for (int64_t c = 0; c < T.C; ++c) {
+    const int n = (int)(T.node_ptr[c + 1] - T.node_ptr[c]), s = (int)(T.sub_ptr[c + 1] - T.sub_ptr[c]);
+    const int ns = (int)(T.slot_ptr[c + 1] - T.slot_ptr[c]);
+    if (R.N == 1) afe::pc_add_cell<1>(n, s, ns, &m->pcells);
+    else if (R.N == 2) afe::pc_add_cell<2>(n, s, ns, &m->pcells);
+    else afe::pc_add_cell<3>(n, s, ns, &m->pcells);
+  }
+  AFE_TRY(plan_cells(m->p.order, m->device, m->n_sm, T.C, !kinds.inviscid, m->pcells, &pc));
   if (!pc.blocks) return AFE_OK;
-  if (m->alloc(&m->dm.m16, (size_t)nminv) != AFE_OK ||
+  if (m->alloc(&m->dm.m16, (size_t)afe::minv_split_start(nminv, T.n_nodes, T.C)) != AFE_OK ||
       m->alloc(&m->dm.gat, afe::pc_gather_bytes(m->dm, T.T, R.Np, R.Nf)) != AFE_OK) {
     (void)cudaGetLastError();  // out of memory: the one-block form needs neither
     return AFE_OK;
@@ -707,7 +723,7 @@ afe_status afe_mesh_create(const afe_params* p, int64_t n_vertices, const double
   AFE_TRY(M->alloc(&d.tacc, 1));
   AFE_TRY(M->alloc(&d.maxbits, 1));
   AFE_TRY(M->alloc(&d.flags, afe::F_COUNT));
-  AFE_TRY(M->alloc(&d.work, 2));
+  AFE_TRY(M->alloc(&d.work, 3));
   AFE_TRY(M->alloc(&M->d_ref, 1));
 
   AFE_TRY(M->alloc(&M->d_totals_partial, (size_t)M->totals_blocks * 5));
@@ -1117,6 +1133,8 @@ afe_status afe_device_bytes(const afe_mesh* m, int64_t* bytes) {
 struct afe_batch {
   std::vector<afe_mesh*> mem;
   afe::Batch bt{};
+  afe::Batch sub[2]{};          // with members on both FP32 forms: those with several cells per SM, the others
+  int32_t* d_suborder[2] = {nullptr, nullptr};
   int* d_work = nullptr;
   cudaStream_t st = nullptr;
   bool own_stream = false;
@@ -1134,6 +1152,8 @@ struct afe_batch {
     if (gexec) cudaGraphExecDestroy(gexec);
     if (graph) cudaGraphDestroy(graph);
     if (d_order) cudaFree(d_order);
+    for (int32_t* o : d_suborder)
+      if (o) cudaFree(o);
     if (d_work) cudaFree(d_work);
     if (own_stream && st) cudaStreamDestroy(st);
   }
@@ -1211,7 +1231,7 @@ afe_status afe_batch_create(afe_mesh* const* members, int n_members, void* cuda_
   if (dev != m0->device) return fail(AFE_EINVAL, "the current device is not the members' device");
   {
     void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, 2 * sizeof(int));
+    cudaError_t e = cudaMalloc(&p, 3 * sizeof(int));
     if (e != cudaSuccess) return fail(AFE_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
     b->d_work = (int*)p;
   }
@@ -1234,17 +1254,34 @@ afe_status afe_batch_create(afe_mesh* const* members, int n_members, void* cuda_
   P.diag = 0;
   P.f32_ok = 1;
   P.f32_smem = m0->f32_smem;
-  P.pref = m0->pref;
-  P.cref = m0->cref;
   for (afe_mesh* m : b->mem) add_kinds(&P, m);
-  {
-    int Fmax = 0;
-    bool all = true;  // every member holds the data of the several-cells form
+  {  // the members by form (the first sub-table: several cells per SM)
+    afe::PcCells q;
     for (afe_mesh* m : b->mem) {
-      Fmax = std::max(Fmax, m->topo.slots_max);
-      all = all && m->pc.blocks > 0;
+      afe::Batch& t = b->sub[m->pc.blocks ? 0 : 1];
+      t.tab[t.nh] = m->dm;
+      t.cpre[t.nh + 1] = t.cpre[t.nh] + m->topo.C;
+      t.gpre[t.nh + 1] = t.gpre[t.nh] + m->topo.n_groups;
+      ++t.nh;
+      t.Nmax = std::max(t.Nmax, m->topo.Nmax);
+      t.Smax = std::max(t.Smax, m->topo.Smax);
+      if (!m->pc.blocks) continue;
+      q.Nmax = std::max(q.Nmax, m->pcells.Nmax);
+      q.Smax = std::max(q.Smax, m->pcells.Smax);
+      q.Fmax = std::max(q.Fmax, m->pcells.Fmax);
+      for (int k = 0; k < 2; ++k) q.need[k] = std::max(q.need[k], m->pcells.need[k]);
+      P.pref = m->pref;
+      P.cref = m->cref;
     }
-    if (all) AFE_TRY(plan_cells(P.order, m0->device, m0->n_sm, C, !P.inviscid, Nmax, Smax, Fmax, &P.pc));
+    b->sub[0].work = b->d_work;
+    b->sub[1].work = b->d_work + 2;
+    const bool mixed = b->sub[0].nh && b->sub[1].nh;
+    if (b->sub[0].nh) {
+      P.cells = mixed ? &b->sub[0] : &b->bt;
+      AFE_TRY(plan_cells(P.order, m0->device, m0->n_sm, b->sub[0].cpre[b->sub[0].nh], !P.inviscid, q, &P.pc));
+      if (!P.pc.blocks) return fail(AFE_ECUDA, "the members' plans do not combine");
+    }
+    if (b->sub[1].nh) P.one = mixed ? &b->sub[1] : &b->bt;
   }
   b->tc_fits = afe::tc_cell_plan(P.order, P.f32_smem, Smax, Nmax).ok ? 1 : 0;
   P.f32_tc = b->tc_fits;
@@ -1328,6 +1365,23 @@ afe_status afe_batch_set_schedule(afe_batch* b, const afe_schedule* s) {
     b->d_order = (int32_t*)p;
     AFE_CUDA(cudaMemcpy(b->d_order, ord.data(), ord.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
   }
+  for (int k = 0; k < 2; ++k) {
+    afe::Batch& t = b->sub[k];
+    if (s->cost_order && t.nh && !b->d_suborder[k]) {
+      std::vector<const afe::Topology*> tops;
+      for (afe_mesh* m : b->mem)
+        if ((m->pc.blocks ? 0 : 1) == k) tops.push_back(&m->topo);
+      const std::vector<int32_t> ord = cost_order(tops, b->plan.order);
+      void* p = nullptr;
+      cudaError_t e = cudaMalloc(&p, ord.size() * sizeof(int32_t));
+      if (e != cudaSuccess) return fail(AFE_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+      b->d_suborder[k] = (int32_t*)p;
+      AFE_CUDA(cudaMemcpy(b->d_suborder[k], ord.data(), ord.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
+    }
+    t.ring_cap = s->ring_cap;
+    t.narrow = s->narrow;
+    t.order = s->cost_order ? b->d_suborder[k] : nullptr;
+  }
   b->sched = *s;
   b->bt.ring_cap = s->ring_cap;
   b->bt.narrow = s->narrow;
@@ -1370,7 +1424,7 @@ afe_status autotune_impl(const std::string& sig, int order, bool tc_fits, int* w
   AFE_CUDA(cudaEventCreate(&e1));
   // several cells per SM: only the order of the cells is a choice (ring_cap and narrow belong to the
   // one-block form, which with either apply is the slower one for these cells)
-  const bool one_block = plan().pc.blocks == 0;
+  const bool one_block = plan().one != nullptr;
   std::vector<afe_schedule> cand;
   for (int co = 0; co < 2; ++co)
     for (int va = 0; va < (one_block && tc_fits ? 2 : 1); ++va)
@@ -1387,7 +1441,7 @@ afe_status autotune_impl(const std::string& sig, int order, bool tc_fits, int* w
     float ms = 0.f;
     for (int r = 0; r <= trials && status == AFE_OK; ++r) {
       if (r == 1) cudaEventRecord(e0, st);
-      cudaMemsetAsync(work, 0, 2 * sizeof(int), st);
+      cudaMemsetAsync(work, 0, 3 * sizeof(int), st);
       status = stage(P, 0);
     }
     if (status != AFE_OK) break;

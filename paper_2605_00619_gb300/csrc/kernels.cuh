@@ -69,7 +69,7 @@ struct DevMesh {
   double* tacc;   // device scalar: accumulated time
   unsigned long long* maxbits;
   int* flags;
-  int* work;      // work counter of the persistent predictor
+  int* work;      // work counters of the persistent predictors
   double* qbar_diag;
   // physics
   double gamma, Rgas, cv, cfl, m1, mu0, Pr, kappa0, tol, h_min;
@@ -88,7 +88,7 @@ struct Batch {
   int ring_cap;                  // FP32 predictor: most M_i^-1 ring stages (0: as many as fit)
   int narrow;                    // FP32 predictor: 1 = narrow right-hand-side chunks everywhere
   int pad;
-  int* work;                     // work counter of the persistent predictor
+  int* work;                     // work counters of the persistent predictors (three)
   const int32_t* order;          // global cells in the order the predictor takes them (NULL: index order)
   int64_t cpre[kMaxBatch + 1];   // prefix sums of the members' cells
   int64_t gpre[kMaxBatch + 1];   // prefix sums of the members' polygonal faces
@@ -368,7 +368,7 @@ static __global__ void flags_clear_kernel(const __grid_constant__ Batch bt) {
 // persistent predictor.
 static __global__ void step_begin_kernel(const __grid_constant__ Batch bt) {
   for (int h = threadIdx.x; h < bt.nh; h += blockDim.x) *bt.tab[h].maxbits = 0ull;
-  if (threadIdx.x < 2) bt.work[threadIdx.x] = 0;
+  if (threadIdx.x < 3) bt.work[threadIdx.x] = 0;
 }
 
 // Sec. 4.5: cell means u_bar_i = w_i . u_i / |P_i| (w_i = M_i 1), one warp per cell, kept as what the

@@ -32,7 +32,8 @@ size_t corr_smem(int n, int ns, int nf) {
 }
 
 template <int N, int SHAPE>
-cudaError_t plan_shape(int device, int Nmax, int Smax, int Fmax, PcPlan* out) {
+cudaError_t plan_shape(int device, const PcCells& q, PcPlan* out) {
+  const int Nmax = q.Nmax, Smax = q.Smax, Fmax = q.Fmax;
   constexpr int W = PcShape<N, SHAPE, false>::W, MB = PcShape<N, SHAPE, false>::MB, THR = 32 * W;
   *out = PcPlan{};
   if (pc_slots(Nmax, THR) > (kPcOver + 1) * THR || Smax > kPcMaxSub) return cudaSuccess;
@@ -48,7 +49,7 @@ cudaError_t plan_shape(int device, int Nmax, int Smax, int Fmax, PcPlan* out) {
     // 1 KB of every block's share is the system's
     const int64_t share = std::min<int64_t>(per_sm / nb - 1024, optin) - stat;
     const size_t smem = share > 0 ? (size_t)share / 128 * 128 : 0;
-    if (pc_need<N>(Nmax, Smax, Fmax, THR) > smem) continue;
+    if (q.need[SHAPE] > smem) continue;
     // the limit is the function's, shared by every handle: the most any plan may ask for
     e = cudaFuncSetAttribute(pc_kernel<N, SHAPE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - stat);
     if (e == cudaSuccess)
@@ -82,18 +83,27 @@ void launch_shape(const PcPlan& p, const Batch& b, const PcRef& ref, bool invisc
 }  // namespace
 
 template <int N>
-cudaError_t pc_plan(int device, int n_sm, int64_t cells, bool viscous, int Nmax, int Smax, int Fmax, PcPlan* out) {
+void pc_add_cell(int n, int s, int ns, PcCells* q) {
+  q->Nmax = std::max(q->Nmax, n);
+  q->Smax = std::max(q->Smax, s);
+  q->Fmax = std::max(q->Fmax, ns);
+  q->need[0] = std::max(q->need[0], pc_need<N>(n, s, ns, 32 * PcShape<N, 0, false>::W));
+  q->need[1] = std::max(q->need[1], pc_need<N>(n, s, ns, 32 * PcShape<N, 1, false>::W));
+}
+
+template <int N>
+cudaError_t pc_plan(int device, int n_sm, int64_t cells, bool viscous, const PcCells& q, PcPlan* out) {
   // the largest cell has to leave room for two blocks per SM (shape 1) in any case: meshes beyond
   // that take the one-block form whatever their size
   PcPlan many;
-  cudaError_t e = plan_shape<N, 1>(device, Nmax, Smax, Fmax, &many);
+  cudaError_t e = plan_shape<N, 1>(device, q, &many);
   *out = many;
   // at P2 the viscous fluxes' registers make eight warps per cell the better shape for any number of
   // cells (21^3 Navier-Stokes: 1,345 us per launch against 1,565)
   const bool wide = cells <= (int64_t)n_sm * PcShape<N, 0, false>::MB || (N == 2 && viscous);
   if (e != cudaSuccess || !many.blocks || !wide) return e;
   PcPlan few;
-  e = plan_shape<N, 0>(device, Nmax, Smax, Fmax, &few);
+  e = plan_shape<N, 0>(device, q, &few);
   if (few.blocks) *out = few;
   return e;
 }
@@ -112,7 +122,8 @@ void pc_correct(const Batch& b, const CorrRef& ref, int Nmax, int Fmax, cudaStre
 }
 
 template void pc_correct<AFE_ORDER>(const Batch&, const CorrRef&, int, int, cudaStream_t);
-template cudaError_t pc_plan<AFE_ORDER>(int, int, int64_t, bool, int, int, int, PcPlan*);
+template cudaError_t pc_plan<AFE_ORDER>(int, int, int64_t, bool, const PcCells&, PcPlan*);
+template void pc_add_cell<AFE_ORDER>(int, int, int, PcCells*);
 template void pc_launch<AFE_ORDER>(const PcPlan&, const Batch&, const PcRef&, bool, bool, int, int, cudaStream_t);
 
 #if AFE_ORDER == 1
@@ -122,7 +133,7 @@ static __global__ void __launch_bounds__(256) split_minv_kernel(DevMesh m) {
   for (int64_t c = blockIdx.x; c < m.C; c += gridDim.x) {
     const int n = (int)(m.node_ptr[c + 1] - m.node_ptr[c]), LD = minv_ld(n);
     const float* A = m.minv32 + m.minv_ptr[c];
-    uint32_t* out = m.m16 + m.minv_ptr[c];
+    uint32_t* out = m.m16 + minv_split_start(m.minv_ptr[c], m.node_ptr[c], c);
     if (threadIdx.x == 0) smax = 0;
     __syncthreads();
     uint32_t mx = 0;

@@ -31,9 +31,19 @@ struct PcPlan {
   int Fmax = 0;
 };
 
-// Plan for `cells` cells (`viscous`: every one with viscous fluxes) of up to Nmax nodes, Smax sub-tets and Fmax face slots on n_sm SMs.
+// What the plan needs to know of a set of cells: maxima of their nodes, sub-tets and face slots, and the
+// shared memory the most demanding one asks for by block shape.  Sets merge by maxima, so a union
+// fits whenever its parts do.
+struct PcCells {
+  int Nmax = 0, Smax = 0, Fmax = 0;
+  size_t need[2] = {0, 0};
+};
 template <int N>
-cudaError_t pc_plan(int device, int n_sm, int64_t cells, bool viscous, int Nmax, int Smax, int Fmax, PcPlan* out);
+void pc_add_cell(int n, int s, int ns, PcCells* q);
+
+// Plan for `cells` cells (`viscous`: every one with viscous fluxes) with the properties q on n_sm SMs.
+template <int N>
+cudaError_t pc_plan(int device, int n_sm, int64_t cells, bool viscous, const PcCells& q, PcPlan* out);
 
 // Launches the kernels of the kinds of cells that may be present.
 template <int N>

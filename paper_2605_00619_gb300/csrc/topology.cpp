@@ -392,11 +392,9 @@ int build_topology(const RefData& R, int64_t n_vertices, const double* xyz, int6
     T.node_ptr[c + 1] = T.node_ptr[c] + cells[c].Ni;
     T.sub_ptr[c + 1] = T.sub_ptr[c] + cells[c].S;
     T.slot_ptr[c + 1] = T.slot_ptr[c] + (int64_t)cells[c].slots.size();
-    // rows padded to minv_ld words, blocks to a multiple of 32 words (128 bytes) that also holds
-    // the split form (more only for cells of fewer than 20 nodes)
-    const int64_t n = cells[c].Ni;
-    const int64_t words = std::max(n * minv_ld((int)n), minv_split_words((int)n));
-    T.minv_ptr[c + 1] = T.minv_ptr[c] + (words + 31) / 32 * 32;
+    // rows padded to minv_ld words, blocks to a multiple of 32 words (128 bytes)
+    const int64_t ld = minv_ld(cells[c].Ni);
+    T.minv_ptr[c + 1] = T.minv_ptr[c] + ((int64_t)cells[c].Ni * ld + 31) / 32 * 32;
     T.Nmax = std::max(T.Nmax, cells[c].Ni);
     T.Smax = std::max(T.Smax, cells[c].S);
     T.slots_max = std::max(T.slots_max, (int)cells[c].slots.size());

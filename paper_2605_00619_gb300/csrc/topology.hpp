@@ -24,6 +24,11 @@ inline constexpr int minv_ld(int n) { return (n + 15) / 16 * 16 + 8; }
 inline constexpr int64_t minv_split_words(int n) {
   return 32 + (int64_t)((n + 15) / 16) * ((n + 15) / 16 + 1) / 2 * 256;
 }
+// Offset (words, a multiple of 32) of a cell's split block from its offset in the dense array, its first
+// node and its index: with t = ceil(n / 16), 32 + 128 t (t + 1) <= n (16 t + 8) / 2 + 12 n + 352 - 31.
+inline constexpr int64_t minv_split_start(int64_t minv_ptr, int64_t n0, int64_t c) {
+  return (minv_ptr / 2 + 12 * n0 + 352 * c) / 32 * 32;
+}
 
 struct Topology {
   int N = 0, Np = 0, Nt = 0, Nf = 0;
@@ -33,7 +38,7 @@ struct Topology {
   std::vector<int64_t> node_ptr;   // [C+1] global node offset of each cell
   std::vector<int64_t> sub_ptr;    // [C+1] sub-tet offset of each cell
   std::vector<int64_t> slot_ptr;   // [C+1] face-slot offset of each cell
-  std::vector<int64_t> minv_ptr;   // [C+1] offset of each cell's block: dense N_i x minv_ld(N_i) rows, or the split form
+  std::vector<int64_t> minv_ptr;   // [C+1] offset of the dense N_i x minv_ld(N_i) block of each cell
 
   std::vector<uint16_t> A;         // [T*Np] cell-local node of sub-tet node j
   std::vector<double> geo;         // [T*10] adj(J) row-major (adj = det(J) J^-1), det(J)

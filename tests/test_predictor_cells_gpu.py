@@ -74,3 +74,33 @@ def test_block_shapes_agree_bit_for_bit(afe, N):
         np.testing.assert_array_equal(afe.afe_get_state(m), afe.afe_get_state(h))
     for h in alone + mem:
         afe.afe_mesh_destroy(h)
+
+
+def test_a_batch_keeps_every_members_form(afe):
+    """Cells too large for two blocks per SM (623 nodes) beside small ones: each member's result is
+    that of stepping it alone, bit for bit."""
+    def handles():
+        out = []
+        for pm in (split_cube_lattice((2, 1, 1), (4, 4, 3), d=0.5), periodic_voronoi(3),
+                   split_cube_lattice((3, 1, 1), (4, 4, 3), d=0.5), periodic_voronoi(4)):
+            p = afe.afe_default_params(3, precision=afe.AFE_FP32, picard_tol=1e-6, cfl=0.1)
+            h = afe.create_from_polymesh(pm, p)
+            afe.afe_set_state(h, states.density_wave(afe.afe_get_node_coords(h), amp=0.1))
+            out.append(h)
+        return out
+
+    alone, mem = handles(), handles()
+    for h in alone:
+        for _ in range(3):
+            afe.afe_step(h, 0.0)
+    b = afe.afe_batch_create(mem)
+    afe.afe_batch_step_async(b, 0.0, 1, False)
+    afe.afe_batch_sync(b, len(mem))
+    afe.afe_batch_set_schedule(b, cost_order=1)
+    afe.afe_batch_step_async(b, 0.0, 2, True)
+    afe.afe_batch_sync(b, len(mem))
+    afe.afe_batch_destroy(b)
+    for h, m in zip(alone, mem):
+        np.testing.assert_array_equal(afe.afe_get_state(m), afe.afe_get_state(h))
+    for h in alone + mem:
+        afe.afe_mesh_destroy(h)
