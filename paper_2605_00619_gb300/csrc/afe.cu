@@ -351,10 +351,10 @@ afe_status record(const StepPlan& P) {
   return AFE_OK;
 }
 
-// kernels per step: begin + [means + limiter] + (set_dt | cfl + finalize) + predictor (one for
+// kernels per step: begin + [means + limiter] + (set_dt | cfl + finalize) + predictor (FP64: one for
 // each kind of cell) + face + corrector + clock
 int launches_per_step(const StepPlan& P, double dt) {
-  const int both = (P.fp32 ? P.cells && !P.f32_tc : P.pd.blocks > 0) && P.inviscid && P.viscous;
+  const int both = !P.fp32 && P.pd.blocks > 0 && P.inviscid && P.viscous;
   const int groups = P.cells && P.one ? (P.f32_tc ? 1 : 2) : 0;  // predictor and corrector once per form
   return 1 + (P.limiter ? 2 : 0) + (dt > 0 ? 1 : 2) + 3 + both + groups + 1;
 }

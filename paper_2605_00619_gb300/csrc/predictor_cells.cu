@@ -11,17 +11,17 @@ namespace {
 // many cells (us per step of the predictor, 24^3 P1 / 8^3 P2 / 32^3 P3 meshes), shape 0 those whose
 // cells all run at once with more warps each, where the slowest cell's latency is the time
 // (4^3 P1: 41 us with 8 warps, 58 with 2).
-template <int N, int SHAPE, bool VISC>
+template <int N, int SHAPE>
 struct PcShape;
-template <bool V> struct PcShape<1, 0, V> { static constexpr int W = 8, MB = 2; };
-template <bool V> struct PcShape<1, 1, V> { static constexpr int W = 2, MB = 10; };
-template <bool V> struct PcShape<2, 0, V> { static constexpr int W = 8, MB = 2; };
-template <bool V> struct PcShape<2, 1, V> { static constexpr int W = 4, MB = 4; };
-template <bool V> struct PcShape<3, 0, V> { static constexpr int W = 16, MB = 1; };
-template <bool V> struct PcShape<3, 1, V> { static constexpr int W = 8, MB = 2; };
+template <> struct PcShape<1, 0> { static constexpr int W = 8, MB = 2; };
+template <> struct PcShape<1, 1> { static constexpr int W = 2, MB = 10; };
+template <> struct PcShape<2, 0> { static constexpr int W = 8, MB = 2; };
+template <> struct PcShape<2, 1> { static constexpr int W = 4, MB = 4; };
+template <> struct PcShape<3, 0> { static constexpr int W = 16, MB = 1; };
+template <> struct PcShape<3, 1> { static constexpr int W = 8, MB = 2; };
 
-template <int N, int SHAPE, bool VISC>
-constexpr auto pc_kernel = predictor_cells_kernel<N, PcShape<N, SHAPE, VISC>::W, PcShape<N, SHAPE, VISC>::MB, VISC>;
+template <int N, int SHAPE, int KINDS>
+constexpr auto pc_kernel = predictor_cells_kernel<N, PcShape<N, SHAPE>::W, PcShape<N, SHAPE>::MB, KINDS>;
 
 // Warps per block of the corrector.
 template <int N>
@@ -34,26 +34,28 @@ size_t corr_smem(int n, int ns, int nf) {
 template <int N, int SHAPE>
 cudaError_t plan_shape(int device, const PcCells& q, PcPlan* out) {
   const int Nmax = q.Nmax, Smax = q.Smax, Fmax = q.Fmax;
-  constexpr int W = PcShape<N, SHAPE, false>::W, MB = PcShape<N, SHAPE, false>::MB, THR = 32 * W;
+  constexpr int W = PcShape<N, SHAPE>::W, MB = PcShape<N, SHAPE>::MB, THR = 32 * W;
   *out = PcPlan{};
   if (pc_slots(Nmax, THR) > (kPcOver + 1) * THR || Smax > kPcMaxSub) return cudaSuccess;
-  cudaFuncAttributes fa, fv;
-  cudaError_t e = cudaFuncGetAttributes(&fa, pc_kernel<N, SHAPE, false>);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fv, pc_kernel<N, SHAPE, true>);
-  int per_sm = 0, optin = 0;
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device);
+  int per_sm = 0, optin = 0, stat = 0;
+  cudaError_t e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+  void (*const kernels[3])(const Batch, const PcRef, int, int) = {pc_kernel<N, SHAPE, 1>, pc_kernel<N, SHAPE, 2>,
+                                                                  pc_kernel<N, SHAPE, 3>};
+  for (auto* k : kernels) {
+    cudaFuncAttributes fa;
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
+    if (e == cudaSuccess) stat = std::max(stat, (int)fa.sharedSizeBytes);
+  }
   if (e != cudaSuccess) return e;
-  const int stat = (int)std::max(fa.sharedSizeBytes, fv.sharedSizeBytes);
   for (int nb = MB; nb >= std::min(MB, 2); --nb) {
     // 1 KB of every block's share is the system's
     const int64_t share = std::min<int64_t>(per_sm / nb - 1024, optin) - stat;
     const size_t smem = share > 0 ? (size_t)share / 128 * 128 : 0;
     if (q.need[SHAPE] > smem) continue;
     // the limit is the function's, shared by every handle: the most any plan may ask for
-    e = cudaFuncSetAttribute(pc_kernel<N, SHAPE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - stat);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(pc_kernel<N, SHAPE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - stat);
+    for (auto* k : kernels)
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - stat);
     auto* corr = corrector_cells_kernel<N, corr_warps<N>>;
     cudaFuncAttributes fc;
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fc, corr);
@@ -72,12 +74,11 @@ cudaError_t plan_shape(int device, const PcCells& q, PcPlan* out) {
 template <int N, int SHAPE>
 void launch_shape(const PcPlan& p, const Batch& b, const PcRef& ref, bool inviscid, bool viscous, int diag, int n_sm,
                   cudaStream_t st) {
-  constexpr int THR = 32 * PcShape<N, SHAPE, false>::W;
-  static_assert(PcShape<N, SHAPE, true>::W == PcShape<N, SHAPE, false>::W, "one plan serves both kinds");
-  const int grid = (int)std::min<int64_t>(b.cpre[b.nh], (int64_t)n_sm * p.blocks);
-  const int smem = (int)p.smem, mixed = inviscid && viscous;
-  if (inviscid) pc_kernel<N, SHAPE, false><<<grid, THR, smem, st>>>(b, ref, diag, smem, mixed);
-  if (viscous) pc_kernel<N, SHAPE, true><<<grid, THR, smem, st>>>(b, ref, diag, smem, mixed);
+  constexpr int THR = 32 * PcShape<N, SHAPE>::W;
+  const int grid = (int)std::min<int64_t>(b.cpre[b.nh], (int64_t)n_sm * p.blocks), smem = (int)p.smem;
+  if (inviscid && viscous) pc_kernel<N, SHAPE, 3><<<grid, THR, smem, st>>>(b, ref, diag, smem);
+  else if (viscous) pc_kernel<N, SHAPE, 2><<<grid, THR, smem, st>>>(b, ref, diag, smem);
+  else pc_kernel<N, SHAPE, 1><<<grid, THR, smem, st>>>(b, ref, diag, smem);
 }
 
 }  // namespace
@@ -87,8 +88,8 @@ void pc_add_cell(int n, int s, int ns, PcCells* q) {
   q->Nmax = std::max(q->Nmax, n);
   q->Smax = std::max(q->Smax, s);
   q->Fmax = std::max(q->Fmax, ns);
-  q->need[0] = std::max(q->need[0], pc_need<N>(n, s, ns, 32 * PcShape<N, 0, false>::W));
-  q->need[1] = std::max(q->need[1], pc_need<N>(n, s, ns, 32 * PcShape<N, 1, false>::W));
+  q->need[0] = std::max(q->need[0], pc_need<N>(n, s, ns, 32 * PcShape<N, 0>::W));
+  q->need[1] = std::max(q->need[1], pc_need<N>(n, s, ns, 32 * PcShape<N, 1>::W));
 }
 
 template <int N>
@@ -100,7 +101,7 @@ cudaError_t pc_plan(int device, int n_sm, int64_t cells, bool viscous, const PcC
   *out = many;
   // at P2 the viscous fluxes' registers make eight warps per cell the better shape for any number of
   // cells (21^3 Navier-Stokes: 1,345 us per launch against 1,565)
-  const bool wide = cells <= (int64_t)n_sm * PcShape<N, 0, false>::MB || (N == 2 && viscous);
+  const bool wide = cells <= (int64_t)n_sm * PcShape<N, 0>::MB || (N == 2 && viscous);
   if (e != cudaSuccess || !many.blocks || !wide) return e;
   PcPlan few;
   e = plan_shape<N, 0>(device, q, &few);

@@ -876,30 +876,20 @@ __device__ __forceinline__ void pc_epilogue() {
       for (int v = 0; v < 5; ++v) vol[(x.n0 + node[r]) * 5 + v] = vacc[r][v];
 }
 
-// W warps per block, at least MB blocks per SM (register limit).  VISC = false takes the cells
-// without viscosity and heat conduction, VISC = true the others; a mesh that may hold both (the
-// limiter's mu_i) gets one launch of each, and each passes over the other's cells.  In one
-// kernel the viscous fluxes' registers would spill in the inviscid path too.
-template <int N, int W, int MB, bool VISC>
-__global__ void __launch_bounds__(32 * W, MB) predictor_cells_kernel(const __grid_constant__ Batch bt,
-                                                                     const __grid_constant__ PcRef ref, int diag,
-                                                                     int smem_bytes, int mixed) {
+// All cells of a kind from the queue: VISC = false the cells without viscosity and heat conduction, VISC =
+// true the others; with both kinds present (`mixed`: the limiter's mu_i) each passes over the other's.
+// One path for both would spill the viscous fluxes' registers in the inviscid cells too.  False when a
+// bounded wait gave up.
+template <int N, int W, bool VISC>
+__device__ __forceinline__ bool predictor_cells(const Batch& bt, int diag, int smem_bytes, bool mixed, uint64_t& sbar,
+                                                int& sCell, int& sAbort, uint32_t& phase) {
   using P = Pc<N>;
   constexpr int NP = P::NP, NT = P::NT, NF = P::NF, NTP = P::NTP, SQ = P::SQ, THR = 32 * W;
   static_assert(P::FB == (P::NNT - 1) * 512 + (20 * NTP - (P::NNT - 1) * 32) * 16, "fragment bytes");
   PcCell& x = pc_shared().x;
   auto& sred = pc_shared().red;
   unsigned char* const srec = pc_smem + pc_up(sizeof(PcShared));
-  __shared__ __align__(8) uint64_t sbar;
-  __shared__ int sCell, sAbort;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) {
-    mbar_init(&sbar, 1);
-    sAbort = 0;
-    pc_shared().ref = ref;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  uint32_t phase = 0;
   // next cell of this kernel's kind from the queue (index order, or the schedule's cost order)
   int* const queue = bt.work + (VISC ? 1 : 0);
   auto take = [&]() {
@@ -989,7 +979,7 @@ __global__ void __launch_bounds__(32 * W, MB) predictor_cells_kernel(const __gri
     __syncthreads();
     if (sAbort) {  // a copy that never completed: wait once more (bounded), then leave
       if (tid == 0) (void)mbar_wait_bounded(&sbar, phase & 1u);
-      return;
+      return false;
     }
     phase ^= 1u;
 
@@ -1031,6 +1021,31 @@ __global__ void __launch_bounds__(32 * W, MB) predictor_cells_kernel(const __gri
     // the next cell's bulk copies (async proxy) overwrite memory read and written here
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  return true;
+}
+
+// W warps per block, at least MB blocks per SM (register limit).  KINDS: 1 inviscid cells, 2 viscous cells, 3
+// both, the viscous ones, which take longer, first: in one launch the blocks go from one kind to the
+// other without waiting for the slowest (a pass of five steps, us, two launches and one: a batch
+// of P2 meshes of which some are limited 2,822 and 2,567, a limited 15^3 P3 mesh 2,982 and 2,848).
+template <int N, int W, int MB, int KINDS>
+__global__ void __launch_bounds__(32 * W, MB) predictor_cells_kernel(const __grid_constant__ Batch bt,
+                                                                     const __grid_constant__ PcRef ref, int diag,
+                                                                     int smem_bytes) {
+  __shared__ __align__(8) uint64_t sbar;
+  __shared__ int sCell, sAbort;
+  if (threadIdx.x == 0) {
+    mbar_init(&sbar, 1);
+    sAbort = 0;
+    pc_shared().ref = ref;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  uint32_t phase = 0;
+  if constexpr (KINDS & 2)
+    if (!predictor_cells<N, W, true>(bt, diag, smem_bytes, KINDS == 3, sbar, sCell, sAbort, phase)) return;
+  __syncthreads();
+  if constexpr (KINDS & 1)
+    (void)predictor_cells<N, W, false>(bt, diag, smem_bytes, KINDS == 3, sbar, sCell, sAbort, phase);
 }
 
 // ----------------------------------------------------------------------------------------

@@ -45,7 +45,7 @@ void pc_add_cell(int n, int s, int ns, PcCells* q);
 template <int N>
 cudaError_t pc_plan(int device, int n_sm, int64_t cells, bool viscous, const PcCells& q, PcPlan* out);
 
-// Launches the kernels of the kinds of cells that may be present.
+// Launches the kernel for the kinds of cells that may be present.
 template <int N>
 void pc_launch(const PcPlan& plan, const Batch& b, const PcRef& ref, bool inviscid, bool viscous, int diag, int n_sm,
                cudaStream_t st);
