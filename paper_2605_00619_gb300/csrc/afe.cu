@@ -323,8 +323,8 @@ afe_status dispatch_stage(const StepPlan& P, int stage) {
 
 afe_status stage(const StepPlan& P, int s) { return P.fp32 ? dispatch_stage<float>(P, s) : dispatch_stage<double>(P, s); }
 
-// limiter (if on) and the time step, all on the device
-afe_status enqueue_dt(const StepPlan& P, double dt) {
+// limiter (if on) and the time step, all on the device; in a step also its clock
+afe_status enqueue_dt(const StepPlan& P, double dt, int mode = afe::CFL_DT) {
   const int64_t C = P.b->cpre[P.b->nh];
   if (P.limiter) {
     afe::cell_means_kernel<<<(int)((C + 7) / 8), 256, 0, P.st>>>(*P.b);
@@ -333,8 +333,7 @@ afe_status enqueue_dt(const StepPlan& P, double dt) {
   if (dt > 0) {
     afe::set_dt_kernel<<<1, 64, 0, P.st>>>(*P.b, dt);
   } else {
-    afe::cfl_kernel<<<(int)((C * 32 + 255) / 256), 256, 0, P.st>>>(*P.b);
-    afe::dt_finalize_kernel<<<1, 64, 0, P.st>>>(*P.b);
+    afe::cfl_kernel<<<(int)((C * 32 + 255) / 256), 256, 0, P.st>>>(*P.b, mode);
   }
   return AFE_OK;
 }
@@ -351,21 +350,20 @@ afe_status record(const StepPlan& P) {
   return AFE_OK;
 }
 
-// kernels per step: begin + [means + limiter] + (set_dt | cfl + finalize) + predictor (FP64: one for
-// each kind of cell) + face + corrector + clock
-int launches_per_step(const StepPlan& P, double dt) {
+// kernels per step: [means + limiter] + (set_dt | cfl) + predictor (FP64: one for each kind of
+// cell) + face + corrector
+int launches_per_step(const StepPlan& P) {
   const int both = !P.fp32 && P.pd.blocks > 0 && P.inviscid && P.viscous;
   const int groups = P.cells && P.one ? (P.f32_tc ? 1 : 2) : 0;  // predictor and corrector once per form
-  return 1 + (P.limiter ? 2 : 0) + (dt > 0 ? 1 : 2) + 3 + both + groups + 1;
+  return (P.limiter ? 2 : 0) + 1 + 3 + both + groups;
 }
 
 afe_status enqueue_step(const StepPlan& P, double dt) {
   NvtxRange step_range("afe step");
-  afe::step_begin_kernel<<<1, 64, 0, P.st>>>(*P.b);
   AFE_TRY(record(P));
   {
     NvtxRange r("afe limiter + time step");
-    AFE_TRY(enqueue_dt(P, dt));
+    AFE_TRY(enqueue_dt(P, dt, afe::CFL_STEP));
   }
   AFE_TRY(record(P));
   {
@@ -383,14 +381,13 @@ afe_status enqueue_step(const StepPlan& P, double dt) {
     AFE_TRY(stage(P, 2));
   }
   AFE_TRY(record(P));
-  afe::advance_time_kernel<<<1, 64, 0, P.st>>>(*P.b);
   AFE_CUDA(cudaGetLastError());
   return AFE_OK;
 }
 
 afe_status enqueue_step(afe_mesh* m, double dt) {
   const StepPlan P = plan_of(m);
-  m->launches += launches_per_step(P, dt);
+  m->launches += launches_per_step(P);
   return enqueue_step(P, dt);
 }
 
@@ -723,7 +720,7 @@ afe_status afe_mesh_create(const afe_params* p, int64_t n_vertices, const double
   AFE_TRY(M->alloc(&d.tacc, 1));
   AFE_TRY(M->alloc(&d.maxbits, 1));
   AFE_TRY(M->alloc(&d.flags, afe::F_COUNT));
-  AFE_TRY(M->alloc(&d.work, 3));
+  AFE_TRY(M->alloc(&d.work, 4));
   AFE_TRY(M->alloc(&M->d_ref, 1));
 
   AFE_TRY(M->alloc(&M->d_totals_partial, (size_t)M->totals_blocks * 5));
@@ -773,6 +770,8 @@ afe_status afe_mesh_create(const afe_params* p, int64_t n_vertices, const double
   // FP64 set-up on the GPU: mass matrices, w_i, inverses
   NvtxRange setup_range("afe set-up: mass matrices and inverses");
   AFE_CUDA(cudaMemsetAsync(d.flags, 0, afe::F_COUNT * sizeof(int), M->stream));
+  AFE_CUDA(cudaMemsetAsync(d.maxbits, 0, sizeof(unsigned long long), M->stream));
+  AFE_CUDA(cudaMemsetAsync(d.work, 0, 4 * sizeof(int), M->stream));
   const int sgrid = (int)std::min<int64_t>(T.C, (int64_t)M->n_sm * 4);
   afe::assemble_mass_kernel<<<sgrid, 256, 0, M->stream>>>(d, M->d_ref);
   afe::invert_spd_kernel<<<(int)std::min<int64_t>(T.C, (int64_t)M->n_sm * 4), 256, 0, M->stream>>>(d);
@@ -879,7 +878,6 @@ afe_status afe_compute_dt(afe_mesh* m, double* dt) {
   if (!m || !dt) return fail(AFE_EINVAL, "NULL argument");
   const StepPlan P = plan_of(m);
   afe::flags_clear_kernel<<<1, 64, 0, P.st>>>(*P.b);
-  afe::step_begin_kernel<<<1, 64, 0, P.st>>>(*P.b);
   AFE_TRY(enqueue_dt(P, -1.0));
   AFE_CUDA(cudaMemcpyAsync(dt, m->dm.dt, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
   int flags[afe::F_COUNT];
@@ -892,7 +890,6 @@ afe_status afe_cfl_pieces(afe_mesh* m, int64_t n_cells, double* bracket_max, dou
   if (n_cells < 1 || n_cells > m->topo.C) return fail(AFE_EINVAL, "n_cells must be in 1..cells of the handle");
   const StepPlan P = plan_of(m);
   afe::flags_clear_kernel<<<1, 64, 0, P.st>>>(*P.b);
-  afe::step_begin_kernel<<<1, 64, 0, P.st>>>(*P.b);
   if (P.limiter) {  // the viscosity of every cell of the handle
     const int64_t C = m->topo.C;
     afe::cell_means_kernel<<<(int)((C + 7) / 8), 256, 0, P.st>>>(*P.b);
@@ -900,10 +897,11 @@ afe_status afe_cfl_pieces(afe_mesh* m, int64_t n_cells, double* bracket_max, dou
   }
   afe::Batch sub = m->self;  // the bracket over the first n_cells cells only
   sub.cpre[1] = n_cells;
-  afe::cfl_kernel<<<(int)((n_cells * 32 + 255) / 256), 256, 0, P.st>>>(sub);
+  afe::cfl_kernel<<<(int)((n_cells * 32 + 255) / 256), 256, 0, P.st>>>(sub, afe::CFL_BOUND);
   AFE_CUDA(cudaGetLastError());
   unsigned long long bits = 0;
   AFE_CUDA(cudaMemcpyAsync(&bits, m->dm.maxbits, sizeof(bits), cudaMemcpyDeviceToHost, m->stream));
+  AFE_CUDA(cudaMemsetAsync(m->dm.maxbits, 0, sizeof(bits), m->stream));  // as a step leaves it
   int flags[afe::F_COUNT];
   AFE_TRY(read_flags(m, flags));
   double bm;
@@ -1231,7 +1229,7 @@ afe_status afe_batch_create(afe_mesh* const* members, int n_members, void* cuda_
   if (dev != m0->device) return fail(AFE_EINVAL, "the current device is not the members' device");
   {
     void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, 3 * sizeof(int));
+    cudaError_t e = cudaMalloc(&p, 4 * sizeof(int));
     if (e != cudaSuccess) return fail(AFE_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
     b->d_work = (int*)p;
   }
@@ -1242,6 +1240,7 @@ afe_status afe_batch_create(afe_mesh* const* members, int n_members, void* cuda_
     AFE_CUDA(cudaStreamCreateWithFlags(&b->st, cudaStreamNonBlocking));
     b->own_stream = true;
   }
+  AFE_CUDA(cudaMemsetAsync(b->d_work, 0, 4 * sizeof(int), b->st));
   b->mem.assign(members, members + n_members);
   StepPlan& P = b->plan;
   P.b = &b->bt;
@@ -1303,7 +1302,7 @@ afe_status afe_batch_step_async(afe_batch* b, double dt, int nsteps, int use_gra
     AFE_CUDA(cudaGetLastError());
     b->launches += 1;
   }
-  const int per = launches_per_step(b->plan, dt);
+  const int per = launches_per_step(b->plan);
   if (use_graph) {
     if (!b->have_graph || b->graph_dt != dt) AFE_TRY(batch_capture(b, dt));
     for (int i = 0; i < nsteps; ++i) AFE_CUDA(cudaGraphLaunch(b->gexec, b->st));
@@ -1416,7 +1415,6 @@ afe_status autotune_impl(const std::string& sig, int order, bool tc_fits, int* w
   {
     const StepPlan P = plan();
     afe::flags_clear_kernel<<<1, 64, 0, st>>>(*P.b);
-    afe::step_begin_kernel<<<1, 64, 0, st>>>(*P.b);
     AFE_TRY(enqueue_dt(P, -1.0));
   }
   cudaEvent_t e0, e1;

@@ -69,7 +69,7 @@ struct DevMesh {
   double* tacc;   // device scalar: accumulated time
   unsigned long long* maxbits;
   int* flags;
-  int* work;      // work counters of the persistent predictors
+  int* work;      // work counters of the persistent predictors (three), blocks done of the CFL launch
   double* qbar_diag;
   // physics
   double gamma, Rgas, cv, cfl, m1, mu0, Pr, kappa0, tol, h_min;
@@ -88,7 +88,7 @@ struct Batch {
   int ring_cap;                  // FP32 predictor: most M_i^-1 ring stages (0: as many as fit)
   int narrow;                    // FP32 predictor: 1 = narrow right-hand-side chunks everywhere
   int pad;
-  int* work;                     // work counters of the persistent predictors (three)
+  int* work;                     // work counters of the persistent predictors (three), blocks done of the CFL launch
   const int32_t* order;          // global cells in the order the predictor takes them (NULL: index order)
   int64_t cpre[kMaxBatch + 1];   // prefix sums of the members' cells
   int64_t gpre[kMaxBatch + 1];   // prefix sums of the members' polygonal faces
@@ -364,13 +364,6 @@ static __global__ void flags_clear_kernel(const __grid_constant__ Batch bt) {
   }
 }
 
-// Start of a step: clear every member's CFL maximum and the shared work counters of the
-// persistent predictor.
-static __global__ void step_begin_kernel(const __grid_constant__ Batch bt) {
-  for (int h = threadIdx.x; h < bt.nh; h += blockDim.x) *bt.tab[h].maxbits = 0ull;
-  if (threadIdx.x < 3) bt.work[threadIdx.x] = 0;
-}
-
 // Sec. 4.5: cell means u_bar_i = w_i . u_i / |P_i| (w_i = M_i 1), one warp per cell, kept as what the
 // detector reads of them, once per cell instead of once per neighbour: density, velocity and
 // sound speed.
@@ -469,10 +462,7 @@ __device__ __forceinline__ float f32_head(double x, bool& ok) {
 // so far) can be the maximum and are evaluated in FP64.  A node whose interval is in doubt (an
 // exponent out of range, a pressure that is not positive beyond its error) always is, so that
 // the maximum and the report of inadmissible states are those of evaluating every node.
-static __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__ Batch bt) {
-  const int64_t gc = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (gc >= bt.cpre[bt.nh]) return;
+__device__ __forceinline__ void cfl_cell(const Batch& bt, int64_t gc, int lane) {
   const int hh = batch_find(bt.cpre, bt.nh, gc);
   const DevMesh& m = bt.tab[hh];
   const int64_t c = gc - bt.cpre[hh];
@@ -547,23 +537,45 @@ static __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__
   if (lane == 0) atomicMax(m.maxbits, (unsigned long long)__double_as_longlong(best));
 }
 
-// dt = CFL h_min / ((2N+1) max_bound) per member (Sec. 4.6)
-static __global__ void dt_finalize_kernel(const __grid_constant__ Batch bt) {
+// What a CFL launch does once the maximum is complete: nothing, dt, or dt and the step's clock.
+enum CflMode { CFL_BOUND = 0, CFL_DT = 1, CFL_STEP = 2 };
+
+// CFL bound of every cell; the last block to finish (bt.work[3] counts them) turns the members' maxima into
+// dt = CFL h_min / ((2N+1) max_bound) (Sec. 4.6), leaves the maxima zero for the next launch and
+// starts the step's clock.  Launches of their own for the start of a step, dt and the clock took 6 to
+// 11 us of a step (us per four steps, with them and here: 4^3 P1 541 and 495, 8^3 P2 732 and 709,
+// 24^3 P1 2,429 and 2,406; 32^3 P3 within 0.1 %).
+static __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__ Batch bt, int mode) {
+  const int64_t gc = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  if (gc < bt.cpre[bt.nh]) cfl_cell(bt, gc, threadIdx.x & 31);
+  if (mode == CFL_BOUND) return;
+  __shared__ int last;
+  __syncthreads();  // the block's maxima are folded
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(&bt.work[3], 1) == (int)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
   for (int h = threadIdx.x; h < bt.nh; h += blockDim.x) {
     const DevMesh& m = bt.tab[h];
-    const double mx = __longlong_as_double((long long)*m.maxbits);
+    const double mx = __longlong_as_double((long long)atomicExch(m.maxbits, 0ull));
     double dt = mx > 0.0 ? m.cfl * m.h_min / ((2 * m.N + 1) * mx) : 0.0;
     if (!(dt > 0.0)) atomicOr(&m.flags[F_NONFINITE], 4);
     *m.dt = dt;
+    if (mode == CFL_STEP) *m.tacc += dt;
   }
+  if (threadIdx.x < 4) bt.work[threadIdx.x] = 0;
 }
 
+// Start of a step of a given size.
 static __global__ void set_dt_kernel(const __grid_constant__ Batch bt, double dt) {
-  for (int h = threadIdx.x; h < bt.nh; h += blockDim.x) *bt.tab[h].dt = dt;
-}
-
-static __global__ void advance_time_kernel(const __grid_constant__ Batch bt) {
-  for (int h = threadIdx.x; h < bt.nh; h += blockDim.x) *bt.tab[h].tacc += *bt.tab[h].dt;
+  for (int h = threadIdx.x; h < bt.nh; h += blockDim.x) {
+    *bt.tab[h].dt = dt;
+    *bt.tab[h].tacc += dt;
+  }
+  if (threadIdx.x < 4) bt.work[threadIdx.x] = 0;
 }
 
 // ----------------------------------------------------------------------------------------
