@@ -879,17 +879,27 @@ __device__ __forceinline__ void pc_epilogue() {
 // All cells of a kind from the queue: VISC = false the cells without viscosity and heat conduction, VISC =
 // true the others; with both kinds present (`mixed`: the limiter's mu_i) each passes over the other's.
 // One path for both would spill the viscous fluxes' registers in the inviscid cells too.  False when a
-// bounded wait gave up.
+// bounded wait gave up.  Each kind has its own barrier and shared scalars: handed in by reference they
+// cost the eight-warp kernels a third (8^3 P2 131 us per launch against 97, 4^3 P1 50 against 39).
 template <int N, int W, bool VISC>
-__device__ __forceinline__ bool predictor_cells(const Batch& bt, int diag, int smem_bytes, bool mixed, uint64_t& sbar,
-                                                int& sCell, int& sAbort, uint32_t& phase) {
+__device__ __forceinline__ bool predictor_cells(const Batch& bt, const PcRef& ref, int diag, int smem_bytes,
+                                                bool mixed) {
   using P = Pc<N>;
   constexpr int NP = P::NP, NT = P::NT, NF = P::NF, NTP = P::NTP, SQ = P::SQ, THR = 32 * W;
   static_assert(P::FB == (P::NNT - 1) * 512 + (20 * NTP - (P::NNT - 1) * 32) * 16, "fragment bytes");
   PcCell& x = pc_shared().x;
   auto& sred = pc_shared().red;
   unsigned char* const srec = pc_smem + pc_up(sizeof(PcShared));
+  __shared__ __align__(8) uint64_t sbar;
+  __shared__ int sCell, sAbort;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) {
+    mbar_init(&sbar, 1);
+    sAbort = 0;
+    pc_shared().ref = ref;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  uint32_t phase = 0;
   // next cell of this kernel's kind from the queue (index order, or the schedule's cost order)
   int* const queue = bt.work + (VISC ? 1 : 0);
   auto take = [&]() {
@@ -1026,26 +1036,16 @@ __device__ __forceinline__ bool predictor_cells(const Batch& bt, int diag, int s
 
 // W warps per block, at least MB blocks per SM (register limit).  KINDS: 1 inviscid cells, 2 viscous cells, 3
 // both, the viscous ones, which take longer, first: in one launch the blocks go from one kind to the
-// other without waiting for the slowest (a pass of five steps, us, two launches and one: a batch
-// of P2 meshes of which some are limited 2,822 and 2,567, a limited 15^3 P3 mesh 2,982 and 2,848).
+// other without waiting for the slowest (us, two launches and one: four steps of a batch of
+// P2 meshes of which some are limited 2,822 and 2,567, two of a limited 15^3 P3 mesh 2,982 and 2,848).
 template <int N, int W, int MB, int KINDS>
 __global__ void __launch_bounds__(32 * W, MB) predictor_cells_kernel(const __grid_constant__ Batch bt,
                                                                      const __grid_constant__ PcRef ref, int diag,
                                                                      int smem_bytes) {
-  __shared__ __align__(8) uint64_t sbar;
-  __shared__ int sCell, sAbort;
-  if (threadIdx.x == 0) {
-    mbar_init(&sbar, 1);
-    sAbort = 0;
-    pc_shared().ref = ref;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  uint32_t phase = 0;
   if constexpr (KINDS & 2)
-    if (!predictor_cells<N, W, true>(bt, diag, smem_bytes, KINDS == 3, sbar, sCell, sAbort, phase)) return;
-  __syncthreads();
-  if constexpr (KINDS & 1)
-    (void)predictor_cells<N, W, false>(bt, diag, smem_bytes, KINDS == 3, sbar, sCell, sAbort, phase);
+    if (!predictor_cells<N, W, true>(bt, ref, diag, smem_bytes, KINDS == 3)) return;
+  if constexpr (KINDS == 3) __syncthreads();  // the last cell of one kind is done with what the next sets up
+  if constexpr (KINDS & 1) (void)predictor_cells<N, W, false>(bt, ref, diag, smem_bytes, KINDS == 3);
 }
 
 // ----------------------------------------------------------------------------------------
