@@ -41,11 +41,11 @@ METRIC = "DOF-updates/s per ADER-DG step"
 STABLE_CFL = {1: 0.3, 2: 0.2, 3: 0.15}
 PAPER_CFL = 0.3
 
-# DRAM bytes (read + write) of one predictor_f32_kernel<3> launch per cell of the density-wave
-# workload, from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of a 12^3 launch
-# of the current kernel; None until that capture exists.  The fixed-point iterations re-read
-# M_i^-1 from L2, so the traffic grows with the cells, not with the iterations.
-PREDICTOR_N3_DRAM_BYTES_PER_CELL = (812361984 + 40285696) / 1728
+# DRAM bytes (read + write) of one predictor_cells_kernel<3, 8, 2, 1> launch per cell of the
+# density-wave workload, from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of a
+# 16^3 launch (2.6 mean fixed-point iterations).  The cells in flight hold more of M_i^-1 than L2
+# keeps, so part of it is read again in every iteration.
+PREDICTOR_N3_DRAM_BYTES_PER_CELL = (2518260224 + 65393664) / 4096
 UNIT = "DOF-updates/s"
 
 
@@ -68,7 +68,7 @@ def _args():
     ap.add_argument("--no-autotune", dest="autotune", action="store_false",
                     help="keep the default predictor schedule instead of the autotuned one")
     ap.add_argument("--variant", type=int, default=0, choices=[0, 1],
-                    help="FP32 predictor's M_i^-1 apply: 0 mma.sync, 1 tcgen05 with tensor memory")
+                    help="FP32 predictor: 0 several cells per SM, 1 one block per SM with the apply on tcgen05")
     ap.add_argument("--serve", action="store_true", help="serving run: Poisson requests on small meshes")
     ap.add_argument("--study", choices=["convergence", "stokes", "vortex", "shock", "tgv"],
                     help="accuracy study instead of the throughput run")
@@ -540,12 +540,15 @@ def ours(args):
     # roofline of the dominant kernel (the predictor), by the pipes the design assigns
     pred_ms = r32["stage_ms"][1]
     out["roofline"] = predictor_roofline(r32["f_con"], r32["f_pw"], r32["abytes"], pred_ms, peaks)
-    out["roofline"]["kernel"] = f"predictor_f32_kernel<{args.order}>"
+    tc = (r32["schedule"] or {}).get("variant", args.variant)
+    out["roofline"]["kernel"] = (f"predictor_kernel<{args.order}, float>" if args.order > 3 else
+                                 f"predictor_f32_kernel<{args.order}, 1>" if tc else
+                                 f"predictor_cells_kernel<{args.order}>")
     out["roofline"]["traffic"] = None
     out["roofline"]["algorithmic_bytes_streamed_per_iteration"] = r32["abytes_streamed"]
     if args.order == 3 and args.workload == "density" and PREDICTOR_N3_DRAM_BYTES_PER_CELL:
         out["roofline"]["traffic"] = PREDICTOR_N3_DRAM_BYTES_PER_CELL * pm.n_cells
-        out["roofline"]["traffic_note"] = "ncu dram__bytes_read+write of a 12^3 launch, scaled by cells"
+        out["roofline"]["traffic_note"] = "ncu dram__bytes_read+write of a 16^3 launch, scaled by cells"
     out["config"]["cfl"] = cfl
     if rst is not None:
         v_st, ms_st = throughput(red, 5 * rst["n_nodes"], K, rst["ms"])

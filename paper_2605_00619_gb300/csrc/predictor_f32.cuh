@@ -1,4 +1,6 @@
-// FP32 space-time predictor for sm_103a (Sec. 4.3, Eqs. ADER-localCauchy, ader4, TAvectors).
+// FP32 space-time predictor for sm_103a (Sec. 4.3, Eqs. ADER-localCauchy, ader4, TAvectors), one block
+// per SM: the form for meshes whose largest cell leaves no room for two blocks per SM (otherwise
+// predictor_cells.cuh), and of the tcgen05 apply.
 //
 // One block of 512 threads per cell (persistent: blocks take cells from a work counter).
 // The cell's working set stays in shared memory for the whole fixed-point iteration:

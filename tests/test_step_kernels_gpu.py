@@ -66,3 +66,33 @@ def test_time_step_is_the_fp64_maximum(afe, N, scales):
         with pytest.raises(afe.AfeError):
             afe.afe_compute_dt(h)
     afe.afe_mesh_destroy(h)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_every_launch_of_the_bound_starts_from_zero(afe, precision):
+    """The CFL launch's last block sets dt and the clock and leaves the maximum at zero: neither a bound
+    read before a step nor a faster state stepped before reaches the next step's dt."""
+    pm = periodic_voronoi(3)
+    prec = afe.AFE_FP32 if precision == "fp32" else afe.AFE_FP64
+    p = afe.afe_default_params(1, precision=prec, picard_tol=1e-6 if precision == "fp32" else 1e-12, cfl=0.3)
+    h, g = afe.create_from_polymesh(pm, p), afe.create_from_polymesh(pm, p)
+    n = afe.afe_num_nodes(h)
+
+    def state(speed):
+        return states.primitive_to_conserved(np.ones(n), np.full((n, 3), speed), np.ones(n))
+
+    afe.afe_set_state(h, state(100.0))
+    fast = afe.afe_compute_dt(h)
+    afe.afe_cfl_pieces(h, 2)
+    afe.afe_set_state(h, state(1.0))
+    afe.afe_set_state(g, state(1.0))
+    slow = afe.afe_compute_dt(g)
+    assert slow > 10 * fast
+    afe.afe_step_async(h, 0.0, 1)
+    assert afe.afe_sync(h) == 0
+    assert afe.afe_get_stats(h).t == afe.afe_get_stats(h).dt == slow
+    afe.afe_step_async(h, slow / 2, 2)
+    assert afe.afe_sync(h) == 0
+    assert afe.afe_get_stats(h).t == pytest.approx(2 * slow, rel=2.0**-51)  # two roundings
+    for m in (h, g):
+        afe.afe_mesh_destroy(m)
