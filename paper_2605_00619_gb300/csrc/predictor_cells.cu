@@ -94,15 +94,18 @@ void pc_add_cell(int n, int s, int ns, PcCells* q) {
 
 template <int N>
 cudaError_t pc_plan(int device, int n_sm, int64_t cells, bool viscous, const PcCells& q, PcPlan* out) {
-  // the largest cell has to leave room for two blocks per SM (shape 1) in any case: meshes beyond
-  // that take the one-block form whatever their size
+  // meshes whose largest cell leaves no room for two blocks per SM take the one-block form, except at
+  // P3, where shape 0 gives a cell the whole SM: 32^3 mesh with cells of up to 539 nodes, step 18.1 ms in
+  // the one-block form, 12.6 ms here (a mesh that fits both shapes is 25 % slower in this one, so a
+  // batch with one such member still gains over the one-block form, but less)
   PcPlan many;
   cudaError_t e = plan_shape<N, 1>(device, q, &many);
   *out = many;
   // at P2 the viscous fluxes' registers make eight warps per cell the better shape for any number of
   // cells (21^3 Navier-Stokes: 1,345 us per launch against 1,565)
-  const bool wide = cells <= (int64_t)n_sm * PcShape<N, 0>::MB || (N == 2 && viscous);
-  if (e != cudaSuccess || !many.blocks || !wide) return e;
+  const bool wide = cells <= (int64_t)n_sm * PcShape<N, 0>::MB || (N == 2 && viscous) ||
+                    (N == 3 && !many.blocks);
+  if (e != cudaSuccess || !(many.blocks || N == 3) || !wide) return e;
   PcPlan few;
   e = plan_shape<N, 0>(device, q, &few);
   if (few.blocks) *out = few;
