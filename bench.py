@@ -42,11 +42,10 @@ STABLE_CFL = {1: 0.3, 2: 0.2, 3: 0.15}
 PAPER_CFL = 0.3
 
 # DRAM bytes (read + write) of one predictor launch per cell of the density-wave workload at N = 3,
-# from ncu captures (dram__bytes_read.sum + dram__bytes_write.sum): the form with several cells per
-# SM on a 16^3 launch (2.6 mean fixed-point iterations; the cells in flight hold more of M_i^-1 than
-# L2 keeps, so part of it is read again in every iteration), and the one-block form, which meshes
-# with larger cells take, on a 12^3 launch (M_i^-1 once).
-PREDICTOR_N3_DRAM_BYTES_PER_CELL = {"cells": (2518260224 + 65393664) / 4096, "one block": (812361984 + 40285696) / 1728}
+# from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of a 16^3 launch with two blocks
+# per SM (2.6 mean fixed-point iterations; the cells in flight hold more of M_i^-1 than L2 keeps, so
+# part of it is read again in every iteration): an upper value for one block per SM.
+PREDICTOR_N3_DRAM_BYTES_PER_CELL = (2518260224 + 65393664) / 4096
 UNIT = "DOF-updates/s"
 
 
@@ -487,8 +486,7 @@ def ours(args):
         _, iters, _, _ = afe.afe_get_diagnostics(h, pm.n_cells, qbar=False)
         rec = dict(status=[st, st2], ms=ms, wall=wall, stage_ms=(stage_ms / max(nst, 1)).tolist(), clocks=clk,
                    n_nodes=n_nodes, launches=launches, iters_mean=float(iters.mean()), iters_max=int(iters.max()),
-                   nonconverged=int(stats.nonconverged), dt=stats.dt, bytes=afe.afe_device_bytes(h), schedule=tune,
-                   predictor_smem=afe.afe_plan_info(h).smem_bytes)
+                   nonconverged=int(stats.nonconverged), dt=stats.dt, bytes=afe.afe_device_bytes(h), schedule=tune)
         rec["f_con"], rec["f_pw"], rec["abytes"], rec["abytes_streamed"] = predictor_model(
             node_ptr, pm.cell_subtet_ptr, iters, args.order, 4 if prec == afe.AFE_FP32 else 8)
         if e2e:
@@ -543,15 +541,14 @@ def ours(args):
     pred_ms = r32["stage_ms"][1]
     out["roofline"] = predictor_roofline(r32["f_con"], r32["f_pw"], r32["abytes"], pred_ms, peaks)
     tc = (r32["schedule"] or {}).get("variant", args.variant)
-    form = "cells" if r32["predictor_smem"] < 120 * 1024 and not tc else "one block"  # two blocks per SM or one
     out["roofline"]["kernel"] = (f"predictor_kernel<{args.order}, float>" if args.order > 3 else
-                                 f"predictor_cells_kernel<{args.order}>" if form == "cells" else
-                                 f"predictor_f32_kernel<{args.order}, {int(bool(tc))}>")
+                                 f"predictor_f32_kernel<{args.order}, 1>" if tc else
+                                 f"predictor_cells_kernel<{args.order}>")
     out["roofline"]["traffic"] = None
     out["roofline"]["algorithmic_bytes_streamed_per_iteration"] = r32["abytes_streamed"]
     if args.order == 3 and args.workload == "density" and not tc:
-        out["roofline"]["traffic"] = PREDICTOR_N3_DRAM_BYTES_PER_CELL[form] * pm.n_cells
-        out["roofline"]["traffic_note"] = "ncu dram__bytes_read+write of a smaller launch of this form, scaled by cells"
+        out["roofline"]["traffic"] = PREDICTOR_N3_DRAM_BYTES_PER_CELL * pm.n_cells
+        out["roofline"]["traffic_note"] = "ncu dram__bytes_read+write of a 16^3 launch, scaled by cells"
     out["config"]["cfl"] = cfl
     if rst is not None:
         v_st, ms_st = throughput(red, 5 * rst["n_nodes"], K, rst["ms"])
