@@ -472,7 +472,8 @@ __device__ __forceinline__ void cfl_cell(const Batch& bt, int64_t gc, int lane) 
   const double gam = m.gamma;
   const double visc =
       mu_i == 0.0 && kap == 0.0 ? 0.0 : fmax(4.0 * mu_i / 3.0, kap / m.cv) * (2.0 * (2 * m.N + 1) / m.cell_hv[c]);
-  const float vf = (float)visc, gf = (float)gam, gg = gf * (gf - 1.f);
+  // gamma (gamma - 1) is rounded once: near gamma = 1 the difference of rounded values is off by far more than kEps
+  const float vf = (float)visc, gg = (float)fma(gam, gam, -gam);
   // interval of a node's bound: relative errors are a few 2^-23 of each term, kEps covers them
   constexpr float kEps = 0x1p-18f;
   auto interval = [&](const double (&q)[5], float& lower) {

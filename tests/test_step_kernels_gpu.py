@@ -96,3 +96,34 @@ def test_every_launch_of_the_bound_starts_from_zero(afe, precision):
     assert afe.afe_get_stats(h).t == pytest.approx(2 * slow, rel=2.0**-51)  # two roundings
     for m in (h, g):
         afe.afe_mesh_destroy(m)
+
+
+# gamma - 1 far from a power of two and down to 1e-4, where gamma in FP32 has lost it to 4 digits
+@pytest.mark.parametrize("gamma", [1.0001, 1.001, 1.005, 5.0 / 3.0])
+@pytest.mark.parametrize("first", ["hot", "fast"])
+def test_time_step_over_gamma_and_kinds_of_nodes(afe, gamma, first):
+    """Nodes whose bound is nearly all sound speed beside nodes whose bound is nearly all velocity, one kind
+    ahead of the other by 1e-5: whatever their order, dt is that of the largest FP64 bound, to the rounding of
+    its operations (a few 2^-53; the bar is that of the uniform states above), and the same in every run."""
+    pm = periodic_voronoi(3)
+    h = afe.create_from_polymesh(pm, afe.afe_default_params(2, precision=afe.AFE_FP32, picard_tol=1e-6, gamma=gamma))
+    n = afe.afe_num_nodes(h)
+    rng = np.random.default_rng(11)
+    one = states.primitive_to_conserved(np.ones(n), np.zeros((n, 3)), np.ones(n), gamma)
+    afe.afe_set_state(h, one)
+    ref = afe.afe_compute_dt(h) * _bound(one, gamma)
+    for _ in range(3):
+        hot = rng.random(n) < 0.5
+        speed = np.where(hot, 1.0, 1.0 - 1e-5) if first == "hot" else np.where(hot, 1.0 - 1e-5, 1.0)
+        speed *= 1 - 1e-6 * rng.random(n)
+        mach = np.where(hot, 1e-3, 20.0)  # |v| / c
+        c = speed / (1 + mach)
+        d = rng.normal(size=(n, 3))
+        rho = rng.uniform(0.5, 2, n)
+        u = states.primitive_to_conserved(rho, (mach * c / np.linalg.norm(d, axis=1))[:, None] * d, rho * c * c / gamma,
+                                          gamma)
+        afe.afe_set_state(h, u)
+        dts = {afe.afe_compute_dt(h) for _ in range(5)}
+        assert len(dts) == 1
+        assert abs(dts.pop() * _bound(u, gamma) / ref - 1) <= 1e-12
+    afe.afe_mesh_destroy(h)
