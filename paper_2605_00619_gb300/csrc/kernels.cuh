@@ -474,6 +474,7 @@ __device__ __forceinline__ void cfl_cell(const Batch& bt, int64_t gc, int lane) 
       mu_i == 0.0 && kap == 0.0 ? 0.0 : fmax(4.0 * mu_i / 3.0, kap / m.cv) * (2.0 * (2 * m.N + 1) / m.cell_hv[c]);
   // gamma (gamma - 1) is rounded once: near gamma = 1 the difference of rounded values is off by far more than kEps
   const float vf = (float)visc, gg = (float)fma(gam, gam, -gam);
+  const bool vis_ok = vf >= 0x1p-120f || visc == 0.0;  // else too small for FP32
   // interval of a node's bound: relative errors are a few 2^-23 of each term, kEps covers them
   constexpr float kEps = 0x1p-18f;
   auto interval = [&](const double (&q)[5], float& lower) {
@@ -484,8 +485,10 @@ __device__ __forceinline__ void cfl_cell(const Batch& bt, int64_t gc, int lane) 
     const float c2 = gg * ir * (e - 0.5f * m2), err = kEps * gg * ir * (fabsf(e) + m2);
     const float s = sqrtf(m2 * ir) + vf * ir;
     const float lo = sqrtf(c2 - err), up = s + sqrtf(c2 + err);
-    // rho > 0, a pressure that is positive whatever the error, everything in range
-    ok = ok && r > 0.f && c2 > err && up < 1e30f && s >= 0.f;
+    // rho > 0, a pressure that is positive whatever the error, everything in range.  The squares of the
+    // momentum lose up to 2^-148 to underflow, 2^-74 / rho of |v|: below 2^-25 c when gamma (gamma - 1)
+    // rho E > 2^-80 and the pressure passes its test (c^2 > 2^-18 gamma (gamma - 1) E / rho).
+    ok = ok && r > 0.f && c2 > err && c2 > 0x1p-100f && gg * (e * r) > 0x1p-80f && vis_ok && up < 1e30f && s >= 0.f;
     lower = ok ? (s + lo) * (1.f - kEps) : 0.f;
     return ok ? up * (1.f + kEps) : __int_as_float(0x7f800000);
   };

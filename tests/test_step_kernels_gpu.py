@@ -127,3 +127,28 @@ def test_time_step_over_gamma_and_kinds_of_nodes(afe, gamma, first):
         assert len(dts) == 1
         assert abs(dts.pop() * _bound(u, gamma) / ref - 1) <= 1e-12
     afe.afe_mesh_destroy(h)
+
+
+# values whose products leave FP32's range though they themselves do not
+@pytest.mark.parametrize("rho,c", [(1e-19, 1.0), (1e-21, 1.0), (1e-24, 1.0), (1e-24, 1e5), (1e12, 1e-21), (1e25, 1e-27)])
+def test_time_step_of_small_products(afe, rho, c):
+    """Fast cold nodes (|v| = 3 c) among hot ones at rest (c' = 2 c), densities down to 1e-24: dt is that of the
+    largest FP64 bound, to the rounding of its operations (the pressure is a tenth of the total energy or
+    more: a few 2^-52)."""
+    pm = periodic_voronoi(3)
+    h = afe.create_from_polymesh(pm, afe.afe_default_params(2, precision=afe.AFE_FP32, picard_tol=1e-6))
+    n = afe.afe_num_nodes(h)
+    rng = np.random.default_rng(13)
+    one = states.primitive_to_conserved(np.ones(n), np.zeros((n, 3)), np.ones(n))
+    afe.afe_set_state(h, one)
+    ref = afe.afe_compute_dt(h) * _bound(one)
+    for _ in range(3):
+        hot = rng.random(n) < 0.5
+        d = rng.normal(size=(n, 3))
+        d /= np.linalg.norm(d, axis=1)[:, None]
+        cs = np.where(hot, 2.0, 1.0) * c * rng.uniform(0.9, 1, n)
+        r = rho * rng.uniform(0.5, 2, n)
+        u = states.primitive_to_conserved(r, np.where(hot, 0.0, 3.0 * c)[:, None] * d, r * cs * cs / 1.4)
+        afe.afe_set_state(h, u)
+        assert abs(afe.afe_compute_dt(h) * _bound(u) / ref - 1) <= 1e-12
+    afe.afe_mesh_destroy(h)
