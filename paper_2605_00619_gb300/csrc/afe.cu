@@ -794,6 +794,8 @@ afe_status afe_mesh_create(const afe_params* p, int64_t n_vertices, const double
   } else {
     AFE_TRY(set_up_f64(M, nminv));
   }
+  // the set-up kernels end before the call returns: the handle's next work may be on another stream
+  AFE_CUDA(cudaStreamSynchronize(M->stream));
   sync_self(M);
   *out = m.release();
   return AFE_OK;

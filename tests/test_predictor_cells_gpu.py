@@ -104,3 +104,29 @@ def test_a_batch_keeps_every_members_form(afe):
         np.testing.assert_array_equal(afe.afe_get_state(m), afe.afe_get_state(h))
     for h in alone + mem:
         afe.afe_mesh_destroy(h)
+
+
+@pytest.mark.parametrize("bits", [32, 64])
+@pytest.mark.parametrize("N", [1, 3])
+def test_a_new_handle_is_complete_on_any_stream(afe, N, bits):
+    """Creation leaves no set-up work behind on its stream: a handle moved to another stream at once steps
+    like one that was waited for, bit for bit."""
+    import torch
+    pm = periodic_voronoi(6)
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    p = afe.afe_default_params(N, precision=afe.AFE_FP32 if bits == 32 else afe.AFE_FP64,
+                               picard_tol=1e-6 if bits == 32 else 1e-12, cfl=0.1)
+    ref = afe.create_from_polymesh(pm, p)
+    u = states.density_wave(afe.afe_get_node_coords(ref))
+    du = torch.from_numpy(u).cuda()
+    torch.cuda.synchronize()
+    afe.afe_set_state(ref, u)
+    assert afe.afe_step(ref, 0.0) == 0
+    for _ in range(3):
+        h = afe.create_from_polymesh(pm, p, a.cuda_stream)
+        afe.afe_set_stream(h, b.cuda_stream)
+        afe.afe_set_state_device(h, du.data_ptr())
+        assert afe.afe_step(h, 0.0) == 0
+        np.testing.assert_array_equal(afe.afe_get_state(h), afe.afe_get_state(ref))
+        afe.afe_mesh_destroy(h)
+    afe.afe_mesh_destroy(ref)
