@@ -131,23 +131,21 @@ template void pc_add_cell<AFE_ORDER>(int, int, int, PcCells*);
 template void pc_launch<AFE_ORDER>(const PcPlan&, const Batch&, const PcRef&, bool, bool, int, int, cudaStream_t);
 
 #if AFE_ORDER == 1
-// The split copy of M_i^-1 (see minv_split_words), from its FP32 rows; one block per cell at a time.
+// The split copy of M_i^-1 (see minv_split_words), from its FP32 rows; one block per cell at a time.  Row
+// exponent p_i: M_ii 2^(2 p_i) in [1/4, 1); entry (i, j) is kept as 2^(13 + p_i + p_j) M_ij, below 2^13
+// in magnitude because the matrix is positive definite.  One power of two for the whole cell would leave
+// the rows of its large sub-tets the bits that FP16's range has left below those of its smallest one.
 static __global__ void __launch_bounds__(256) split_minv_kernel(DevMesh m) {
-  __shared__ uint32_t smax;
   for (int64_t c = blockIdx.x; c < m.C; c += gridDim.x) {
     const int n = (int)(m.node_ptr[c + 1] - m.node_ptr[c]), LD = minv_ld(n);
     const float* A = m.minv32 + m.minv_ptr[c];
     uint32_t* out = m.m16 + minv_split_start(m.minv_ptr[c], m.node_ptr[c], c);
-    if (threadIdx.x == 0) smax = 0;
-    __syncthreads();
-    uint32_t mx = 0;
-    for (int e = threadIdx.x; e < n * LD; e += blockDim.x) mx = max(mx, __float_as_uint(fabsf(A[e])));
-    mx = __reduce_max_sync(0xffffffffu, mx);
-    if ((threadIdx.x & 31) == 0) atomicMax(&smax, mx);
-    __syncthreads();
-    const int e = f16_scale_exp(smax);
-    const float s = __uint_as_float((uint32_t)e << 23);
-    if (threadIdx.x == 0) out[0] = (uint32_t)(254 - e) << 23;
+    auto expo = [&](int i) {
+      const int e = (int)(__float_as_uint(A[(int64_t)i * LD + i]) >> 23 & 255u) - 126;  // M_ii < 2^e
+      return -((e + 1) >> 1);
+    };
+    for (int i = threadIdx.x; i < 4 * minv_split_head(n); i += blockDim.x)
+      reinterpret_cast<int8_t*>(out)[i] = (int8_t)(i < n ? expo(i) : 0);
     const int nt = (n + 15) / 16;
     // word (tile, part, lane, i): entries (row, col), (row, col + 1) with row = 16 ti + lane / 4 + 8 (i & 1),
     // col = 16 tj + 2 (lane & 3) + 8 (i >> 1)
@@ -158,16 +156,17 @@ static __global__ void __launch_bounds__(256) split_minv_kernel(DevMesh m) {
       uint32_t hi = 0, lo = 0;
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
-        const float x = (row < n && col + q < n) ? s * A[(int64_t)row * LD + col + q] : 0.f;
+        const float x = (row < n && col + q < n)
+                            ? (A[(int64_t)row * LD + col + q] * pow2f(expo(row))) * pow2f(expo(col + q) + 13)
+                            : 0.f;
         const __half h = __float2half_rn(x), l = __float2half_rn(x - __half2float(h));
         hi |= (uint32_t)__half_as_ushort(h) << (16 * q);
         lo |= (uint32_t)__half_as_ushort(l) << (16 * q);
       }
-      uint32_t* o = out + 32 + tri_tile(ti, tj) * 256 + lane * 4 + i;
+      uint32_t* o = out + minv_split_head(n) + tri_tile(ti, tj) * 256 + lane * 4 + i;
       o[0] = hi;
       o[128] = lo;
     }
-    __syncthreads();
   }
 }
 

@@ -6,6 +6,7 @@
 // serial tails are covered by another cell's arithmetic.  What the cell needs on chip:
 //   srec  [S][REC]       its packed sub-tet records (adj(J), det J, node ids)
 //   sgat                 its node -> (sub-tet, local node) lists, 16 bits per entry
+//   sexp  [N_i]          row exponents of M_i^-1, 8 bits
 //   suh   [N_i][5]       u^, the state at t^n
 //   sq    [N_i][5][NTP]  space-time coefficients q, time innermost (one vector load per variable)
 // and a region that phase 1 uses for the pre-contracted fluxes of a chunk of sub-tets and
@@ -22,15 +23,17 @@
 //      the thread that owns the node (no atomics; the order does not depend on the chunks).
 //      The first iteration starts from q^0 = u^ at every time node: one time slice serves all.
 //   2. Y = M_i^-1 RHS on the tensor cores.  M_i^-1 is kept, beside its FP32 rows, as pairs of
-//      FP16 values hi + lo = s M_i^-1 (s a power of two per cell, both parts rounded to nearest:
-//      22 bits and a sign, where the TF32 head and tail taken by truncation carry 21) in the
+//      FP16 values hi + lo of M_i^-1 scaled to a unit diagonal by powers of two per row and column (both
+//      parts rounded to nearest: 22 bits and a sign, where the TF32 head and tail taken by truncation
+//      carry 21) in the
 //      register layout of mma.sync.m16n8k16, so that a warp streams its own 16-row tiles from L2
 //      straight into registers, 1 KB per tile and 16 columns, with no staging in shared memory
 //      and no splitting arithmetic.  M_i^-1 is symmetric: only the tiles of its lower triangle are
 //      kept (a tile above the diagonal is the mirrored one, transposed in registers), which
-//      halves what the cells in flight hold in L2 between iterations and what comes from HBM.  The right-hand side is split the same way with a power of
-//      two per variable (taken from its maximum over the cell).  The products hi hi + lo hi +
-//      hi lo are accumulated in FP32.
+//      halves what the cells in flight hold in L2 between iterations and what comes from HBM.  The
+//      right-hand side is split the same way, its rows scaled by the inverse powers, then with a power
+//      of two per variable (taken from its maximum over the cell).  The products hi hi + lo hi + hi lo
+//      are accumulated in FP32.
 //      q^{r+1}[n,s] = u^[n] - dt sum_t K1t^-1[s,t] w_t Y[n,t] straight from the accumulators.
 // Epilogue: vol, q_bar and F_bar . n as the FP64 kernel; F_bar . n comes from the volume term's
 // adj(J)_d . F_bar, because the rows of adj(J) are the area normals of the sub-tet's faces.
@@ -150,11 +153,14 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], const uint4& a, uint32_t 
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
 }
-// Biased exponent of the power of two that takes a maximum of magnitude x into [2^13, 2^14).
+// Biased exponent of the power of two that takes a maximum of magnitude x into [2^13, 2^14) (at most 2^126, so
+// that its inverse is a normal number too).
 __host__ __device__ __forceinline__ int f16_scale_exp(uint32_t bits) {
   const int e = 267 - (int)(bits >> 23 & 255u);
-  return e > 254 ? 254 : e;
+  return e > 253 ? 253 : e;
 }
+// 2^e, -126 <= e <= 127.
+__device__ __forceinline__ float pow2f(int e) { return __uint_as_float((uint32_t)(127 + e) << 23); }
 
 // adj(J)_d . F_e at one state, Euler: out[d][v].
 __device__ __forceinline__ void contravariant_flux(const float (&Q)[5], const float (&g)[9], float gm1,
@@ -182,9 +188,9 @@ struct PcCell {
   const uint32_t* m16;    // fragments of the split M_i^-1
   int64_t c, n0, s0;
   int Ni, S, ns, nks, nlong, slots, room;
-  uint32_t o_gat, o_inc, o_uh, o_q, o_region;  // bytes from the start of dynamic shared memory
-  float dt, gam, gm1, mu, kap, isc;     // isc = 1 / (power of two of M_i^-1)
-  float isv[5];                         // dt / (power of two of the right-hand side), per variable
+  uint32_t o_gat, o_inc, o_exp, o_uh, o_q, o_region;  // bytes from the start of dynamic shared memory
+  float dt, gam, gm1, mu, kap;
+  float isv[5];                         // 1 / (power of two of the right-hand side), per variable
 };
 
 // At the start of dynamic shared memory (every function names that memory itself, so that the
@@ -200,8 +206,8 @@ __device__ __forceinline__ PcShared& pc_shared() { return *reinterpret_cast<PcSh
 // Bytes of the fixed part for a cell of n nodes and s sub-tets, and of its smallest region.
 template <int N>
 __host__ __device__ constexpr size_t pc_fixed(int n, int s, int ns) {
-  return pc_up(sizeof(PcShared)) + pc_up((size_t)s * Pc<N>::REC) + pc_up(gat_bytes(n, s, ns, Pc<N>::NP, Pc<N>::NF)) + pc_up((size_t)n * 20) +
-         pc_up((size_t)n * Pc<N>::SQ * 4);
+  return pc_up(sizeof(PcShared)) + pc_up((size_t)s * Pc<N>::REC) + pc_up(gat_bytes(n, s, ns, Pc<N>::NP, Pc<N>::NF)) +
+         (size_t)minv_split_head(n) * 4 + pc_up((size_t)n * 20) + pc_up((size_t)n * Pc<N>::SQ * 4);
 }
 // Gather slots of a cell at most (a warp shares at most one long list).
 __host__ __device__ constexpr int pc_slots(int n, int thr) { return n + 31 * (thr / 32 < kMaxLong ? thr / 32 : kMaxLong); }
@@ -221,12 +227,14 @@ template <int N>
 struct PcView {  // pointers into the cell's shared memory
   const unsigned char* srec;
   const uint16_t *slist, *sinc;
+  const int8_t* sexp;
   const float* suh;
   float *sq, *region;
   __device__ __forceinline__ PcView()
       : srec(pc_smem + pc_up(sizeof(PcShared))),
         slist(reinterpret_cast<const uint16_t*>(pc_smem + pc_shared().x.o_gat)),
         sinc(reinterpret_cast<const uint16_t*>(pc_smem + pc_shared().x.o_inc)),
+        sexp(reinterpret_cast<const int8_t*>(pc_smem + pc_shared().x.o_exp)),
         suh(reinterpret_cast<const float*>(pc_smem + pc_shared().x.o_uh)),
         sq(reinterpret_cast<float*>(pc_smem + pc_shared().x.o_q)),
         region(reinterpret_cast<float*>(pc_smem + pc_shared().x.o_region)) {}
@@ -472,8 +480,16 @@ __device__ __forceinline__ void pc_rhs(bool first) {
         for (int o = 16; o > 0; o >>= 1) racc[v][t] += __shfl_xor_sync(0xffffffffu, racc[v][t], o);
       }
   }
-  // the right-hand side's power of two per variable.  The fragments overwrite the region up to
-  // the sums of the third slots: those of the second slots are read before the barrier.
+  // row scaling, then the right-hand side's power of two per variable.  The fragments overwrite the
+  // region up to the sums of the third slots: those of the second slots are read before the barrier.
+  auto scale = [&](int n, float (&a)[5][NTP]) {
+    const float f = pow2f(-(int)V.sexp[n]);
+#pragma unroll
+    for (int v = 0; v < 5; ++v)
+#pragma unroll
+      for (int t = 0; t < NTP; ++t) a[v][t] *= f;
+  };
+  if (node0 >= 0) scale(node0, racc);
   float a[5][NTP];
 #pragma unroll
   for (int v = 0; v < 5; ++v)
@@ -484,6 +500,7 @@ __device__ __forceinline__ void pc_rhs(bool first) {
   for (int v = 0; v < 5; ++v) omax[v] = 0.f;
   for (int i = tid + (x.slots - 1 - tid) / THR * THR; i >= THR; i -= THR) {  // the second slot last
     load_sums(reinterpret_cast<const float4*>(sover + (i - THR) * SQ), a);
+    scale(V.slist[1 + 2 * (i - 31 * x.nlong)], a);
 #pragma unroll
     for (int v = 0; v < 5; ++v)
 #pragma unroll
@@ -507,7 +524,7 @@ __device__ __forceinline__ void pc_rhs(bool first) {
     for (int w = 1; w < W; ++w) y = fmaxf(y, sred[v][w]);
     const int e = f16_scale_exp(__float_as_uint(y));
     sc[v] = __uint_as_float((uint32_t)e << 23);
-    if (tid == 0) x.isv[v] = __uint_as_float((uint32_t)(254 - e) << 23) * x.dt;
+    if (tid == 0) x.isv[v] = __uint_as_float((uint32_t)(254 - e) << 23);
   }
   // fragments: entry (row n, column col) at 16-row step n / 16, column tile col / 8, lane
   // (col & 7) 4 + ((n & 7) >> 1), words {b0 hi, b1 hi, b0 lo, b1 lo}, b = (n & 15) >> 3
@@ -537,7 +554,10 @@ __device__ __forceinline__ void pc_rhs(bool first) {
     i += THR;
     if (i >= x.slots) break;
     n = V.slist[1 + 2 * (i - 31 * x.nlong)];
-    if (i >= 2 * THR) load_sums(reinterpret_cast<const float4*>(sover + (i - THR) * SQ), a);
+    if (i >= 2 * THR) {
+      load_sums(reinterpret_cast<const float4*>(sover + (i - THR) * SQ), a);
+      scale(n, a);
+    }
 #pragma unroll
     for (int v = 0; v < 5; ++v)
 #pragma unroll
@@ -569,10 +589,11 @@ __device__ __forceinline__ float2 pc_apply() {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int Ni = x.Ni, nks = x.nks;
   const unsigned char* const frag = reinterpret_cast<const unsigned char*>(V.region) + lane * 16;
-  const float isc = x.isc;
   float res = 0.f, qmax = 0.f;
+  // dt over the scaling of row n of the product
+  auto unscale = [&](int n) { return pow2f(-(int)V.sexp[n] - 13) * x.dt; };
   // q^{r+1} of (node n, variable v) from its NT values of M_i^-1 RHS
-  auto update = [&](int n, int v, float (&y)[NTP]) {
+  auto update = [&](int n, int v, float (&y)[NTP], float isc) {
     const float si = x.isv[v], uh = V.suh[n * 5 + v];
     float old[NTP], z[NTP];
     float* qp = V.sq + n * SQ + v * NTP;
@@ -656,6 +677,7 @@ __device__ __forceinline__ float2 pc_apply() {
     asm volatile("" ::: "memory");  // the update's constants are loaded behind the products, not held through them
     const int gq = lane >> 2, tq = lane & 3;
     const int row = mt * 16 + gq;
+    const float is0 = unscale(row), is1 = unscale(row + 8);
       if constexpr (FIRST) {
         // columns 2 tq, 2 tq + 1 are variables
 #pragma unroll
@@ -663,7 +685,7 @@ __device__ __forceinline__ float2 pc_apply() {
           const int v = 2 * tq + (i & 1), n = row + (i >> 1) * 8;
           float y[NTP];
           y[0] = acc[0][i];
-          if (v < 5 && n < Ni) update(n, v, y);
+          if (v < 5 && n < Ni) update(n, v, y, i >> 1 ? is1 : is0);
         }
       } else if constexpr (NTP == 2) {
 #pragma unroll
@@ -672,7 +694,7 @@ __device__ __forceinline__ float2 pc_apply() {
           for (int h = 0; h < 2; ++h) {
             const int v = nt * 4 + tq, n = row + 8 * h;
             float y[2] = {acc[nt][2 * h], acc[nt][2 * h + 1]};
-            if (v < 5 && n < Ni) update(n, v, y);
+            if (v < 5 && n < Ni) update(n, v, y, h ? is1 : is0);
           }
       } else {
         // a lane pair holds the four time slices of rows g and g + 8: the even lane takes
@@ -685,7 +707,7 @@ __device__ __forceinline__ float2 pc_apply() {
           const float r0 = __shfl_xor_sync(0xffffffffu, s0, 1), r1 = __shfl_xor_sync(0xffffffffu, s1, 1);
           const int v = nt * 2 + (tq >> 1), n = row + (odd ? 8 : 0);
           float y[4] = {odd ? r0 : d[0], odd ? r1 : d[1], odd ? d[2] : r0, odd ? d[3] : r1};
-          if (v < 5 && n < Ni) update(n, v, y);
+          if (v < 5 && n < Ni) update(n, v, y, odd ? is1 : is0);
         }
       }
   }
@@ -934,7 +956,9 @@ __device__ __forceinline__ bool predictor_cells(const Batch& bt, const PcRef& re
       const int ns = (int)(m.slot_ptr[c + 1] - s0);
       const uint32_t* const m16 = m.m16 + minv_split_start(m.minv_ptr[c], n0, c);
       const uint32_t gbytes = (uint32_t)gat_bytes(Ni, S, ns, NP, NF);
-      const uint32_t o_gat = (uint32_t)(pc_up(sizeof(PcShared)) + pc_up((size_t)S * P::REC)), o_uh = o_gat + (uint32_t)pc_up(gbytes),
+      const int head = minv_split_head(Ni);
+      const uint32_t o_gat = (uint32_t)(pc_up(sizeof(PcShared)) + pc_up((size_t)S * P::REC)),
+                     o_exp = o_gat + (uint32_t)pc_up(gbytes), o_uh = o_exp + head * 4,
                      o_q = o_uh + (uint32_t)pc_up((size_t)Ni * 20), o_region = o_q + (uint32_t)pc_up((size_t)Ni * SQ * 4);
       // records and gather block by two bulk copies; meanwhile u^, and M_i^-1 on its way into L2
       if (tid == 0) {
@@ -945,7 +969,7 @@ __device__ __forceinline__ bool predictor_cells(const Batch& bt, const PcRef& re
         bulk_g2s(pc_smem + o_gat, m.gat + gat_start(n0, kbase, s0, c, NP, NF), gbytes, &sbar);
         const double mu = m.mu[c];
         x.m = &m;
-        x.m16 = m16 + 32;
+        x.m16 = m16 + head;
         x.c = c;
         x.n0 = n0;
         x.s0 = s0;
@@ -956,6 +980,7 @@ __device__ __forceinline__ bool predictor_cells(const Batch& bt, const PcRef& re
         x.room = smem_bytes - (int)o_region;
         x.o_gat = o_gat;
         x.o_inc = o_gat + (uint32_t)gat_up(2 * (size_t)(2 * Ni + 3));
+        x.o_exp = o_exp;
         x.o_uh = o_uh;
         x.o_q = o_q;
         x.o_region = o_region;
@@ -964,16 +989,16 @@ __device__ __forceinline__ bool predictor_cells(const Batch& bt, const PcRef& re
         x.gm1 = x.gam - 1.f;
         x.mu = (float)mu;
         x.kap = (float)cell_kappa(m, mu);
-        x.isc = __uint_as_float(m16[0]);
       }
       if (warp == W - 1) {
-        const uint32_t bytes = (uint32_t)(minv_split_words(Ni) - 32) * 4u;
+        const uint32_t bytes = (uint32_t)(minv_split_words(Ni) - head) * 4u;
         for (uint32_t o = lane * 16384u; o < bytes; o += 32 * 16384u)
           asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(
-                           reinterpret_cast<const unsigned char*>(m16 + 32) + o),
+                           reinterpret_cast<const unsigned char*>(m16 + head) + o),
                        "r"(min(16384u, bytes - o))
                        : "memory");
       }
+      for (int e = tid; e < head; e += THR) reinterpret_cast<uint32_t*>(pc_smem + o_exp)[e] = m16[e];
       float* const suh = reinterpret_cast<float*>(pc_smem + o_uh);
       for (int e = tid; e < 5 * Ni; e += THR) suh[e] = (float)m.u[n0 * 5 + e];
       if (tid == 0) {
@@ -1086,14 +1111,16 @@ __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) correc
   const int Ni = (int)(m.node_ptr[c + 1] - n0), ns = (int)(m.slot_ptr[c + 1] - s0), nks = (Ni + 15) / 16;
   const uint32_t* const m16 = m.m16 + minv_split_start(m.minv_ptr[c], n0, c);
   unsigned char* const frag = pc_smem;                                   // [nks][320] split right-hand side
-  float* const sr = reinterpret_cast<float*>(pc_smem + nks * 320);       // [N_i][5] r, then du
+  float* const sr = reinterpret_cast<float*>(pc_smem + nks * 320);       // [N_i][5] r (rows scaled), then du
   float* const sf = sr + ((Ni * 5 + 3) & ~3);                            // [ns][NF][5] face integrals
   const float* const vol = (const float*)m.vol;
   const float* const sG = (const float*)m.slot_G;
+  const int8_t* const ex = reinterpret_cast<const int8_t*>(m16);
+  const uint32_t* const tiles = m16 + minv_split_head(Ni);
   if (warp == W - 1) {  // M_i^-1 on its way into L2
-    const uint32_t bytes = (uint32_t)(minv_split_words(Ni) - 32) * 4u;
+    const uint32_t bytes = (uint32_t)(minv_split_words(Ni) - minv_split_head(Ni)) * 4u;
     for (uint32_t o = lane * 8192u; o < bytes; o += 32 * 8192u)
-      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<const unsigned char*>(m16 + 32) + o),
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<const unsigned char*>(tiles) + o),
                    "r"(min(8192u, bytes - o))
                    : "memory");
   }
@@ -1126,6 +1153,7 @@ __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) correc
     float acc[5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) acc[v] = vol[(n0 + n) * 5 + v];
+    const float f0 = pow2f(-(int)ex[n]);
     const int64_t p1 = m.finc_ptr[n0 + n + 1];
     for (int64_t p = m.finc_ptr[n0 + n]; p < p1; ++p) {
       const uint32_t w = m.finc[p];
@@ -1135,6 +1163,7 @@ __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) correc
     }
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
+      acc[v] *= f0;
       sr[n * 5 + v] = acc[v];
       mx[v] = fmaxf(mx[v], fabsf(acc[v]));
     }
@@ -1147,7 +1176,6 @@ __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) correc
   __syncthreads();
   // split right-hand side in fragment order, a power of two per variable
   float sc[5], isc[5];
-  const float is0 = __uint_as_float(m16[0]);
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
     float x = smax[v][0];
@@ -1170,7 +1198,7 @@ __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) correc
   __syncthreads();
   for (int mt = warp; mt < nks; mt += W) {
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    const uint32_t* const a0 = m16 + 32 + lane * 4;
+    const uint32_t* const a0 = tiles + lane * 4;
     uint4 ah[DP], al[DP];
     auto load = [&](int s, int ks) {
       const uint32_t* t = a0 + tri_tile(mt, min(ks, nks - 1)) * 256;
@@ -1209,7 +1237,7 @@ __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) correc
 #pragma unroll
         for (int q = 1; q < 5; ++q)
           if (v == q) si = isc[q];
-        sr[n * 5 + v] = (acc[i] * is0) * si;
+        sr[n * 5 + v] = (acc[i] * pow2f(-(int)ex[n] - 13)) * si;
       }
     }
   }

@@ -18,14 +18,15 @@ namespace afe {
 // four consecutive rows hit 32 different shared-memory banks.
 inline constexpr int minv_ld(int n) { return (n + 15) / 16 * 16 + 8; }
 
-// Words (32 bits) of a cell's block of split M_i^-1 (pairs of 16-bit values): a 32-word header
-// (word 0: 1 / s), then the 16 x 16 tiles (i, j), j <= i, of the lower triangle at i (i + 1) / 2 + j,
+// Words (32 bits) of a cell's block of split M_i^-1 (pairs of 16-bit values): the row exponents (8 bits
+// each, padded to 128), then the 16 x 16 tiles (i, j), j <= i, of the lower triangle at i (i + 1) / 2 + j,
 // 128 words of hi and 128 of lo each.
+inline constexpr int minv_split_head(int n) { return (n + 127) / 128 * 32; }
 inline constexpr int64_t minv_split_words(int n) {
-  return 32 + (int64_t)((n + 15) / 16) * ((n + 15) / 16 + 1) / 2 * 256;
+  return minv_split_head(n) + (int64_t)((n + 15) / 16) * ((n + 15) / 16 + 1) / 2 * 256;
 }
 // Offset (words, a multiple of 32) of a cell's split block from its offset in the dense array, its first
-// node and its index: with t = ceil(n / 16), 32 + 128 t (t + 1) <= n (16 t + 8) / 2 + 12 n + 352 - 31.
+// node and its index: with t = ceil(n / 16), n / 4 + 32 + 128 t (t + 1) <= n (16 t + 8) / 2 + 12 n + 352 - 31.
 inline constexpr int64_t minv_split_start(int64_t minv_ptr, int64_t n0, int64_t c) {
   return (minv_ptr / 2 + 12 * n0 + 352 * c) / 32 * 32;
 }
