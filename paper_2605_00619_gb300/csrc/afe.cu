@@ -423,10 +423,24 @@ void sync_self(afe_mesh* m) {
   b.tab[0] = m->dm;
 }
 
+// Allocates the blocks of M_i^-1, the gather blocks and `extra` words (see block_layout).
+template <typename Words>
+afe_status alloc_blocks(afe_mesh* m, Words words, size_t extra, uint32_t** tail) {
+  const afe::BlockLayout L = afe::block_layout(m->topo.node_ptr, words, extra,
+                                               afe::pc_gather_bytes(m->dm, m->topo.T, m->ref.Np, m->ref.Nf));
+  unsigned char* p = nullptr;
+  AFE_TRY(m->alloc(&p, L.bytes));
+  m->dm.m16 = (uint32_t*)p;
+  *tail = (uint32_t*)(p + L.tail);
+  m->dm.gat = p + L.gather;
+  AFE_CUDA(cudaMemcpy(p, L.ptr.data(), L.ptr.size() * 8, cudaMemcpyHostToDevice));
+  return AFE_OK;
+}
+
 // What predictor_cells_kernel needs beside the one-block form's data: the split copy of M_i^-1
 // and the gather blocks.  A handle whose cells do not fit the plan, or for which the device
 // has no room left, keeps the one-block form.
-afe_status set_up_cells(afe_mesh* m, int64_t nminv) {
+afe_status set_up_cells(afe_mesh* m) {
   const afe::Topology& T = m->topo;
   const afe::RefData& R = m->ref;
   for (int s = 0; s < R.Nt; ++s) {
@@ -455,11 +469,13 @@ afe_status set_up_cells(afe_mesh* m, int64_t nminv) {
   }
   AFE_TRY(plan_cells(m->p.order, m->device, m->n_sm, T.C, !kinds.inviscid, m->pcells, &pc));
   if (!pc.blocks) return AFE_OK;
-  if (m->alloc(&m->dm.m16, (size_t)afe::minv_split_start(nminv, T.n_nodes, T.C)) != AFE_OK ||
-      m->alloc(&m->dm.gat, afe::pc_gather_bytes(m->dm, T.T, R.Np, R.Nf)) != AFE_OK) {
-    (void)cudaGetLastError();  // out of memory: the one-block form needs neither
+  uint32_t* none = nullptr;
+  const afe_status s = alloc_blocks(m, afe::minv_split_words, 0, &none);
+  if (s == AFE_ENOMEM) {
+    (void)cudaGetLastError();  // the one-block form needs none of them
     return AFE_OK;
   }
+  AFE_TRY(s);
   afe::pc_set_up(m->dm, R.Np, R.Nf, (int)std::min<int64_t>(T.C, (int64_t)m->n_sm * 8), m->stream);
   AFE_CUDA(cudaGetLastError());
   m->pc = pc;
@@ -469,7 +485,7 @@ afe_status set_up_cells(afe_mesh* m, int64_t nminv) {
 // What the FP64 predictor of predictor_f64.cuh needs: the digits of M_i^-1 and the gather blocks.  A
 // handle whose cells do not fit its plan, or for which the device has no room left, keeps
 // predictor_kernel and its scratch.
-afe_status set_up_f64(afe_mesh* m, int64_t nminv) {
+afe_status set_up_f64(afe_mesh* m) {
   const afe::Topology& T = m->topo;
   const afe::RefData& R = m->ref;
   if (R.N > 3) return AFE_OK;
@@ -488,17 +504,18 @@ afe_status set_up_f64(afe_mesh* m, int64_t nminv) {
   }
   if (!pd.blocks) return AFE_OK;
   std::vector<uint32_t> table(2 * afe::pd_stiffness_words(R.N));
-  m->dref.sexp = afe::pd_stiffness_digits(R, false, table.data());
-  (void)afe::pd_stiffness_digits(R, true, table.data() + table.size() / 2);
   uint32_t* dtab = nullptr;
-  AFE_TRY(m->upload(&dtab, table));
-  m->dref.sdig = dtab;
-  m->dref.sdig_t = dtab + table.size() / 2;
-  if (m->alloc(&m->dm.m16, 2 * (size_t)afe::pd_start(nminv, T.n_nodes, T.C)) != AFE_OK ||
-      m->alloc(&m->dm.gat, afe::pc_gather_bytes(m->dm, T.T, R.Np, R.Nf)) != AFE_OK) {
+  const afe_status s = alloc_blocks(m, afe::pd_words, table.size(), &dtab);
+  if (s == AFE_ENOMEM) {
     (void)cudaGetLastError();
     return AFE_OK;
   }
+  AFE_TRY(s);
+  m->dref.sexp = afe::pd_stiffness_digits(R, false, table.data());
+  (void)afe::pd_stiffness_digits(R, true, table.data() + table.size() / 2);
+  AFE_CUDA(cudaMemcpy(dtab, table.data(), table.size() * 4, cudaMemcpyHostToDevice));
+  m->dref.sdig = dtab;
+  m->dref.sdig_t = dtab + table.size() / 2;
   const int grid = (int)std::min<int64_t>(T.C, (int64_t)m->n_sm * 8);
   afe::pd_set_up(m->dm, grid, m->stream);
   afe::pc_gather_set_up(m->dm, R.Np, R.Nf, grid, m->stream);
@@ -790,9 +807,9 @@ afe_status afe_mesh_create(const afe_params* p, int64_t n_vertices, const double
         d.minv64 = nullptr;
         break;
       }
-    if (M->f32_ok) AFE_TRY(set_up_cells(M, nminv));
+    if (M->f32_ok) AFE_TRY(set_up_cells(M));
   } else {
-    AFE_TRY(set_up_f64(M, nminv));
+    AFE_TRY(set_up_f64(M));
   }
   // the set-up kernels end before the call returns: the handle's next work may be on another stream
   AFE_CUDA(cudaStreamSynchronize(M->stream));

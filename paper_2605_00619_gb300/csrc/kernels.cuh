@@ -54,7 +54,8 @@ struct DevMesh {
   double* wvec;
   double* minv64;
   float* minv32;
-  uint32_t* m16;       // M_i^-1 as pairs of FP16 values in matrix-fragment order (reduced precision)
+  uint32_t* m16;       // M_i^-1 as pairs of FP16 values (reduced precision) or digits, in matrix-fragment
+                       // order, behind the offsets of the cells' blocks (see m16_block)
   unsigned char* gat;  // per cell: gather lists and face data of the reduced-precision predictor
   double* u;
   void* vol;
@@ -151,6 +152,11 @@ __device__ __forceinline__ void phys_flux(const Real* Q, const Real (*gq)[5], bo
     for (int a = 0; a < 3; ++a) F[e][1 + a] = Q[1 + a] * v[e] + sig[a][e];
     F[e][4] = Q[4] * v[e] + v[0] * sig[0][e] + v[1] * sig[1][e] + v[2] * sig[2][e] - heat[e];
   }
+}
+
+// A cell's block of M_i^-1 in fragment order.
+__device__ __forceinline__ uint32_t* m16_block(const DevMesh& m, int64_t c) {
+  return m.m16 + reinterpret_cast<const int64_t*>(m.m16)[c];
 }
 
 // Block-wide max of two values (blockDim.x a multiple of 32, <= 1024).

@@ -139,7 +139,7 @@ static __global__ void __launch_bounds__(256) split_minv_kernel(DevMesh m) {
   for (int64_t c = blockIdx.x; c < m.C; c += gridDim.x) {
     const int n = (int)(m.node_ptr[c + 1] - m.node_ptr[c]), LD = minv_ld(n);
     const float* A = m.minv32 + m.minv_ptr[c];
-    uint32_t* out = m.m16 + minv_split_start(m.minv_ptr[c], m.node_ptr[c], c);
+    uint32_t* out = m16_block(m, c);
     auto expo = [&](int i) {
       const int e = (int)(__float_as_uint(A[(int64_t)i * LD + i]) >> 23 & 255u) - 126;  // M_ii < 2^e
       return -((e + 1) >> 1);

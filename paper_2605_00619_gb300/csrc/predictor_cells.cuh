@@ -954,7 +954,7 @@ __device__ __forceinline__ bool predictor_cells(const Batch& bt, const PcRef& re
       const int64_t n0 = m.node_ptr[c], kbase = m.sub_ptr[c], s0 = m.slot_ptr[c];
       const int Ni = (int)(m.node_ptr[c + 1] - n0), S = (int)(m.sub_ptr[c + 1] - kbase);
       const int ns = (int)(m.slot_ptr[c + 1] - s0);
-      const uint32_t* const m16 = m.m16 + minv_split_start(m.minv_ptr[c], n0, c);
+      const uint32_t* const m16 = m16_block(m, c);
       const uint32_t gbytes = (uint32_t)gat_bytes(Ni, S, ns, NP, NF);
       const int head = minv_split_head(Ni);
       const uint32_t o_gat = (uint32_t)(pc_up(sizeof(PcShared)) + pc_up((size_t)S * P::REC)),
@@ -1109,7 +1109,7 @@ __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) correc
   const int64_t c = gc - bt.cpre[h];
   const int64_t n0 = m.node_ptr[c], s0 = m.slot_ptr[c];
   const int Ni = (int)(m.node_ptr[c + 1] - n0), ns = (int)(m.slot_ptr[c + 1] - s0), nks = (Ni + 15) / 16;
-  const uint32_t* const m16 = m.m16 + minv_split_start(m.minv_ptr[c], n0, c);
+  const uint32_t* const m16 = m16_block(m, c);
   unsigned char* const frag = pc_smem;                                   // [nks][320] split right-hand side
   float* const sr = reinterpret_cast<float*>(pc_smem + nks * 320);       // [N_i][5] r (rows scaled), then du
   float* const sf = sr + ((Ni * 5 + 3) & ~3);                            // [ns][NF][5] face integrals

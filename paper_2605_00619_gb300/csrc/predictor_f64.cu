@@ -67,7 +67,7 @@ static __global__ void __launch_bounds__(256) digits_kernel(DevMesh m) {
     const int64_t n0 = m.node_ptr[c];
     const int n = (int)(m.node_ptr[c + 1] - n0), LD = minv_ld(n), nks = (n + 15) / 16;
     const double* A = m.minv64 + m.minv_ptr[c];
-    uint32_t* out = m.m16 + 2 * pd_start(m.minv_ptr[c], n0, c);
+    uint32_t* out = m16_block(m, c);
     int16_t* ex = reinterpret_cast<int16_t*>(out + (size_t)nks * nks * 512);
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
       const int e = (__double2hiint(A[(int64_t)i * LD + i]) >> 20 & 0x7ff) - 1022;  // M_ii < 2^e

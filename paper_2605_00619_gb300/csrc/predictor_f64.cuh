@@ -810,7 +810,7 @@ __global__ void __launch_bounds__(32 * W, MB) predictor_f64_kernel(const __grid_
                    o_exp = o_A + (uint32_t)pc_up((size_t)S * NP * 2), o_uh = o_exp + (uint32_t)pc_up((size_t)Ni * 2),
                    o_q = o_uh + (uint32_t)pc_up((size_t)Ni * 40), o_region = o_q + (uint32_t)pc_up((size_t)Ni * SQ * 8);
     const int nks = (Ni + 15) / 16;
-    const uint32_t* const dig = m.m16 + 2 * pd_start(m.minv_ptr[c], n0, c);
+    const uint32_t* const dig = m16_block(m, c);
     {
       const uint4* src = reinterpret_cast<const uint4*>(m.gat + gat_start(n0, k0, s0, c, NP, NF));
       uint4* dst = reinterpret_cast<uint4*>(pc_smem + kPdGat);

@@ -37,18 +37,7 @@ template <int N>
 void pd_launch(const PdPlan& plan, const Batch& b, const PdRef& ref, bool inviscid, bool viscous, int diag, int n_sm,
                cudaStream_t st);
 
-// 32-bit words of a cell's digit block: 16 x 16 tiles of 512 words, then the row exponents.
-inline constexpr int64_t pd_words(int n) {
-  return (int64_t)((n + 15) / 16) * ((n + 15) / 16) * 512 + (n + 63) / 64 * 32;
-}
-// Offset of a cell's digit block from its offset in the M_i^-1 array (which counts FP64 words of
-// rows padded to 16 columns + 8: a 16-aligned square of 8-byte values needs at most 15 rows more).
-inline constexpr int64_t pd_start(int64_t minv_ptr, int64_t n0, int64_t c) {
-  // N_i (up16 + 8) + 32 N_i + 1024 >= up16^2 + N_i / 2 + 32 words of 8 bytes
-  return minv_ptr + 32 * n0 + 1024 * c;
-}
-
-// Digit blocks of M_i^-1 (m.m16, words at 2 pd_start) from m.minv64.
+// Digit blocks of M_i^-1 (m.m16) from m.minv64.
 void pd_set_up(const DevMesh& m, int grid, cudaStream_t st);
 
 }  // namespace afe

@@ -25,10 +25,31 @@ inline constexpr int minv_split_head(int n) { return (n + 127) / 128 * 32; }
 inline constexpr int64_t minv_split_words(int n) {
   return minv_split_head(n) + (int64_t)((n + 15) / 16) * ((n + 15) / 16 + 1) / 2 * 256;
 }
-// Offset (words, a multiple of 32) of a cell's split block from its offset in the dense array, its first
-// node and its index: with t = ceil(n / 16), n / 4 + 32 + 128 t (t + 1) <= n (16 t + 8) / 2 + 12 n + 352 - 31.
-inline constexpr int64_t minv_split_start(int64_t minv_ptr, int64_t n0, int64_t c) {
-  return (minv_ptr / 2 + 12 * n0 + 352 * c) / 32 * 32;
+// The same of a cell's digit block (the FP64 form): 16 x 16 tiles of 512 words, then the row exponents.
+inline constexpr int64_t pd_words(int n) {
+  return (int64_t)((n + 15) / 16) * ((n + 15) / 16) * 512 + (n + 63) / 64 * 32;
+}
+
+// What the tensor-core forms keep of a mesh, in one allocation: the word offsets of the cells' blocks from
+// its start, the blocks (words(n) for a cell of n nodes), `tail` further words and gather blocks of
+// `gather` bytes.  Parts start at multiples of 128 bytes, of which the blocks and the tail are whole
+// multiples.  One allocation, because a device with room for a part only would keep that part for
+// nothing while the handle lives.
+struct BlockLayout {
+  std::vector<int64_t> ptr;      // [C+1]
+  size_t tail = 0, gather = 0;   // byte offsets
+  size_t bytes = 0;
+};
+template <typename Words>
+BlockLayout block_layout(const std::vector<int64_t>& node_ptr, Words words, size_t tail, size_t gather) {
+  BlockLayout L;
+  L.ptr.assign(node_ptr.size(), (int64_t)(node_ptr.size() + 15) / 16 * 32);
+  for (size_t c = 0; c + 1 < node_ptr.size(); ++c)
+    L.ptr[c + 1] = L.ptr[c] + words((int)(node_ptr[c + 1] - node_ptr[c]));
+  L.tail = (size_t)L.ptr.back() * 4;
+  L.gather = L.tail + tail * 4;
+  L.bytes = L.gather + gather;
+  return L;
 }
 
 struct Topology {
