@@ -225,7 +225,10 @@ afe_status afe_plan_info(const afe_mesh* m, afe_plan* out);
  * (tcgen05), for meshes whose every cell fits its shared-memory plan (up to 640 nodes per cell;
  * else AFE_EINVAL).  Both form FP32-level products of split operands (16-bit pairs or 3xTF32; results
  * agree to FP32 rounding, not bit for bit); on the measured workloads form 0 is the faster one.  A batch takes
- * the tensor-memory form only when every member asks for it.  Other values: AFE_EINVAL. */
+ * the tensor-memory form only when every member asks for it.  Form 1 reads FP32 rows of M_i^-1, which a
+ * handle on the form with several cells per SM has not: the first request (here, or by a schedule of the
+ * handle or of a batch it is a member of) forms them, 4 bytes per entry of device memory that the
+ * handle then keeps (AFE_ENOMEM: no room).  Other values: AFE_EINVAL. */
 afe_status afe_set_predictor_variant(afe_mesh* m, int32_t variant);
 
 /* Poll limit of the first bounded wait the FP32 shared-memory predictor makes for every cell

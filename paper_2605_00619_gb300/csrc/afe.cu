@@ -106,6 +106,17 @@ struct afe_mesh {
     if (!v.empty()) AFE_CUDA(cudaMemcpy(*ptr, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
     return AFE_OK;
   }
+  template <typename T>
+  void release(T** ptr, size_t count) {  // of an alloc() of the same count
+    for (size_t i = 0; i < allocs.size(); ++i)
+      if (allocs[i] == (void*)*ptr) {
+        cudaFree(*ptr);
+        allocs.erase(allocs.begin() + i);
+        bytes -= (int64_t)(count * sizeof(T));
+        break;
+      }
+    *ptr = nullptr;
+  }
   ~afe_mesh() {
     for (cudaEvent_t e : ev) cudaEventDestroy(e);
     for (void* p : allocs) cudaFree(p);
@@ -437,6 +448,55 @@ afe_status alloc_blocks(afe_mesh* m, Words words, size_t extra, uint32_t** tail)
   return AFE_OK;
 }
 
+// Inverse mass matrices in d.minv64 and w_i in d.wvec (FP64 set-up on the GPU); d.flags reports a
+// matrix that is not positive definite.
+void invert_masses(const afe_mesh* m, const afe::DevMesh& d) {
+  const int grid = (int)std::min<int64_t>(d.C, (int64_t)m->n_sm * 4);
+  afe::assemble_mass_kernel<<<grid, 256, 0, m->stream>>>(d, m->d_ref);
+  afe::invert_spd_kernel<<<grid, 256, 0, m->stream>>>(d);
+  afe::symmetrize_kernel<<<grid, 256, 0, m->stream>>>(d);
+}
+
+void round_rows(const afe_mesh* m, const afe::DevMesh& d) {
+  const int grid = (int)std::min<int64_t>(d.C, (int64_t)m->n_sm * 4);
+  afe::round_rows_kernel<<<grid, 256, 0, m->stream>>>(d);
+}
+
+// The FP32 rows of M_i^-1.  Handles on the form with several cells per SM read its split copy
+// and carry no rows, until they are asked for the tensor-memory form: the rows are then formed from
+// FP64 inverses as in set-up.
+afe_status ensure_rows(afe_mesh* m) {
+  if (m->p.precision != AFE_FP32 || m->dm.minv32) return AFE_OK;
+  AFE_CUDA(cudaStreamSynchronize(m->stream));
+  afe::DevMesh d = m->dm;  // of the handle's data only the rows are written: a batch may be reading the rest
+  const size_t nminv = (size_t)m->topo.minv_ptr[m->topo.C], nodes = (size_t)m->topo.n_nodes;
+  double* tmp = nullptr;
+  float* rows = nullptr;
+  const size_t ntmp = nminv + nodes + afe::F_COUNT;
+  afe_status s = m->alloc(&tmp, ntmp);
+  if (s == AFE_OK) s = m->alloc(&rows, nminv);
+  if (s == AFE_OK) {
+    d.minv64 = tmp;
+    d.wvec = tmp + nminv;
+    d.flags = (int*)(d.wvec + nodes);
+    d.minv32 = rows;
+    invert_masses(m, d);
+    round_rows(m, d);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
+    if (e != cudaSuccess) s = fail(AFE_ECUDA, std::string("rows of M_i^-1: ") + cudaGetErrorString(e));
+  }
+  (void)cudaGetLastError();
+  if (tmp) m->release(&tmp, ntmp);
+  if (s != AFE_OK) {
+    if (rows) m->release(&rows, nminv);
+    return s;
+  }
+  m->dm.minv32 = rows;
+  sync_self(m);
+  return AFE_OK;
+}
+
 // What predictor_cells_kernel needs beside the one-block form's data: the split copy of M_i^-1
 // and the gather blocks.  A handle whose cells do not fit the plan, or for which the device
 // has no room left, keeps the one-block form.
@@ -521,14 +581,9 @@ afe_status set_up_f64(afe_mesh* m) {
   afe::pc_gather_set_up(m->dm, R.Np, R.Nf, grid, m->stream);
   AFE_CUDA(cudaGetLastError());
   m->pd = pd;
-  for (size_t i = 0; i < m->allocs.size(); ++i)  // predictor_kernel's scratch is not needed then
-    if (m->allocs[i] == m->scratch) {
-      cudaFree(m->scratch);
-      m->allocs.erase(m->allocs.begin() + i);
-      m->bytes -= m->scratch_stride * m->pred_grid * 8;
-      m->scratch = nullptr;
-      break;
-    }
+  double* scratch = (double*)m->scratch;  // predictor_kernel's is not needed then
+  m->release(&scratch, (size_t)m->scratch_stride * m->pred_grid);
+  m->scratch = nullptr;
   return AFE_OK;
 }
 
@@ -715,7 +770,6 @@ afe_status afe_mesh_create(const afe_params* p, int64_t n_vertices, const double
   AFE_TRY(M->alloc(&d.wvec, T.n_nodes));
   const int64_t nminv = T.minv_ptr[T.C];
   AFE_TRY(M->alloc(&d.minv64, nminv));
-  if (p->precision == AFE_FP32) AFE_TRY(M->alloc(&d.minv32, nminv));
   AFE_TRY(M->alloc(&d.u, T.n_nodes * 5));
   const size_t rb = p->precision == AFE_FP32 ? 4 : 8;
   {
@@ -789,25 +843,21 @@ afe_status afe_mesh_create(const afe_params* p, int64_t n_vertices, const double
   AFE_CUDA(cudaMemsetAsync(d.flags, 0, afe::F_COUNT * sizeof(int), M->stream));
   AFE_CUDA(cudaMemsetAsync(d.maxbits, 0, sizeof(unsigned long long), M->stream));
   AFE_CUDA(cudaMemsetAsync(d.work, 0, 4 * sizeof(int), M->stream));
-  const int sgrid = (int)std::min<int64_t>(T.C, (int64_t)M->n_sm * 4);
-  afe::assemble_mass_kernel<<<sgrid, 256, 0, M->stream>>>(d, M->d_ref);
-  afe::invert_spd_kernel<<<(int)std::min<int64_t>(T.C, (int64_t)M->n_sm * 4), 256, 0, M->stream>>>(d);
-  afe::symmetrize_kernel<<<sgrid, 256, 0, M->stream>>>(d, p->precision == AFE_FP32);
+  invert_masses(M, d);
   AFE_CUDA(cudaGetLastError());
   int flags[afe::F_COUNT];
   AFE_TRY(read_flags(M, flags));
   if (flags[afe::F_NONFINITE]) return fail(AFE_EMESH, "a cell mass matrix is not positive definite");
   if (p->precision == AFE_FP32) {
-    // only the FP32 copy is used by the reduced-precision step
-    for (size_t i = 0; i < M->allocs.size(); ++i)
-      if (M->allocs[i] == d.minv64) {
-        cudaFree(d.minv64);
-        M->allocs.erase(M->allocs.begin() + i);
-        M->bytes -= nminv * 8;
-        d.minv64 = nullptr;
-        break;
-      }
+    // the reduced-precision step reads the split copy of the inverses, or their FP32 rows
     if (M->f32_ok) AFE_TRY(set_up_cells(M));
+    if (!M->pc.blocks) {
+      AFE_TRY(M->alloc(&d.minv32, nminv));
+      round_rows(M, d);
+      AFE_CUDA(cudaGetLastError());
+    }
+    AFE_CUDA(cudaStreamSynchronize(M->stream));
+    M->release(&d.minv64, nminv);
   } else {
     AFE_TRY(set_up_f64(M));
   }
@@ -1098,6 +1148,7 @@ afe_status afe_set_schedule(afe_mesh* m, const afe_schedule* s) {
   if (s->variant == 1 && m->p.precision == AFE_FP32 && !(m->f32_ok && m->f32_tc_fits))
     return fail(AFE_EINVAL, "the cells do not fit the tensor-memory plan of the FP32 predictor");
   AFE_CUDA(cudaStreamSynchronize(m->stream));
+  if (s->variant == 1) AFE_TRY(ensure_rows(m));
   if (s->cost_order && !m->d_order) {
     const std::vector<int32_t> ord = cost_order({&m->topo}, m->p.order);
     AFE_TRY(m->upload(&m->d_order, ord));
@@ -1121,6 +1172,7 @@ afe_status afe_set_predictor_variant(afe_mesh* m, int32_t variant) {
   if (variant != 0 && variant != 1) return fail(AFE_EINVAL, "variant must be 0 (mma.sync) or 1 (tcgen05)");
   if (variant == 1 && m->p.precision == AFE_FP32 && !(m->f32_ok && m->f32_tc_fits))
     return fail(AFE_EINVAL, "the cells do not fit the tensor-memory plan of the FP32 predictor");
+  if (variant == 1) AFE_TRY(ensure_rows(m));
   m->variant = variant;
   m->sched.variant = variant;
   m->f32_tc = (m->f32_ok && m->f32_tc_fits && variant == 1) ? 1 : 0;
@@ -1373,6 +1425,15 @@ afe_status afe_batch_set_schedule(afe_batch* b, const afe_schedule* s) {
   if (s->variant == 1 && !b->tc_fits)
     return fail(AFE_EINVAL, "the members' cells do not fit the tensor-memory plan together");
   AFE_CUDA(cudaStreamSynchronize(b->st));
+  if (s->variant == 1) {
+    int at[2] = {0, 0};
+    for (size_t h = 0; h < b->mem.size(); ++h) {
+      afe_mesh* m = b->mem[h];
+      AFE_TRY(ensure_rows(m));
+      const int k = m->pc.blocks ? 0 : 1;
+      b->bt.tab[h].minv32 = b->sub[k].tab[at[k]++].minv32 = m->dm.minv32;
+    }
+  }
   if (s->cost_order && !b->d_order) {
     std::vector<const afe::Topology*> tops;
     for (afe_mesh* m : b->mem) tops.push_back(&m->topo);
@@ -1453,6 +1514,10 @@ afe_status autotune_impl(const std::string& sig, int order, bool tc_fits, int* w
   afe_status status = AFE_OK;
   for (const afe_schedule& c : cand) {
     status = set(c);
+    if (status == AFE_ENOMEM && c.variant == 1) {  // no room for that form's rows of M_i^-1
+      status = AFE_OK;
+      continue;
+    }
     if (status != AFE_OK) break;
     const StepPlan P = plan();
     float ms = 0.f;

@@ -335,8 +335,8 @@ static __global__ void __launch_bounds__(256) invert_spd_kernel(DevMesh m) {
   }
 }
 
-// Symmetrise in FP64 and keep the FP32 copy used by the reduced-precision path.
-static __global__ void symmetrize_kernel(DevMesh m, int make32) {
+// Symmetrise in FP64.
+static __global__ void symmetrize_kernel(DevMesh m) {
   for (int64_t c = blockIdx.x; c < m.C; c += gridDim.x) {
     const int n = (int)(m.node_ptr[c + 1] - m.node_ptr[c]);
     const int LD = minv_ld(n);
@@ -348,13 +348,18 @@ static __global__ void symmetrize_kernel(DevMesh m, int make32) {
       A[(int64_t)r * LD + q] = v;
       A[(int64_t)q * LD + r] = v;
     }
-    __syncthreads();
-    if (make32)  // padding (columns >= n, rows >= n) written as zeros
-      for (int64_t e = threadIdx.x; e < m.minv_ptr[c + 1] - m.minv_ptr[c]; e += blockDim.x) {
-        const int64_t r = e / LD, q = e % LD;
-        m.minv32[m.minv_ptr[c] + e] = (r < n && q < n) ? (float)A[e] : 0.f;
-      }
-    __syncthreads();
+  }
+}
+
+// FP32 rows of the inverses; padding (columns >= n, rows >= n) written as zeros.
+static __global__ void round_rows_kernel(DevMesh m) {
+  for (int64_t c = blockIdx.x; c < m.C; c += gridDim.x) {
+    const int n = (int)(m.node_ptr[c + 1] - m.node_ptr[c]), LD = minv_ld(n);
+    const int64_t at = m.minv_ptr[c];
+    for (int64_t e = threadIdx.x; e < m.minv_ptr[c + 1] - at; e += blockDim.x) {
+      const int64_t r = e / LD, q = e % LD;
+      m.minv32[at + e] = (r < n && q < n) ? (float)m.minv64[at + e] : 0.f;
+    }
   }
 }
 

@@ -131,18 +131,19 @@ template void pc_add_cell<AFE_ORDER>(int, int, int, PcCells*);
 template void pc_launch<AFE_ORDER>(const PcPlan&, const Batch&, const PcRef&, bool, bool, int, int, cudaStream_t);
 
 #if AFE_ORDER == 1
-// The split copy of M_i^-1 (see minv_split_words), from its FP32 rows; one block per cell at a time.  Row
-// exponent p_i: M_ii 2^(2 p_i) in [1/4, 1); entry (i, j) is kept as 2^(13 + p_i + p_j) M_ij, below 2^13
-// in magnitude because the matrix is positive definite.  One power of two for the whole cell would leave
-// the rows of its large sub-tets the bits that FP16's range has left below those of its smallest one.
+// The split copy of M_i^-1 (see minv_split_words); one block per cell at a time.  Row exponent p_i:
+// M_ii 2^(2 p_i) in [1/4, 1) (bounded where M_ii is far outside FP32's range); entry (i, j) is kept as
+// 2^(13 + p_i + p_j) M_ij, below 2^13 in magnitude because the matrix is positive definite.  One power of two
+// for the whole cell would leave the rows of its large sub-tets the bits that FP16's range has left
+// below those of its smallest one.  Both parts come from the FP64 inverses.
 static __global__ void __launch_bounds__(256) split_minv_kernel(DevMesh m) {
   for (int64_t c = blockIdx.x; c < m.C; c += gridDim.x) {
     const int n = (int)(m.node_ptr[c + 1] - m.node_ptr[c]), LD = minv_ld(n);
-    const float* A = m.minv32 + m.minv_ptr[c];
+    const double* A = m.minv64 + m.minv_ptr[c];
     uint32_t* out = m16_block(m, c);
     auto expo = [&](int i) {
-      const int e = (int)(__float_as_uint(A[(int64_t)i * LD + i]) >> 23 & 255u) - 126;  // M_ii < 2^e
-      return -((e + 1) >> 1);
+      const int e = (__double2hiint(A[(int64_t)i * LD + i]) >> 20 & 0x7ff) - 1022;  // M_ii < 2^e
+      return max(-100, min(100, -((e + 1) >> 1)));
     };
     for (int i = threadIdx.x; i < 4 * minv_split_head(n); i += blockDim.x)
       reinterpret_cast<int8_t*>(out)[i] = (int8_t)(i < n ? expo(i) : 0);
@@ -156,10 +157,11 @@ static __global__ void __launch_bounds__(256) split_minv_kernel(DevMesh m) {
       uint32_t hi = 0, lo = 0;
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
-        const float x = (row < n && col + q < n)
-                            ? (A[(int64_t)row * LD + col + q] * pow2f(expo(row))) * pow2f(expo(col + q) + 13)
-                            : 0.f;
-        const __half h = __float2half_rn(x), l = __float2half_rn(x - __half2float(h));
+        const double x = (row < n && col + q < n)
+                             ? A[(int64_t)row * LD + col + q] *
+                                   __hiloint2double((1023 + 13 + expo(row) + expo(col + q)) << 20, 0)
+                             : 0.0;
+        const __half h = __double2half(x), l = __double2half(x - (double)__half2float(h));
         hi |= (uint32_t)__half_as_ushort(h) << (16 * q);
         lo |= (uint32_t)__half_as_ushort(l) << (16 * q);
       }
