@@ -28,7 +28,7 @@ template <int N>
 constexpr int corr_warps = N == 3 ? 8 : (N == 2 ? 4 : 1);
 
 size_t corr_smem(int n, int ns, int nf) {
-  return (size_t)(n + 15) / 16 * 320 + (size_t)((n * 5 + 3) & ~3) * 4 + (size_t)ns * nf * 20;
+  return (size_t)(n + 15) / 16 * kCorrFrag + (size_t)((n * 5 + 3) & ~3) * 4 + (size_t)ns * nf * 20;
 }
 
 template <int N, int SHAPE>

@@ -1077,8 +1077,9 @@ __global__ void __launch_bounds__(32 * W, MB) predictor_cells_kernel(const __gri
 // FP32 corrector on the split M_i^-1 (Sec. 4.4), one block of W warps per cell.
 //   f[slot][a] = 2 area sum_b Z^[a][b] G[b]     (a thread per slot and variable, once per slot)
 //   r = vol - sum over the node's face incidences of f   (fixed order)
-//   du = M_i^-1 r on the tensor cores: the operands, tiles and products of the predictor's first
-//        iteration (5 columns)
+//   du = M_i^-1 r on the tensor cores: the tiles of the predictor's first iteration (5 columns), with r
+//        in three FP16 parts (all of its 24 bits), every product but lo times the third part, and the
+//        leading ones added up outside the tensor cores, which truncate: FP32's accuracy (see below)
 //   u += du + (T - w_i . du) / |P_i|            (FP64: T = exact cell total of r, see
 //                                                corrector_f32_kernel)
 // What bounds it: M_i^-1 from HBM, once per step.  The lower triangle in 16-bit pairs is 53 % of the
@@ -1095,6 +1096,9 @@ __device__ __forceinline__ double f64_of(float x) {
   return __hiloint2double((int)((b & 0x80000000u) | ((b & 0x7fffffffu) >> 3) + 0x38000000u), (int)(b << 29));
 }
 
+// Bytes of the split right-hand side per 16 rows: two parts as the predictor's, behind them the third.
+constexpr int kCorrFrag = 480;
+
 template <int N, int W>
 __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) corrector_cells_kernel(
     const __grid_constant__ Batch bt, const __grid_constant__ CorrRef ref) {
@@ -1110,8 +1114,8 @@ __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) correc
   const int64_t n0 = m.node_ptr[c], s0 = m.slot_ptr[c];
   const int Ni = (int)(m.node_ptr[c + 1] - n0), ns = (int)(m.slot_ptr[c + 1] - s0), nks = (Ni + 15) / 16;
   const uint32_t* const m16 = m16_block(m, c);
-  unsigned char* const frag = pc_smem;                                   // [nks][320] split right-hand side
-  float* const sr = reinterpret_cast<float*>(pc_smem + nks * 320);       // [N_i][5] r (rows scaled), then du
+  unsigned char* const frag = pc_smem;                                   // [nks][kCorrFrag] split right-hand side
+  float* const sr = reinterpret_cast<float*>(pc_smem + nks * kCorrFrag); // [N_i][5] r (rows scaled), then du
   float* const sf = sr + ((Ni * 5 + 3) & ~3);                            // [ns][NF][5] face integrals
   const float* const vol = (const float*)m.vol;
   const float* const sG = (const float*)m.slot_G;
@@ -1186,18 +1190,23 @@ __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) correc
     isc[v] = __uint_as_float((uint32_t)(254 - e) << 23);
   }
   for (int n = tid; n < 16 * nks; n += THR) {
-    unsigned char* b = frag + (n >> 4) * 320 + ((n & 7) >> 1) * 16 + ((n >> 3) & 1) * 4 + (n & 1) * 2;
+    unsigned char* const rows = frag + (n >> 4) * kCorrFrag;
+    const int at = ((n >> 3) & 1) * 4 + (n & 1) * 2, ln = (n & 7) >> 1;
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       const float y = n < Ni ? sr[n * 5 + v] * sc[v] : 0.f;
       const __half hi = __float2half_rn(y);
-      *reinterpret_cast<__half*>(b + v * 64) = hi;
-      *reinterpret_cast<__half*>(b + v * 64 + 8) = __float2half_rn(y - __half2float(hi));
+      const float rest = y - __half2float(hi);
+      const __half lo = __float2half_rn(rest);
+      unsigned char* const b = rows + (v * 4 + ln) * 16 + at;
+      *reinterpret_cast<__half*>(b) = hi;
+      *reinterpret_cast<__half*>(b + 8) = lo;
+      *reinterpret_cast<__half*>(rows + 320 + (v * 4 + ln) * 8 + at) = __float2half_rn(rest - __half2float(lo));
     }
   }
   __syncthreads();
   for (int mt = warp; mt < nks; mt += W) {
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    float acc[4] = {0.f, 0.f, 0.f, 0.f}, low[4] = {0.f, 0.f, 0.f, 0.f};
     const uint32_t* const a0 = tiles + lane * 4;
     uint4 ah[DP], al[DP];
     auto load = [&](int s, int ks) {
@@ -1206,15 +1215,24 @@ __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) correc
       al[s] = ldg_stream(t + 128);
     };
     auto step = [&](int s, int ks) {
-      const uint4 b = lane < 20 ? *reinterpret_cast<const uint4*>(frag + ks * 320 + lane * 16) : make_uint4(0, 0, 0, 0);
+      const unsigned char* const f = frag + ks * kCorrFrag;
+      const uint4 b = lane < 20 ? *reinterpret_cast<const uint4*>(f + lane * 16) : make_uint4(0, 0, 0, 0);
+      const uint2 b3 = lane < 20 ? *reinterpret_cast<const uint2*>(f + 320 + lane * 8) : make_uint2(0, 0);
       uint4 x = ah[s], l = al[s];
       if (ks > mt) {  // above the diagonal: the mirrored tile
         x = transpose16(x);
         l = transpose16(l);
       }
-      mma_f16(acc, l, b.x, b.y);
-      mma_f16(acc, x, b.z, b.w);
-      mma_f16(acc, x, b.x, b.y);
+      // A tensor-core accumulator is truncated after every product: sums of 20 steps would be off by
+      // 1e-6 of themselves.  The leading products go to an accumulator of their own per step.
+      float lead[4] = {0.f, 0.f, 0.f, 0.f};
+      mma_f16(lead, x, b.x, b.y);
+      mma_f16(low, l, b.z, b.w);
+      mma_f16(low, x, b3.x, b3.y);
+      mma_f16(low, l, b.x, b.y);
+      mma_f16(low, x, b.z, b.w);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[i] += lead[i];
     };
 #pragma unroll
     for (int s = 0; s < DP; ++s) load(s, s);
@@ -1237,7 +1255,7 @@ __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) correc
 #pragma unroll
         for (int q = 1; q < 5; ++q)
           if (v == q) si = isc[q];
-        sr[n * 5 + v] = (acc[i] * pow2f(-(int)ex[n] - 13)) * si;
+        sr[n * 5 + v] = ((acc[i] + low[i]) * pow2f(-(int)ex[n] - 13)) * si;
       }
     }
   }
