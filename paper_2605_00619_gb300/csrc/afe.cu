@@ -787,7 +787,11 @@ afe_status afe_mesh_create(const afe_params* p, int64_t n_vertices, const double
   AFE_TRY(M->alloc(&d.beta, T.C));
   AFE_TRY(M->alloc(&d.mu, T.C));
   AFE_TRY(M->alloc(&d.means, T.C * 5));
-  AFE_TRY(M->alloc(&d.dt, 1));
+  {
+    const bool given = d.kappa0 >= 0.0;
+    const afe::ViscFace vf = {given ? 4.0 / 3.0 : std::max(4.0 / 3.0, d.gamma / d.Pr), given ? d.kappa0 / d.cv : 0.0};
+    AFE_TRY(M->upload(&d.dt, std::vector<double>{0.0, 0.0, vf.factor, vf.least}));
+  }
   AFE_TRY(M->alloc(&d.tacc, 1));
   AFE_TRY(M->alloc(&d.maxbits, 1));
   AFE_TRY(M->alloc(&d.flags, afe::F_COUNT));

@@ -66,7 +66,8 @@ struct DevMesh {
   double* beta;
   double* mu;     // per-cell dynamic viscosity mu_i (physical + artificial)
   double* means;  // [C][5] density, velocity and sound speed of the cell means
-  double* dt;     // device scalar: time step of the current step
+  double* dt;     // device scalars: time step of the current step, its inverse rounded to FP32, and the
+                  // face fluxes' viscous constants (see ViscFace)
   double* tacc;   // device scalar: accumulated time
   unsigned long long* maxbits;
   int* flags;
@@ -158,6 +159,16 @@ __device__ __forceinline__ void phys_flux(const Real* Q, const Real (*gq)[5], bo
 __device__ __forceinline__ uint32_t* m16_block(const DevMesh& m, int64_t c) {
   return m.m16 + reinterpret_cast<const int64_t*>(m.m16)[c];
 }
+
+__device__ __forceinline__ void store_dt(const DevMesh& m, double dt) {
+  m.dt[0] = dt;
+  m.dt[1] = (double)(float)(1.0 / dt);
+}
+// max(4 mu / 3, kappa / c_v) = max(mu factor, least): factor = 4/3, least = kappa / c_v with kappa given,
+// factor = max(4/3, gamma / Pr), least = 0 with kappa = mu gamma c_v / Pr.
+struct ViscFace {
+  double factor, least;
+};
 
 // Block-wide max of two values (blockDim.x a multiple of 32, <= 1024).
 __device__ __forceinline__ void block_max2(double& a, double& b, double* sh /* >= 64 */) {
@@ -578,7 +589,7 @@ static __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__
     const double mx = __longlong_as_double((long long)atomicExch(m.maxbits, 0ull));
     double dt = mx > 0.0 ? m.cfl * m.h_min / ((2 * m.N + 1) * mx) : 0.0;
     if (!(dt > 0.0)) atomicOr(&m.flags[F_NONFINITE], 4);
-    *m.dt = dt;
+    store_dt(m, dt);
     if (mode == CFL_STEP) *m.tacc += dt;
   }
   if (threadIdx.x < 4) bt.work[threadIdx.x] = 0;
@@ -587,7 +598,7 @@ static __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__
 // Start of a step of a given size.
 static __global__ void set_dt_kernel(const __grid_constant__ Batch bt, double dt) {
   for (int h = threadIdx.x; h < bt.nh; h += blockDim.x) {
-    *bt.tab[h].dt = dt;
+    store_dt(bt.tab[h], dt);
     *bt.tab[h].tacc += dt;
   }
   if (threadIdx.x < 4) bt.work[threadIdx.x] = 0;
@@ -1070,11 +1081,42 @@ __device__ __forceinline__ float f32_of(double x) {
   return __uint_as_float(bits);
 }
 
+// x as the sum of two FP32 values, the first of them x to nearest (48 bits; the first alone where the
+// second would leave FP32's normal range).
+__device__ __forceinline__ float2 f32_pair(double x) {
+  const float h = f32_of(x);
+  const int rest = __double2loint(x) & 0x1fffffff;  // the 29 bits dropped, of weight 2^(e - 127 - 52)
+  const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
+  if ((unsigned)(ex - 950) > 200u) return make_float2(h, 0.f);
+  const bool up = (__float_as_uint(h) & 0x7fffffffu) !=
+                  ((unsigned)((ex - 896) << 23) | (__funnelshift_l((unsigned)__double2loint(x), (unsigned)hi, 3) & 0x7fffffu));
+  const float l = (float)(up ? rest - 0x20000000 : rest) * __uint_as_float((unsigned)(ex - 896 - 52) << 23);
+  return make_float2(h, hi < 0 ? -l : l);
+}
+// x y rounded once.
+__device__ __forceinline__ float f32_product(double x, double y) {
+  const float2 a = f32_pair(x), b = f32_pair(y);
+  const float p = a.x * b.x;
+  return p + (fmaf(a.x, b.x, -p) + (a.x * b.y + a.y * b.x));
+}
+// (2N+1) / ((h_i + h_j) sqrt(pi / 2)) rounded once.
+template <int N>
+__device__ __forceinline__ float f32_face_eps(double hi, double hj) {
+  constexpr double c = (2 * N + 1) * 0.79788456080286535588;  // sqrt(2 / pi)
+  constexpr float c0 = (float)c, c1 = (float)(c - (double)c0), ic = (float)(1.0 / c);
+  const float2 a = f32_pair(hi), b = f32_pair(hj);
+  const float s = a.x + b.x, t = s - a.x;
+  const float rest = ((a.x - (s - t)) + (b.x - t)) + (a.y + b.y);
+  const float q = c0 / s;
+  return q + (fmaf(-q, s, c0) + fmaf(-q, rest, c1)) * (q * ic);
+}
+
 // The FP32 form's fluxes: L lanes per polygonal face (8, 16, 32 at N = 1, 2, 3: about the face nodes of
 // three sub-triangles), the states and fluxes of a lane's first two face nodes held in registers
 // from the wave speeds to the fluxes.  What it waited for before: the FP64 pipe (1 / dt, eps and the
 // conversions of mu, h and the normals, per lane), then chains of dependent loads; the
-// conversions are integer instructions now and slots and partners come as one pair.
+// conversions are integer instructions now, 1 / dt comes with dt, eps and the viscous coefficients are
+// formed in pairs of FP32 values, to the same single rounding, and slots and partners come as one pair.
 // us per launch before and after: 32^3 P3 1,177 and 493 (127 for the bytes at
 // the copy rate), 21^3 P2 258 and 98, 24^3 P1 479 and 82, 4^3 P1 18 and 14.
 template <int N>
@@ -1092,17 +1134,15 @@ __global__ void __launch_bounds__(256) face_f32_kernel(const __grid_constant__ B
   const float* sfn = (const float*)m.slot_fn;
   float* sG = (float*)m.slot_G;
   const int2* pairs = m.group_pair + g0;
-  const float rdt = f32_of(*m.dt), idt = 1.f / rdt, gam = f32_of(m.gamma);
+  const float rdt = f32_of(m.dt[0]), idt = f32_of(m.dt[1]), gam = f32_of(m.gamma);
   const int2 first = pairs[0];
   const int32_t ci = m.slot_cell[first.x];
   const int32_t cj = first.y >= 0 ? m.slot_cell[first.y] : ci;
   // |lambda_v| = max(4 mu / 3, kappa / c_v) / rho: the coefficient per side
-  const float icv = 1.f / f32_of(m.cv), k0 = f32_of(m.kappa0), gcp = f32_of(m.gamma * m.cv / m.Pr);
-  const float mu_i = f32_of(m.mu[ci]), mu_j = f32_of(m.mu[cj]);
-  const bool given = m.kappa0 >= 0.0;
-  const float cvis_i = fmaxf(4.f / 3.f * mu_i, (given ? k0 : mu_i * gcp) * icv);
-  const float cvis_j = fmaxf(4.f / 3.f * mu_j, (given ? k0 : mu_j * gcp) * icv);
-  const float hsum = f32_of(m.cell_h[ci]) + f32_of(m.cell_h[cj]);
+  const ViscFace vf = *reinterpret_cast<const ViscFace*>(m.dt + 2);
+  const double mu_i = m.mu[ci], mu_j = m.mu[cj], h_i = m.cell_h[ci], h_j = m.cell_h[cj];
+  const float least = f32_of(vf.least);
+  const float cvis_i = fmaxf(f32_product(mu_i, vf.factor), least), cvis_j = fmaxf(f32_product(mu_j, vf.factor), least);
   float smax = 0.f, vmax = 0.f;
   auto speeds = [&](const float* Q, const float (&n)[3], float cvis) {
     const float ir = 1.f / Q[0], rho = Q[0] * idt;
@@ -1149,8 +1189,7 @@ __global__ void __launch_bounds__(256) face_f32_kernel(const __grid_constant__ B
     smax = fmaxf(smax, __shfl_xor_sync(0xffffffffu, smax, o));
     vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
   }
-  // eps = (2N+1) / ((h_i + h_j) sqrt(pi / 2))
-  const float eps = (2 * N + 1) * 0.797884560802865f / hsum;
+  const float eps = f32_face_eps<N>(h_i, h_j);
   const float diss = 0.5f * (smax + 2.f * eps * vmax);
   auto flux = [&](int2 p, int a1, const float* q1, const float* q2, const float* f1, const float* f2) {
     float* go = sG + ((int64_t)p.x * NF + a1) * 5;
