@@ -284,6 +284,12 @@ afe_status launch_corrector(const StepPlan& P) {
       if (!P.one) return AFE_OK;
     }
   }
+  if constexpr (N <= 3 && sizeof(Real) == 8) {
+    if (P.pd.blocks) {  // the cells' digits are there
+      afe::pd_correct<N>(*P.b, P.d_ref, P.b->Nmax, P.st);
+      return AFE_OK;
+    }
+  }
   const afe::Batch& b = sizeof(Real) == 4 && P.one ? *P.one : *P.b;
   if (sizeof(Real) == 4 && corrector_f32_fits(b.Nmax)) {
     const size_t smem = (size_t)b.Nmax * 10 * sizeof(float);
@@ -542,9 +548,9 @@ afe_status set_up_cells(afe_mesh* m) {
   return AFE_OK;
 }
 
-// What the FP64 predictor of predictor_f64.cuh needs: the digits of M_i^-1 and the gather blocks.  A
-// handle whose cells do not fit its plan, or for which the device has no room left, keeps
-// predictor_kernel and its scratch.
+// What the FP64 predictor and corrector of predictor_f64.cuh need: the digits of M_i^-1 and the gather
+// blocks.  A handle whose cells do not fit their plan, or for which the device has no room left, keeps
+// the FP64 rows, predictor_kernel with its scratch, and corrector_kernel.
 afe_status set_up_f64(afe_mesh* m) {
   const afe::Topology& T = m->topo;
   const afe::RefData& R = m->ref;
@@ -864,6 +870,10 @@ afe_status afe_mesh_create(const afe_params* p, int64_t n_vertices, const double
     M->release(&d.minv64, nminv);
   } else {
     AFE_TRY(set_up_f64(M));
+    if (M->pd.blocks) {  // predictor and corrector read the digits
+      AFE_CUDA(cudaStreamSynchronize(M->stream));
+      M->release(&d.minv64, nminv);
+    }
   }
   // the set-up kernels end before the call returns: the handle's next work may be on another stream
   AFE_CUDA(cudaStreamSynchronize(M->stream));

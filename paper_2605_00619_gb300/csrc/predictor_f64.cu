@@ -17,6 +17,12 @@ struct PdShape {
 template <int N, bool VISC>
 constexpr auto pd_kernel = predictor_f64_kernel<N, PdShape<N>::W, PdShape<N>::MB, VISC>;
 
+// Warps per block of the corrector, and blocks per SM (register limit).
+template <int N>
+constexpr int pd_corr_warps = N == 3 ? 8 : 4;
+template <int N>
+constexpr auto pd_corr_kernel = corrector_f64_kernel<N, pd_corr_warps<N>, 16 / pd_corr_warps<N>>;
+
 }  // namespace
 
 template <int N>
@@ -32,6 +38,13 @@ cudaError_t pd_plan(int device, int Nmax, int Smax, int Fmax, PdPlan* out) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
   if (e != cudaSuccess) return e;
   const int stat = (int)std::max(fa.sharedSizeBytes, fv.sharedSizeBytes);
+  cudaFuncAttributes fc;
+  e = cudaFuncGetAttributes(&fc, pd_corr_kernel<N>);
+  if (e != cudaSuccess) return e;
+  const size_t corr = (size_t)optin - fc.sharedSizeBytes;
+  if (pd_corr_smem<N>(Nmax) > corr) return cudaSuccess;
+  e = cudaFuncSetAttribute(pd_corr_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)corr);
+  if (e != cudaSuccess) return e;
   for (int nb = PdShape<N>::MB; nb >= 1; --nb) {
     const int64_t share = std::min<int64_t>(per_sm / nb - 1024, optin) - stat;
     const size_t smem = share > 0 ? (size_t)share / 128 * 128 : 0;
@@ -56,6 +69,12 @@ void pd_launch(const PdPlan& p, const Batch& b, const PdRef& ref, bool inviscid,
   if (viscous) pd_kernel<N, true><<<grid, THR, smem, st>>>(b, ref, diag, smem, mixed);
 }
 
+template <int N>
+void pd_correct(const Batch& b, const RefData* ref, int Nmax, cudaStream_t st) {
+  pd_corr_kernel<N><<<(unsigned)b.cpre[1], 32 * pd_corr_warps<N>, pd_corr_smem<N>(Nmax), st>>>(b, ref);
+}
+
+template void pd_correct<AFE_ORDER>(const Batch&, const RefData*, int, cudaStream_t);
 template cudaError_t pd_plan<AFE_ORDER>(int, int, int, int, PdPlan*);
 template void pd_launch<AFE_ORDER>(const PdPlan&, const Batch&, const PdRef&, bool, bool, int, int, cudaStream_t);
 

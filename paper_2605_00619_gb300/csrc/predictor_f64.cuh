@@ -897,4 +897,107 @@ __global__ void __launch_bounds__(32 * W, MB) predictor_f64_kernel(const __grid_
   }
 }
 
+// ----------------------------------------------------------------------------------------
+// FP64 corrector on the digits of M_i^-1 (Sec. 4.4), one block per cell: r as corrector_kernel forms it, du = M_i^-1 r
+// by the digit products of the predictor's first iteration (5 columns), u += du.  With the FP64 rows read
+// here a handle would hold M_i^-1 twice.  us per launch, corrector_kernel on the rows and here: 8^3 P3 816 and 220,
+// 10^3 P2 254 and 112, 6^3 P1 18 and 18.
+template <int N>
+__host__ __device__ constexpr size_t pd_corr_smem(int n) {
+  return (size_t)(n + 15) / 16 * Pd<N>::FB1 + (size_t)n * 40;
+}
+template <int N, int W, int MB>
+__global__ void __launch_bounds__(32 * W, MB) corrector_f64_kernel(const __grid_constant__ Batch bt,
+                                                                   const RefData* __restrict__ ref) {
+  using P = Pd<N>;
+  constexpr int NF = P::NF, THR = 32 * W;
+  const DevMesh& m = bt.tab[0];
+  const int64_t c = blockIdx.x, n0 = m.node_ptr[c], s0 = m.slot_ptr[c];
+  const int Ni = (int)(m.node_ptr[c + 1] - n0), nks = (Ni + 15) / 16;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ double sZ[NF][NF];
+  __shared__ int ired[5][W];
+  unsigned char* const frag = pc_smem;                                        // digits of r (rows scaled)
+  double* const r = reinterpret_cast<double*>(pc_smem + (size_t)nks * P::FB1);  // [N_i][5] r, then du
+  const uint32_t* const dig = m16_block(m, c);
+  const int16_t* const sexp = reinterpret_cast<const int16_t*>(dig + (size_t)nks * nks * 512);
+  const double* const vol = (const double*)m.vol;
+  const double* const sG = (const double*)m.slot_G;
+  for (int e = tid; e < NF * NF; e += THR) sZ[e / NF][e % NF] = ref->Z[e / NF][e % NF];
+  __syncthreads();
+  // a thread's items are of one variable (its stride is a multiple of 5)
+  constexpr int FS = THR / 5 * 5;
+  int mx = -20000;
+  for (int e = tid; e < Ni * 5 && tid < FS; e += FS) {
+    const int n = e / 5, v = e - n * 5;
+    double acc = vol[(n0 + n) * 5 + v];
+    for (int64_t p = m.finc_ptr[n0 + n]; p < m.finc_ptr[n0 + n + 1]; ++p) {
+      const uint32_t w = m.finc[p];
+      const int64_t s = s0 + (w >> 4);
+      const double* z = sZ[w & 15];
+      double f = 0;
+#pragma unroll
+      for (int b = 0; b < NF; ++b) f += z[b] * sG[(s * NF + b) * 5 + v];
+      acc -= 2.0 * m.slot_geo[s * 4 + 3] * f;
+    }
+    r[e] = acc;
+    const int ex = __double2hiint(acc) >> 20 & 0x7ff;
+    mx = max(mx, ex == 0x7ff ? kPdNone : max(ex, 1) - 1022 - sexp[n]);
+  }
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    const int x = __reduce_max_sync(0xffffffffu, tid % 5 == v ? mx : -20000);
+    if (lane == 0) ired[v][warp] = x;
+  }
+  __syncthreads();
+  int ev[5];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+    ev[v] = ired[v][0];
+#pragma unroll
+    for (int w = 1; w < W; ++w) ev[v] = max(ev[v], ired[v][w]);
+  }
+  // fragments as pd_rhs writes them; rows past N_i: the digit zero
+  for (int n = tid; n < 16 * nks; n += THR) {
+    unsigned char* const row = frag + (n >> 4) * P::FB1 + ((n & 7) >> 1) * 32 + ((n >> 3) & 1) * 2 + (n & 1);
+    const int p = n < Ni ? sexp[n] : 0;
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      const unsigned long long d = n < Ni ? digits(r[n * 5 + v], ev[v] + p) : 0x8080808080808080ull;
+#pragma unroll
+      for (int s = 0; s < 8; ++s) row[v * 128 + 4 * s] = (unsigned char)(d >> (56 - 8 * s));
+    }
+  }
+  __syncthreads();
+  for (int mt = warp; mt < nks; mt += W) {
+    long long hi[4], lo[4];
+    digit_product(dig + (size_t)mt * nks * 512 + lane * 4, frag + lane * 32, P::FB1, lane < 20, nks, hi, lo);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int v = 2 * (lane & 3) + (i & 1), n = mt * 16 + (lane >> 2) + (i >> 1) * 8;
+      if (v < 5 && n < Ni) {
+        int e = ev[0];
+#pragma unroll
+        for (int q = 1; q < 5; ++q)
+          if (v == q) e = ev[q];
+        r[n * 5 + v] = digit_value(hi[i], lo[i], 56 - 124 + e - sexp[n], e >= kPdNone);
+      }
+    }
+  }
+  __syncthreads();
+  for (int n = tid; n < Ni; n += THR) {
+    bool bad = false;
+    double* un = m.u + (n0 + n) * 5;
+    double x[5];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) {
+      x[v] = un[v] + r[n * 5 + v];
+      un[v] = x[v];
+      bad |= !isfinite(x[v]);
+    }
+    const double p = (m.gamma - 1.0) * (x[4] - 0.5 * (x[1] * x[1] + x[2] * x[2] + x[3] * x[3]) / x[0]);
+    if (bad || !(x[0] > 0.0) || !(p > 0.0)) atomicOr(&m.flags[F_NONFINITE], 8);
+  }
+}
+
 }  // namespace afe

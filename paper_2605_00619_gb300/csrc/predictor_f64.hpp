@@ -37,6 +37,10 @@ template <int N>
 void pd_launch(const PdPlan& plan, const Batch& b, const PdRef& ref, bool inviscid, bool viscous, int diag, int n_sm,
                cudaStream_t st);
 
+// The corrector on the digits of M_i^-1, for cells of up to Nmax nodes.
+template <int N>
+void pd_correct(const Batch& b, const RefData* ref, int Nmax, cudaStream_t st);
+
 // Digit blocks of M_i^-1 (m.m16) from m.minv64.
 void pd_set_up(const DevMesh& m, int grid, cudaStream_t st);
 

@@ -19,6 +19,16 @@ def afe():
     return a
 
 
+# bytes of the same handles when the predictor read FP64 rows and kept its coefficients in global memory
+@pytest.mark.parametrize("N,k,rows_alone", [(1, 16, 173409210), (2, 11, 361215064), (3, 8, 788863260)])
+def test_digits_replace_the_fp64_rows(afe, N, k, rows_alone):
+    h = afe.create_from_polymesh(periodic_voronoi(k), afe.afe_default_params(N))
+    bytes_ = afe.afe_device_bytes(h)
+    print(f"P{N} FP64: {bytes_} bytes, rows alone {rows_alone}")
+    assert bytes_ <= rows_alone
+    afe.afe_mesh_destroy(h)
+
+
 def _handle(afe, pm, N):
     p = afe.afe_default_params(N, precision=afe.AFE_FP32, picard_tol=1e-6, cfl=0.1)
     h = afe.create_from_polymesh(pm, p)
