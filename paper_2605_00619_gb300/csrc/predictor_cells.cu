@@ -27,8 +27,9 @@ constexpr auto pc_kernel = predictor_cells_kernel<N, PcShape<N, SHAPE>::W, PcSha
 template <int N>
 constexpr int corr_warps = N == 3 ? 8 : (N == 2 ? 4 : 1);
 
-size_t corr_smem(int n, int ns, int nf) {
-  return (size_t)(n + 15) / 16 * kCorrFrag + (size_t)((n * 5 + 3) & ~3) * 4 + (size_t)ns * nf * 20;
+template <int N>
+size_t corr_smem(int n, int ns) {
+  return (size_t)(n + 15) / 16 * corr_frag<N> + (size_t)((n * 5 + 3) & ~3) * 4 + (size_t)ns * nf_of(N) * 20;
 }
 
 template <int N, int SHAPE>
@@ -60,7 +61,7 @@ cudaError_t plan_shape(int device, const PcCells& q, PcPlan* out) {
     cudaFuncAttributes fc;
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fc, corr);
     if (e != cudaSuccess) return e;
-    if (corr_smem(Nmax, Fmax, nf_of(N)) > optin - fc.sharedSizeBytes) return cudaSuccess;
+    if (corr_smem<N>(Nmax, Fmax) > optin - fc.sharedSizeBytes) return cudaSuccess;
     e = cudaFuncSetAttribute(corr, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fc.sharedSizeBytes);
     out->Fmax = Fmax;
     out->shape = SHAPE;
@@ -122,7 +123,7 @@ void pc_launch(const PcPlan& p, const Batch& b, const PcRef& ref, bool inviscid,
 template <int N>
 void pc_correct(const Batch& b, const CorrRef& ref, int Nmax, int Fmax, cudaStream_t st) {
   corrector_cells_kernel<N, corr_warps<N>>
-      <<<(unsigned)b.cpre[b.nh], 32 * corr_warps<N>, corr_smem(Nmax, Fmax, nf_of(N)), st>>>(b, ref);
+      <<<(unsigned)b.cpre[b.nh], 32 * corr_warps<N>, corr_smem<N>(Nmax, Fmax), st>>>(b, ref);
 }
 
 template void pc_correct<AFE_ORDER>(const Batch&, const CorrRef&, int, int, cudaStream_t);

@@ -1077,9 +1077,10 @@ __global__ void __launch_bounds__(32 * W, MB) predictor_cells_kernel(const __gri
 // FP32 corrector on the split M_i^-1 (Sec. 4.4), one block of W warps per cell.
 //   f[slot][a] = 2 area sum_b Z^[a][b] G[b]     (a thread per slot and variable, once per slot)
 //   r = vol - sum over the node's face incidences of f   (fixed order)
-//   du = M_i^-1 r on the tensor cores: the tiles of the predictor's first iteration (5 columns), with r
-//        in three FP16 parts (all of its 24 bits), every product but lo times the third part, and the
-//        leading ones added up outside the tensor cores, which truncate: FP32's accuracy (see below)
+//   du = M_i^-1 r on the tensor cores: the tiles of the predictor's first iteration (5 columns), with the
+//        leading products added up outside the tensor cores, which truncate, and at N <= 2, where sums are
+//        short, r in three FP16 parts (all of its 24 bits) and the product of the low parts: no further
+//        off than FP32 multiply-adds over FP32 rows
 //   u += du + (T - w_i . du) / |P_i|            (FP64: T = exact cell total of r, see
 //                                                corrector_f32_kernel)
 // What bounds it: M_i^-1 from HBM, once per step.  The lower triangle in 16-bit pairs is 53 % of the
@@ -1096,13 +1097,20 @@ __device__ __forceinline__ double f64_of(float x) {
   return __hiloint2double((int)((b & 0x80000000u) | ((b & 0x7fffffffu) >> 3) + 0x38000000u), (int)(b << 29));
 }
 
-// Bytes of the split right-hand side per 16 rows: two parts as the predictor's, behind them the third.
-constexpr int kCorrFrag = 480;
+// Parts of the split right-hand side, and its bytes per 16 rows: two parts as the predictor's, behind them the
+// third.  Relative L2 error of M_i^-1 r against 64 bits (random r, smooth du; FP32 multiply-adds): P3 1.2e-7, 3.4e-7
+// with two parts (3.2e-7, 5.2e-7); P2 0.9e-7, 2.4e-7 (1.9e-7, 3.4e-7) and P1 0.7e-7, 1.5e-7 (0.9e-7, 1.8e-7)
+// with three, above the multiply-adds' with two.
+template <int N>
+constexpr int corr_parts = N == 3 ? 2 : 3;
+template <int N>
+constexpr int corr_frag = 160 * corr_parts<N>;
 
 template <int N, int W>
 __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) corrector_cells_kernel(
     const __grid_constant__ Batch bt, const __grid_constant__ CorrRef ref) {
-  constexpr int NF = nf_of(N), THR = 32 * W, DP = N == 1 ? 2 : kPcDeep;
+  constexpr int NF = nf_of(N), THR = 32 * W, DP = N == 1 ? 2 : kPcDeep, FB = corr_frag<N>;
+  constexpr bool three = corr_parts<N> == 3;
   extern __shared__ __align__(128) unsigned char pc_smem[];
   __shared__ double sred[10][W];
   __shared__ float smax[5][W];
@@ -1114,8 +1122,8 @@ __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) correc
   const int64_t n0 = m.node_ptr[c], s0 = m.slot_ptr[c];
   const int Ni = (int)(m.node_ptr[c + 1] - n0), ns = (int)(m.slot_ptr[c + 1] - s0), nks = (Ni + 15) / 16;
   const uint32_t* const m16 = m16_block(m, c);
-  unsigned char* const frag = pc_smem;                                   // [nks][kCorrFrag] split right-hand side
-  float* const sr = reinterpret_cast<float*>(pc_smem + nks * kCorrFrag); // [N_i][5] r (rows scaled), then du
+  unsigned char* const frag = pc_smem;                                   // [nks][FB] split right-hand side
+  float* const sr = reinterpret_cast<float*>(pc_smem + nks * FB);        // [N_i][5] r (rows scaled), then du
   float* const sf = sr + ((Ni * 5 + 3) & ~3);                            // [ns][NF][5] face integrals
   const float* const vol = (const float*)m.vol;
   const float* const sG = (const float*)m.slot_G;
@@ -1190,7 +1198,7 @@ __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) correc
     isc[v] = __uint_as_float((uint32_t)(254 - e) << 23);
   }
   for (int n = tid; n < 16 * nks; n += THR) {
-    unsigned char* const rows = frag + (n >> 4) * kCorrFrag;
+    unsigned char* const rows = frag + (n >> 4) * FB;
     const int at = ((n >> 3) & 1) * 4 + (n & 1) * 2, ln = (n & 7) >> 1;
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
@@ -1201,7 +1209,8 @@ __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) correc
       unsigned char* const b = rows + (v * 4 + ln) * 16 + at;
       *reinterpret_cast<__half*>(b) = hi;
       *reinterpret_cast<__half*>(b + 8) = lo;
-      *reinterpret_cast<__half*>(rows + 320 + (v * 4 + ln) * 8 + at) = __float2half_rn(rest - __half2float(lo));
+      if constexpr (three)
+        *reinterpret_cast<__half*>(rows + 320 + (v * 4 + ln) * 8 + at) = __float2half_rn(rest - __half2float(lo));
     }
   }
   __syncthreads();
@@ -1215,9 +1224,8 @@ __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) correc
       al[s] = ldg_stream(t + 128);
     };
     auto step = [&](int s, int ks) {
-      const unsigned char* const f = frag + ks * kCorrFrag;
+      const unsigned char* const f = frag + ks * FB;
       const uint4 b = lane < 20 ? *reinterpret_cast<const uint4*>(f + lane * 16) : make_uint4(0, 0, 0, 0);
-      const uint2 b3 = lane < 20 ? *reinterpret_cast<const uint2*>(f + 320 + lane * 8) : make_uint2(0, 0);
       uint4 x = ah[s], l = al[s];
       if (ks > mt) {  // above the diagonal: the mirrored tile
         x = transpose16(x);
@@ -1227,8 +1235,11 @@ __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) correc
       // 1e-6 of themselves.  The leading products go to an accumulator of their own per step.
       float lead[4] = {0.f, 0.f, 0.f, 0.f};
       mma_f16(lead, x, b.x, b.y);
-      mma_f16(low, l, b.z, b.w);
-      mma_f16(low, x, b3.x, b3.y);
+      if constexpr (three) {
+        const uint2 b3 = lane < 20 ? *reinterpret_cast<const uint2*>(f + 320 + lane * 8) : make_uint2(0, 0);
+        mma_f16(low, l, b.z, b.w);
+        mma_f16(low, x, b3.x, b3.y);
+      }
       mma_f16(low, l, b.x, b.y);
       mma_f16(low, x, b.z, b.w);
 #pragma unroll
