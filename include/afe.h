@@ -193,9 +193,11 @@ afe_status afe_stage_times(afe_mesh* m, double* ms, int64_t* nsteps, int reset);
 
 /* How the handle's step runs (a host-side report; no GPU work).  The FP32 form keeps each
  * cell's fixed-point iteration in the shared memory of one predictor block when the cell fits
- * (fp32_shared = 1).  Meshes whose largest cell leaves room for at least two such blocks per SM
- * run the form with several cells in flight per SM (M_i^-1 as split 16-bit pairs streamed from L2).
- * The others, and the tensor-memory variant, run one block per SM: the right-hand side of Eq.
+ * (fp32_shared = 1).  Such handles run the form with several cells in flight per SM (M_i^-1 as split
+ * 16-bit pairs streamed from L2; at N = 3 one cell of 16 warps where the largest cell leaves no room for
+ * two blocks), but for P1 and P2 meshes with a cell of more than about 130 or 320 nodes, cells of more
+ * than 1,023 sub-tets, and handles created when the device had no room for the pairs.  These, and
+ * the tensor-memory variant, run one block per SM: the right-hand side of Eq.
  * ader4 is formed in chunks of sub-tets (16 per chunk at N = 2, 3 when the cell leaves room for
  * them, else 8: a "narrow" cell) and M_i^-1 streams through a ring of stages of 32 rows (in the
  * tensor-memory form 16 or 8 rows when a large cell leaves less room; as many stages as fit, at

@@ -1117,8 +1117,8 @@ __device__ __forceinline__ float f32_face_eps(double hi, double hj) {
 // conversions of mu, h and the normals, per lane), then chains of dependent loads; the
 // conversions are integer instructions now, 1 / dt comes with dt, eps and the viscous coefficients are
 // formed in pairs of FP32 values, to the same single rounding, and slots and partners come as one pair.
-// us per launch before and after: 32^3 P3 1,177 and 493 (127 for the bytes at
-// the copy rate), 21^3 P2 258 and 98, 24^3 P1 479 and 82, 4^3 P1 18 and 14.
+// us per launch before and after: 32^3 P3 1,177 and 440 (127 for the bytes at
+// the copy rate), 21^3 P2 258 and 90, 24^3 P1 479 and 76, 4^3 P1 18 and 12.
 template <int N>
 __global__ void __launch_bounds__(256) face_f32_kernel(const __grid_constant__ Batch bt) {
   constexpr int NF = nf_of(N), L = N == 1 ? 8 : (N == 2 ? 16 : 32), R = 2;

@@ -95,10 +95,11 @@ void pc_add_cell(int n, int s, int ns, PcCells* q) {
 
 template <int N>
 cudaError_t pc_plan(int device, int n_sm, int64_t cells, bool viscous, const PcCells& q, PcPlan* out) {
-  // meshes whose largest cell leaves no room for two blocks per SM take the one-block form, except at
-  // P3, where shape 0 gives a cell the whole SM: 32^3 mesh with cells of up to 539 nodes, step 18.1 ms in
-  // the one-block form, 12.6 ms here (a mesh that fits both shapes is 25 % slower in this one, so a
-  // batch with one such member still gains over the one-block form, but less)
+  // P3 meshes whose largest cell leaves no room for two blocks of shape 1 take shape 0, which gives a cell the
+  // whole SM: 32^3 mesh with cells of up to 539 nodes, step 18.1 ms in the one-block form, 12.6 ms here (a mesh
+  // that fits both shapes is 25 % slower in this one, so a batch with one such member still gains over
+  // the one-block form, but less).  P1 and P2 meshes that do not fit shape 1 (three gather slots per
+  // thread: cells of up to 130 and 322 nodes) keep the one-block form: shape 0 has not been timed on them.
   PcPlan many;
   cudaError_t e = plan_shape<N, 1>(device, q, &many);
   *out = many;

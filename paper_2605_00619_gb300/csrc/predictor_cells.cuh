@@ -1,8 +1,8 @@
 // FP32 space-time predictor with several cells in flight per SM (Sec. 4.3, Eqs.
-// ADER-localCauchy, ader4, TAvectors): the form that runs whenever at least two blocks fit an SM.
+// ADER-localCauchy, ader4, TAvectors): the form of every mesh that its plan takes (pc_plan, predictor_cells.cu).
 //
 // One block of 32 W threads per cell, persistent (blocks take cells from a work counter), two
-// blocks per SM at N = 3 and more at N = 1, 2, so that one cell's barriers, gathers and
+// blocks per SM at N = 3 (one of 16 warps where the largest cell needs the SM) and more at N = 1, 2, so that one cell's barriers, gathers and
 // serial tails are covered by another cell's arithmetic.  What the cell needs on chip:
 //   srec  [S][REC]       its packed sub-tet records (adj(J), det J, node ids)
 //   sgat                 its node -> (sub-tet, local node) lists, 16 bits per entry
@@ -22,11 +22,10 @@
 //      per variable.  The gather adds a node's incidences in (k, j) order in the registers of
 //      the thread that owns the node (no atomics; the order does not depend on the chunks).
 //      The first iteration starts from q^0 = u^ at every time node: one time slice serves all.
-//   2. Y = M_i^-1 RHS on the tensor cores.  M_i^-1 is kept, beside its FP32 rows, as pairs of
+//   2. Y = M_i^-1 RHS on the tensor cores.  M_i^-1 is kept as pairs of
 //      FP16 values hi + lo of M_i^-1 scaled to a unit diagonal by powers of two per row and column (both
 //      parts rounded to nearest: 22 bits and a sign, where the TF32 head and tail taken by truncation
-//      carry 21) in the
-//      register layout of mma.sync.m16n8k16, so that a warp streams its own 16-row tiles from L2
+//      carry 21) in the register layout of mma.sync.m16n8k16, so that a warp streams its own 16-row tiles from L2
 //      straight into registers, 1 KB per tile and 16 columns, with no staging in shared memory
 //      and no splitting arithmetic.  M_i^-1 is symmetric: only the tiles of its lower triangle are
 //      kept (a tile above the diagonal is the mirrored one, transposed in registers), which
@@ -1086,11 +1085,11 @@ __global__ void __launch_bounds__(32 * W, MB) predictor_cells_kernel(const __gri
 // What bounds it: M_i^-1 from HBM, once per step.  The lower triangle in 16-bit pairs is 53 % of the
 // FP32 rows that corrector_f32_kernel streams (75 % of the copy rate there); each tile is read a
 // second time for its mirror, from L2, which holds the cells in flight as long as few blocks
-// share an SM (three: 2,210 us at 32^3 P3, two 2,841).  FP64 work per node is kept to the update
+// share an SM (three: 2,210 us at 32^3 P3, two 2,841, before the sums outside the tensor cores).  FP64 work per node is kept to the update
 // itself and conversions are integer instructions: with ten FP64 reductions per warp and FP64
 // admissibility tests the launch took 3,017 us.
-// us per launch, corrector_f32_kernel and here: 32^3 P3 3,155 and 2,210 (1,500 for the bytes at the copy
-// rate), 16^3 P3 465 and 310, 21^3 P2 432 and 200, 24^3 P1 436 and 121, 8^3 P2 49 and 26.
+// us per launch, corrector_f32_kernel and here: 32^3 P3 3,155 and 2,264 (1,500 for the bytes at the copy
+// rate), 16^3 P3 465 and 316, 21^3 P2 432 and 205, 24^3 P1 436 and 122, 8^3 P2 49 and 26.
 __device__ __forceinline__ double f64_of(float x) {
   const unsigned b = __float_as_uint(x), e = b >> 23 & 255u;
   if (e - 1u >= 254u) return (double)x;  // zero, denormal, infinity, NaN

@@ -33,7 +33,9 @@ struct PcPlan {
 
 // What the plan needs to know of a set of cells: maxima of their nodes, sub-tets and face slots, and the
 // shared memory the most demanding one asks for by block shape.  Sets merge by maxima, so a union
-// fits whenever its parts do.
+// fits whenever its parts do.  (The corrector's shared memory is a sum of two maxima, of nodes and of face
+// slots; it stays below 140 KB for all cells that the gather slots admit, because a closed surface of f
+// triangles has f / 2 + 2 vertices and more nodes: at N = 3 f <= N_i / 4.5.)
 struct PcCells {
   int Nmax = 0, Smax = 0, Fmax = 0;
   size_t need[2] = {0, 0};

@@ -266,7 +266,7 @@ __device__ __forceinline__ void pd_contract(const PdRef& ref, bool transposed, i
   using P = Pd<N>;
   constexpr int NP = P::NP, KK = 3 * NP, KST = P::KST, THR = 32 * W, QN = KST * 4;  // values per lane
   double* const col0 = PdView<N>().region;
-  if constexpr (N == 1) {  // 12 values per column: 36 multiply-adds are less than the digits' own work
+  if constexpr (N == 1) {  // 12 values per column: 24 multiply-adds are less than the digits' own work
     for (int c = threadIdx.x; c < cols; c += THR) {
       double acc[NP];
 #pragma unroll
