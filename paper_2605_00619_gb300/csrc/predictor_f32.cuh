@@ -1,7 +1,7 @@
 // FP32 space-time predictor for sm_103a (Sec. 4.3, Eqs. ADER-localCauchy, ader4, TAvectors), one block
 // per SM: the form of the tcgen05 apply, and of meshes that predictor_cells.cuh does not take (P1 and P2 with
 // cells of more than about 130 and 320 nodes, cells of more than 1,023 sub-tets, no device memory for
-// the split M_i^-1; at N = 3 the mma.sync apply is reached by the last two only).
+// the split M_i^-1; at N = 3 the mma.sync apply is reached by the last only).
 //
 // One block of 512 threads per cell (persistent: blocks take cells from a work counter).
 // The cell's working set stays in shared memory for the whole fixed-point iteration:
