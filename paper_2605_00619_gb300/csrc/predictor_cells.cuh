@@ -479,16 +479,8 @@ __device__ __forceinline__ void pc_rhs(bool first) {
         for (int o = 16; o > 0; o >>= 1) racc[v][t] += __shfl_xor_sync(0xffffffffu, racc[v][t], o);
       }
   }
-  // row scaling, then the right-hand side's power of two per variable.  The fragments overwrite the
+  // the right-hand side's power of two per variable, over the scaled rows.  The fragments overwrite the
   // region up to the sums of the third slots: those of the second slots are read before the barrier.
-  auto scale = [&](int n, float (&a)[5][NTP]) {
-    const float f = pow2f(-(int)V.sexp[n]);
-#pragma unroll
-    for (int v = 0; v < 5; ++v)
-#pragma unroll
-      for (int t = 0; t < NTP; ++t) a[v][t] *= f;
-  };
-  if (node0 >= 0) scale(node0, racc);
   float a[5][NTP];
 #pragma unroll
   for (int v = 0; v < 5; ++v)
@@ -499,18 +491,23 @@ __device__ __forceinline__ void pc_rhs(bool first) {
   for (int v = 0; v < 5; ++v) omax[v] = 0.f;
   for (int i = tid + (x.slots - 1 - tid) / THR * THR; i >= THR; i -= THR) {  // the second slot last
     load_sums(reinterpret_cast<const float4*>(sover + (i - THR) * SQ), a);
-    scale(V.slist[1 + 2 * (i - 31 * x.nlong)], a);
+    const float f = pow2f(-(int)V.sexp[V.slist[1 + 2 * (i - 31 * x.nlong)]]);
 #pragma unroll
-    for (int v = 0; v < 5; ++v)
+    for (int v = 0; v < 5; ++v) {
+      float mx = 0.f;
 #pragma unroll
-      for (int t = 0; t < NT; ++t) omax[v] = fmaxf(omax[v], fabsf(a[v][t]));
+      for (int t = 0; t < NT; ++t) mx = fmaxf(mx, fabsf(a[v][t]));
+      omax[v] = fmaxf(omax[v], mx * f);
+    }
   }
-  float sc[5];
+  const float f0 = node0 >= 0 ? pow2f(-(int)V.sexp[node0]) : 0.f;
+  int sc[5];  // biased exponents
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
-    float mx = omax[v];
+    float mx = 0.f;
 #pragma unroll
     for (int t = 0; t < NT; ++t) mx = fmaxf(mx, fabsf(racc[v][t]));
+    mx = fmaxf(omax[v], mx * f0);
     // non-negative floats order as integers
     mx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx)));
     if (lane == 0) sred[v][warp] = mx;
@@ -521,9 +518,8 @@ __device__ __forceinline__ void pc_rhs(bool first) {
     float y = sred[v][0];
 #pragma unroll
     for (int w = 1; w < W; ++w) y = fmaxf(y, sred[v][w]);
-    const int e = f16_scale_exp(__float_as_uint(y));
-    sc[v] = __uint_as_float((uint32_t)e << 23);
-    if (tid == 0) x.isv[v] = __uint_as_float((uint32_t)(254 - e) << 23);
+    sc[v] = f16_scale_exp(__float_as_uint(y));
+    if (tid == 0) x.isv[v] = __uint_as_float((uint32_t)(254 - sc[v]) << 23);
   }
   // fragments: entry (row n, column col) at 16-row step n / 16, column tile col / 8, lane
   // (col & 7) 4 + ((n & 7) >> 1), words {b0 hi, b1 hi, b0 lo, b1 lo}, b = (n & 15) >> 3
@@ -532,19 +528,23 @@ __device__ __forceinline__ void pc_rhs(bool first) {
   auto row = [&](int n) { return frag + (n >> 4) * fb + ((n & 7) >> 1) * 16 + ((n >> 3) & 1) * 4 + (n & 1) * 2; };
   auto put = [&](int n, const float (&a)[5][NTP]) {
     unsigned char* const b = row(n);
+    const int p = V.sexp[n];
 #pragma unroll
-    for (int v = 0; v < 5; ++v)
+    for (int v = 0; v < 5; ++v) {
+      // row and variable in one power of two (bounded: sums below 2^-112 of a cell's would need more)
+      const float s = __uint_as_float((uint32_t)min(254, max(1, sc[v] - p)) << 23);
 #pragma unroll
       for (int t = 0; t < NTP; ++t) {
         if (first && t > 0) continue;
         const int col = first ? v : v * NTP + t;
-        const float y = a[v][t] * sc[v];
+        const float y = a[v][t] * s;
         const __half hi = __float2half_rn(y);
         const __half lo = __float2half_rn(y - __half2float(hi));
         unsigned char* d = b + (col >> 3) * 512 + (col & 7) * 64;
         *reinterpret_cast<__half*>(d) = hi;
         *reinterpret_cast<__half*>(d + 8) = lo;
       }
+    }
   };
   int n = warp >= x.nlong || lane == 0 ? node0 : -1;
 #pragma unroll 1
@@ -553,10 +553,7 @@ __device__ __forceinline__ void pc_rhs(bool first) {
     i += THR;
     if (i >= x.slots) break;
     n = V.slist[1 + 2 * (i - 31 * x.nlong)];
-    if (i >= 2 * THR) {
-      load_sums(reinterpret_cast<const float4*>(sover + (i - THR) * SQ), a);
-      scale(n, a);
-    }
+    if (i >= 2 * THR) load_sums(reinterpret_cast<const float4*>(sover + (i - THR) * SQ), a);
 #pragma unroll
     for (int v = 0; v < 5; ++v)
 #pragma unroll
@@ -1077,9 +1074,9 @@ __global__ void __launch_bounds__(32 * W, MB) predictor_cells_kernel(const __gri
 //   f[slot][a] = 2 area sum_b Z^[a][b] G[b]     (a thread per slot and variable, once per slot)
 //   r = vol - sum over the node's face incidences of f   (fixed order)
 //   du = M_i^-1 r on the tensor cores: the tiles of the predictor's first iteration (5 columns), with the
-//        leading products added up outside the tensor cores, which truncate, and at N <= 2, where sums are
-//        short, r in three FP16 parts (all of its 24 bits) and the product of the low parts: no further
-//        off than FP32 multiply-adds over FP32 rows
+//        leading products added up outside the tensor cores, which truncate, at N <= 2, where sums are
+//        short, the product of the low parts, and at N = 1 r in three FP16 parts (all of its 24 bits): no
+//        further off than FP32 multiply-adds over FP32 rows
 //   u += du + (T - w_i . du) / |P_i|            (FP64: T = exact cell total of r, see
 //                                                corrector_f32_kernel)
 // What bounds it: M_i^-1 from HBM, once per step.  The lower triangle in 16-bit pairs is 53 % of the
@@ -1089,7 +1086,7 @@ __global__ void __launch_bounds__(32 * W, MB) predictor_cells_kernel(const __gri
 // itself and conversions are integer instructions: with ten FP64 reductions per warp and FP64
 // admissibility tests the launch took 3,017 us.
 // us per launch, corrector_f32_kernel and here: 32^3 P3 3,155 and 2,264 (1,500 for the bytes at the copy
-// rate), 16^3 P3 465 and 316, 21^3 P2 432 and 205, 24^3 P1 436 and 122, 8^3 P2 49 and 26.
+// rate), 16^3 P3 465 and 316, 21^3 P2 432 and 200, 24^3 P1 436 and 121, 8^3 P2 49 and 26.
 __device__ __forceinline__ double f64_of(float x) {
   const unsigned b = __float_as_uint(x), e = b >> 23 & 255u;
   if (e - 1u >= 254u) return (double)x;  // zero, denormal, infinity, NaN
@@ -1097,11 +1094,11 @@ __device__ __forceinline__ double f64_of(float x) {
 }
 
 // Parts of the split right-hand side, and its bytes per 16 rows: two parts as the predictor's, behind them the
-// third.  Relative L2 error of M_i^-1 r against 64 bits (random r, smooth du; FP32 multiply-adds): P3 1.2e-7, 3.4e-7
-// with two parts (3.2e-7, 5.2e-7); P2 0.9e-7, 2.4e-7 (1.9e-7, 3.4e-7) and P1 0.7e-7, 1.5e-7 (0.9e-7, 1.8e-7)
-// with three, above the multiply-adds' with two.
+// third.  Relative L2 error of M_i^-1 r against 64 bits (random r, smooth du; FP32 multiply-adds), without the
+// product of the low parts P3 1.2e-7, 3.4e-7 (3.2e-7, 5.2e-7), with it P2 1.0e-7, 3.2e-7 (1.9e-7, 3.4e-7), with
+// the third part too P1 0.7e-7, 1.5e-7 (0.9e-7, 1.8e-7).
 template <int N>
-constexpr int corr_parts = N == 3 ? 2 : 3;
+constexpr int corr_parts = N == 1 ? 3 : 2;
 template <int N>
 constexpr int corr_frag = 160 * corr_parts<N>;
 
@@ -1236,9 +1233,9 @@ __global__ void __launch_bounds__(32 * W, N == 3 ? 3 : (N == 2 ? 8 : 24)) correc
       mma_f16(lead, x, b.x, b.y);
       if constexpr (three) {
         const uint2 b3 = lane < 20 ? *reinterpret_cast<const uint2*>(f + 320 + lane * 8) : make_uint2(0, 0);
-        mma_f16(low, l, b.z, b.w);
         mma_f16(low, x, b3.x, b3.y);
       }
+      if constexpr (N <= 2) mma_f16(low, l, b.z, b.w);
       mma_f16(low, l, b.x, b.y);
       mma_f16(low, x, b.z, b.w);
 #pragma unroll
