@@ -1499,11 +1499,14 @@ afe_status autotune_impl(const std::string& sig, int order, bool tc_fits, int* w
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     auto it = g_tune_cache.find(sig);
     if (it != g_tune_cache.end()) {
-      AFE_TRY(set(it->second));
-      if (best) *best = it->second;
-      if (best_ms) *best_ms = -1.0;
-      if (default_ms) *default_ms = -1.0;
-      return AFE_OK;
+      const afe_status s = set(it->second);
+      if (s != AFE_ENOMEM || it->second.variant != 1) {  // (no room for that form's rows: timed without it)
+        AFE_TRY(s);
+        if (best) *best = it->second;
+        if (best_ms) *best_ms = -1.0;
+        if (default_ms) *default_ms = -1.0;
+        return AFE_OK;
+      }
     }
   }
   {
