@@ -204,8 +204,8 @@ afe_status afe_stage_times(afe_mesh* m, double* ms, int64_t* nsteps, int reset);
  * most 8; a cell whose N_i is not a multiple of the stage height ends with a partial, "masked"
  * stage).  The ring, chunk and stage fields below report that one-block plan for every mesh with
  * fp32_shared = 1, smem_bytes the form that runs.  Meshes whose largest cell does not fit it run
- * the FP32 form with global-memory scratch on the CUDA cores (fp32_shared = 0), as does, always,
- * the FP64 form. */
+ * the FP32 form with global-memory scratch on the CUDA cores (fp32_shared = 0).  For the FP64 form only
+ * the node and sub-tet counts are reported. */
 typedef struct {
   int32_t fp32_shared;     /* 1: FP32 shared-memory predictor (M_i^-1 apply on the tensor cores)  */
   int32_t corrector_block; /* 1: FP32 corrector with one block per cell                           */
